@@ -24,6 +24,7 @@
 #include "pdas_internal.cuh"
 #include "chol_dig.cuh"
 #include "syrk_dig.cuh"
+#include "syrk_simt.cuh"
 #include "syrk_tc.cuh"
 
 using namespace pdas;
@@ -50,6 +51,9 @@ struct pdas_ctx {
   float* M32 = nullptr;
   double* dinv64 = nullptr;  // reciprocals of the pivots of the FP64 / FP32 factor
   float* dinv32 = nullptr;
+  void* simt_part = nullptr;        // SIMT normal matrices: partial tiles of their K slices
+  unsigned* simt_tickets = nullptr;  // one per tile, zero between launches
+  float* simt_planes = nullptr;      // FP32_IR: operand planes of the normal matrix
   TcWorkspace tc{};
   DigWorkspace dig{};  // FP64 tier on the tensor cores (BF16 A): digit planes
   CholDigWorkspace cdig{};  // FP64 tier: the factor's trailing updates on the tensor cores
@@ -337,10 +341,10 @@ pdas_status form_normal(pdas_ctx* h, const void* A) {
         cols = kept;
       }
       if constexpr (std::is_same<T, double>::value) {
-        KL(launch_syrk_simt<T>(h->st, h->m, cols, Aop, Dop, h->M64, nullptr, h->ldm, h->sc), 1);
+        KL(launch_syrk_fp64<T>(h->st, h->m, cols, Aop, Dop, h->M64, h->ldm, h->simt_part, h->simt_tickets, h->sc), 1);
       } else {
         if (df) KL(launch_syrk_df<T>(h->st, h->m, cols, Aop, Dop, h->d2, h->M64, h->ldm, h->sc), 2);
-        else KL(launch_syrk_simt<T>(h->st, h->m, cols, Aop, Dop, h->M64, nullptr, h->ldm, h->sc), 1);
+        else KL(launch_syrk_fp64<T>(h->st, h->m, cols, Aop, Dop, h->M64, h->ldm, h->simt_part, h->simt_tickets, h->sc), 1);
       }
       return PDAS_OK;
     });
@@ -350,7 +354,10 @@ pdas_status form_normal(pdas_ctx* h, const void* A) {
   if (h->opt.form == PDAS_FP32_IR) {
     return with_dtype(h->opt.a_dtype, [&](auto tag) -> pdas_status {
       using T = std::remove_const_t<std::remove_pointer_t<decltype(tag)>>;
-      KL(launch_syrk_simt<T>(h->st, h->m, h->n, (const T*)A, h->D, nullptr, h->M32, h->ldm, h->sc), 1);
+      int kl = 0;
+      CK(launch_syrk_fp32<T>(h->st, h->m, h->n, (const T*)A, h->D, h->simt_planes, h->M32, h->ldm, h->simt_part,
+                             h->simt_tickets, h->sc, &kl));
+      h->launches += kl;
       return PDAS_OK;
     });
   }
@@ -789,6 +796,17 @@ pdas_status pdas_create(int64_t m, int64_t n, const pdas_options* opt_in, pdas_h
       }
     }
   }
+  {  // the SIMT normal matrices
+    size_t part = simt_fp64_part_bytes(m);
+    if (opt.form == PDAS_FP32_IR) {
+      const SimtPlan p = simt_plan_fp32(m, n);
+      part = std::max(part, p.part_bytes);
+      al((void**)&h->simt_planes, sizeof(float) * 2 * m * p.ldk);
+    }
+    if (part) al(&h->simt_part, part);
+    al((void**)&h->simt_tickets, sizeof(unsigned) * simt_ticket_count(m));
+    if (e == cudaSuccess) e = cudaMemsetAsync(h->simt_tickets, 0, sizeof(unsigned) * simt_ticket_count(m), h->st);
+  }
   if (e == cudaSuccess && opt.form != PDAS_FP64 && chol_tile_count(m) <= kTileCholMaxTiles) {
     // the single-launch tile Cholesky of the FP32 factor
     std::vector<int4> tasks;
@@ -836,6 +854,9 @@ void pdas_destroy(pdas_handle h) {
                     h->part, h->gt_part, h->M64, h->rd};
   for (double* p : vecs)
     if (p) cudaFree(p);
+  if (h->simt_part) cudaFree(h->simt_part);
+  if (h->simt_tickets) cudaFree(h->simt_tickets);
+  if (h->simt_planes) cudaFree(h->simt_planes);
   if (h->M32) cudaFree(h->M32);
   if (h->akept) cudaFree(h->akept);
   if (h->dkept) cudaFree(h->dkept);

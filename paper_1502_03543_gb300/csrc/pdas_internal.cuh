@@ -127,10 +127,6 @@ cudaError_t launch_krylov_update(cudaStream_t st, int64_t n, const double* base,
 cudaError_t launch_krylov_direction(cudaStream_t st, int64_t n, const double* z, double* p, double beta_num,
                                     const Scalars* sc);
 
-template <typename T>
-cudaError_t launch_syrk_simt(cudaStream_t st, int64_t m, int64_t n, const T* A, const double* D, double* M64,
-                             float* M32, int64_t ldm, const Scalars* sc);
-
 // Blocked Cholesky in place; dinv (m) receives the reciprocals of the pivots.
 template <typename T>
 cudaError_t cholesky(cudaStream_t st, int64_t m, int64_t ldm, T* M, T* dinv, Scalars* sc);

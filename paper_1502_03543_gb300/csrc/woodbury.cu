@@ -29,6 +29,7 @@
 #include <vector>
 
 #include "pdas_internal.cuh"
+#include "syrk_simt.cuh"
 #include "pdas_woodbury.h"
 
 struct pdas_wb_ctx {
@@ -43,6 +44,8 @@ struct pdas_wb_ctx {
   double* den = nullptr;    // den_l (n)
   pdas::Scalars* sc = nullptr;
   pdas::Scalars* sc_host = nullptr;  // pinned
+  void* simt_part = nullptr;  // partial tiles of A A' (syrk_simt.cuh)
+  unsigned* simt_tickets = nullptr;
   bool prepared = false;
   char errmsg[256] = {0};
 };
@@ -211,6 +214,9 @@ pdas_status pdas_woodbury_create(int64_t m, int64_t n, int a_dtype, void* stream
   al((void**)&h->Y0, sizeof(double) * n * m);
   al((void**)&h->W, sizeof(double) * (n + 1) * m);
   al((void**)&h->den, sizeof(double) * n);
+  if (simt_fp64_part_bytes(m)) al(&h->simt_part, simt_fp64_part_bytes(m));
+  al((void**)&h->simt_tickets, sizeof(unsigned) * simt_ticket_count(m));
+  if (e == cudaSuccess) e = cudaMemsetAsync(h->simt_tickets, 0, sizeof(unsigned) * simt_ticket_count(m), h->st);
   al((void**)&h->sc, sizeof(Scalars));
   if (e == cudaSuccess) e = cudaMallocHost((void**)&h->sc_host, sizeof(Scalars));
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_wb_step<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -236,7 +242,8 @@ pdas_status pdas_woodbury_prepare(pdas_wb_handle h, const void* A) {
   WCK(cudaGetLastError());
   const cudaError_t pe = with_a_dtype(h->a_dtype, [&](auto tag) -> cudaError_t {
     using T = std::remove_const_t<std::remove_pointer_t<decltype(tag)>>;
-    cudaError_t e = launch_syrk_simt<T>(h->st, h->m, h->n, (const T*)A, h->ones, h->G, nullptr, h->ldm, h->sc);
+    cudaError_t e = launch_syrk_fp64<T>(h->st, h->m, h->n, (const T*)A, h->ones, h->G, h->ldm, h->simt_part,
+                                          h->simt_tickets, h->sc);
     if (e == cudaSuccess) e = cholesky<double>(h->st, h->m, h->ldm, h->G, h->ginv, h->sc);
     if (e != cudaSuccess) return e;
     k_wb_solve_cols<T><<<solve_grid(h->n), kWbThreads, 0, h->st>>>(h->m, h->n, h->ldm, h->G, h->ginv, (const T*)A,
@@ -293,6 +300,8 @@ void pdas_woodbury_destroy(pdas_wb_handle h) {
   double* bufs[] = {h->G, h->ginv, h->ones, h->Y0, h->W, h->den};
   for (double* p : bufs)
     if (p) cudaFree(p);
+  if (h->simt_part) cudaFree(h->simt_part);
+  if (h->simt_tickets) cudaFree(h->simt_tickets);
   if (h->sc) cudaFree(h->sc);
   if (h->sc_host) cudaFreeHost(h->sc_host);
   delete h;
