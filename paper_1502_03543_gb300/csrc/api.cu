@@ -75,7 +75,7 @@ struct pdas_ctx {
   double* adj = nullptr;        // adjoint vectors (5 n + m)
   int4* chol_tasks = nullptr;   // task list of the tile Cholesky (FP32 factor)
   int chol_ntasks = 0;
-  int* chol_state = nullptr;    // per-tile counters of the tile Cholesky
+  int* chol_state = nullptr;    // counters of the tile Cholesky: per tile, then panels per diagonal tile
   float* uinv32 = nullptr;      // L_ll^{-T} of every diagonal tile of the FP32 tile factor
   unsigned char* chol_planes = nullptr;  // BF16 operand planes of the tile factor's off-diagonal tiles
   float2* pairs = nullptr;      // the vector of a double-float pass as FP32 pairs (max(m, n))
@@ -816,7 +816,7 @@ pdas_status pdas_create(int64_t m, int64_t n, const pdas_options* opt_in, pdas_h
     const int64_t nb = chol_tile_count(m);
     h->chol_ntasks = (int)tasks.size();
     al((void**)&h->chol_tasks, sizeof(int4) * tasks.size());
-    al((void**)&h->chol_state, sizeof(int) * nb * nb);
+    al((void**)&h->chol_state, sizeof(int) * (nb * nb + nb));
     al((void**)&h->uinv32, sizeof(float) * nb * kCholTile * kCholTile);
     if (nb > 1) al((void**)&h->chol_planes, (size_t)chol_plane_bytes(m));
     if (e == cudaSuccess)

@@ -12,8 +12,9 @@
 //                  when i = l + 1 (rank 128)
 // In the FP32 factor every product L_ik L_lk' runs on the tcgen05 tensor
 // cores (BF16 operand planes, FP32 accumulation in tensor memory; see the
-// section "FP32 products on the tensor cores"); the FP64 instantiation keeps
-// SIMT products.
+// section "FP32 products on the tensor cores") and the tile operations are those
+// of chol_f32_tile.cuh; the double-float instantiation keeps SIMT products and
+// the tile operations below.
 // A tile's last update and its factorisation or triangular solve run in one
 // task on the tile held in registers (except the sub-diagonal tiles, see
 // below), and the dependency chain of the factorisation (FINAL(l,l) ->
@@ -21,15 +22,16 @@
 // the lower triangle has a counter in global memory: the number of updates
 // applied to it, then l + 1 once it holds its final L values.
 //
-// Block 0 runs the dependency chain itself: FINAL(l, l), then the solve of
-// the sub-diagonal tile (l + 1, l) against L_ll while L_ll and its pivot
-// reciprocals are still in its shared memory (that tile's last update,
-// k = l - 1, is an ordinary UPDATE task), then FINAL(l + 1, l + 1), ...  The
-// head of the chain never queues behind trailing updates, and no chain link
-// crosses between CTAs.  The
-// other CTAs take the remaining tasks from a ticket counter in a fixed list
-// order.  In that order every task comes after all tasks it waits for (block
-// 0's tasks included), so the first unfinished task is always held by a
+// The dependency chain runs in CTAs of its own, so that its head never queues
+// behind trailing updates: in the FP32 factor in blocks 0 and 1 (chol_chain),
+// tile rows in turn, so that the solve of a sub-diagonal tile runs beside the
+// factorisation it depends on, panel by panel; these also apply that tile's last
+// update (k = l - 1).  In the double-float factor block 0 runs FINAL(l, l), then
+// the solve of tile (l + 1, l) while L_ll is still in its shared memory, then
+// FINAL(l + 1, l + 1), ..., and the update is an ordinary task.  The other
+// CTAs take the remaining tasks from a ticket counter in a fixed list
+// order.  In that order every task comes after all tasks it waits for (the
+// chain's included), so the first unfinished task is always held by a
 // running CTA and has all it waits for done, and every task finishes by
 // induction on the order; every wait is also bounded (2 s, PDAS_ERR_TIMEOUT).
 // The order itself comes from
@@ -40,6 +42,7 @@
 // trailing updates around it.  A non-positive pivot records PDAS_ERR_NOT_SPD
 // and its index; the other CTAs see the status and stop.
 #include <algorithm>
+#include <cstddef>
 #include <type_traits>
 #include <queue>
 #include <vector>
@@ -49,6 +52,7 @@
 #include "sync_util.cuh"
 #include "tc_util.cuh"
 #include "df_util.cuh"
+#include "chol_f32_tile.cuh"
 #include "tile_core.cuh"
 
 namespace pdas {
@@ -88,11 +92,22 @@ constexpr uint32_t kTcIdesc = tc::idesc_bf16(kBig, kBig);
 // Slot of the off-diagonal tile (i, k), i > k, in the plane buffer.
 __host__ __device__ constexpr int64_t plane_slot(int64_t i, int64_t k) { return i * (i - 1) / 2 + k; }
 
+// FP32 chain: the operand planes of its product (one tile, both K chunks) lie
+// past the tile to be solved and the panels, and under the diagonal tile, which
+// is loaded once the product is complete.
+constexpr int kChainOps = 100 * 1024;
+
 template <typename T>
 struct TileCholSmem {
   union {
     T stage[2][2][kBig][upd_pitch<T>()];  // UPDATE (FP64): [buffer][row tile i | row tile l][row][k]
-    T ls[kBig][kBig + 1];                 // TRSM: the factor of the diagonal tile; FP32 products: D
+    T ls[sizeof(T) == 4 ? 1 : kBig][kBig + 1];  // TRSM (double-float): the factor of the diagonal tile
+    struct {
+      float c[kBig][ft::kPt];      // FP32: the tile to be solved
+      float panel[2][32][ft::kPt];  // FP32: panels of the factor it is solved against
+      float s[kBig][ft::kPt];      // FP32 chain: the diagonal tile
+    } f;
+    unsigned char chain[kChainOps + kTcOpsBytes / 2 + 1024];  // FP32 chain: operand planes at kChainOps
     unsigned char tc_ops[kTcOpsBytes + 1024];  // FP32 products: the BF16 planes (1024-aligned inside)
   };
   T cb[2][kBig];  // column buffers of the POTRF / TRSM sweeps (double-buffered)
@@ -103,6 +118,7 @@ struct TileCholSmem {
   int tc_ok;
   int4 task;
   int go;
+  int trsm_go[2];  // FP32 solves: outcome of the waits for the factor's panels
 };
 
 __device__ __forceinline__ void cp_async16(void* smem, const void* gmem, bool valid) {
@@ -123,8 +139,6 @@ __device__ __forceinline__ bool pivot_bad(T d) {
 
 // One element from global memory through L2 (the tile counters order it after
 // its producer's release).
-__device__ __forceinline__ float ld_cg(const float* p) { return __ldcg(p); }
-__device__ __forceinline__ double ld_cg(const double* p) { return __ldcg(p); }
 __device__ __forceinline__ dfloat ld_cg(const dfloat* p) {
   const float2 v = __ldcg(reinterpret_cast<const float2*>(p));
   return dfloat(v.x, v.y);
@@ -224,12 +238,6 @@ __device__ __forceinline__ void rank_update(T (&acc)[8][8], int64_t m, int64_t l
     if (ch + 2 < NCH) issue(ch + 2, buf);
   }
 }
-
-// 1 / sqrt(d) of a pivot: the hardware estimate (within 2 ulp in FP32; the
-// FP32 factor is a preconditioner, and every entry of a column is scaled by
-// the same value); IEEE for FP64.
-__device__ __forceinline__ float inv_sqrt(float d) { return rsqrtf(d); }
-__device__ __forceinline__ double inv_sqrt(double d) { return 1.0 / sqrt(d); }
 
 // Right-looking factorisation of a 32 x 32 block held by one warp (lane =
 // row), as a loop over the pivot column C: row[] is shifted left every step,
@@ -400,14 +408,6 @@ __device__ __forceinline__ bool tile_potrf(const T (&acc)[8][8], int64_t m, int6
 template <typename T>
 struct Vec16Reg;
 template <>
-struct Vec16Reg<float> {
-  using V = float4;
-  static constexpr int N = 4;
-  __device__ static V load(const float* p) { return __ldcg(reinterpret_cast<const float4*>(p)); }
-  __device__ static float get(const V& v, int k) { return k == 0 ? v.x : k == 1 ? v.y : k == 2 ? v.z : v.w; }
-  __device__ static V make(const float (&a)[4]) { return make_float4(a[0], a[1], a[2], a[3]); }
-};
-template <>
 struct Vec16Reg<dfloat> {
   using V = float4;
   static constexpr int N = 2;
@@ -415,15 +415,6 @@ struct Vec16Reg<dfloat> {
   __device__ static dfloat get(const V& v, int k) { return k == 0 ? dfloat(v.x, v.y) : dfloat(v.z, v.w); }
   __device__ static V make(const dfloat (&a)[2]) { return make_float4(a[0].hi, a[0].lo, a[1].hi, a[1].lo); }
 };
-template <>
-struct Vec16Reg<double> {
-  using V = double2;
-  static constexpr int N = 2;
-  __device__ static V load(const double* p) { return __ldcg(reinterpret_cast<const double2*>(p)); }
-  __device__ static double get(const V& v, int k) { return k == 0 ? v.x : v.y; }
-  __device__ static V make(const double (&a)[2]) { return make_double2(a[0], a[1]); }
-};
-
 // Loads L_ll (strictly lower part; rows and columns past m read as the
 // identity) and its pivot reciprocals into shared memory: 16-byte loads,
 // issued in batches of eight before their stores.
@@ -520,26 +511,6 @@ __device__ __forceinline__ void trsm_sweep(T (&acc)[8][8], TileCholSmem<T>& sm) 
   __syncwarp();
 }
 
-// U_l = L_ll^{-T} (upper triangular; the identity past m): the sweep above
-// applied to C = I.  Stored row-major 128 x 128 at Uinv + l 128^2; the
-// blocked triangular solves apply it in place of a substitution.
-template <typename T>
-__device__ __forceinline__ void tile_inverse(T (&acc)[8][8], int64_t m, int64_t ldm, const T* M, const T* dinv,
-                                             T* Uinv, int l, TileCholSmem<T>& sm) {
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  load_diag_factor<T>(m, ldm, M, dinv, l, sm);
-#pragma unroll
-  for (int i = 0; i < 8; ++i)
-#pragma unroll
-    for (int j = 0; j < 8; ++j) acc[i][j] = (ty + 16 * i == tx + 16 * j) ? T(1) : T(0);
-  trsm_sweep<T>(acc, sm);
-  T* U = Uinv + (int64_t)l * kBig * kBig;
-#pragma unroll
-  for (int i = 0; i < 8; ++i)
-#pragma unroll
-    for (int j = 0; j < 8; ++j) U[(ty + 16 * i) * kBig + tx + 16 * j] = acc[i][j];
-}
-
 // ---- FP32 products on the tensor cores ---------------------------------------
 // D = L_ik L_lk' for one tile column k (K = 128) of the FP32 factor, with
 // every operand split into three BF16 planes: the leading term A0 B0' goes
@@ -573,44 +544,52 @@ __device__ __forceinline__ void bulk_copy(uint32_t dst, const void* src, uint32_
                : "memory");
 }
 
-// The BF16 planes of the finished tile held in acc (tile layout) to its slot
-// of the plane buffer.  The tile passes through a staging area as FP32 rows;
-// thread item e (8 per thread) is K chunk e / 1024, row (e / 8) % 128 and
-// 16-byte chunk e % 8 of that row.  Rows past m hold zeros in acc.
-__device__ __forceinline__ void tc_write_planes(const float (&acc)[8][8], unsigned char* slot, TileCholSmem<float>& sm) {
-  float(*S)[kStagePitch] = reinterpret_cast<float(*)[kStagePitch]>(sm.tc_ops);
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  __syncthreads();  // (the staging area overlaps L_ll)
+// Block b (32 columns) of the finished tile X (column-major, rows past m zero):
+// to rows p0.., columns q0 + 32 b.. of M, and as BF16 planes to its slot of the
+// plane buffer and, if ops is given, to shared memory as the operand of this
+// CTA's own next product.  Thread item (2 per thread): row r, 8 columns cc; a
+// warp covers 16 rows x 2 items, so its stores fill 32-byte sectors and its
+// shared-memory reads are at most 2-way conflicted.
+template <bool OPS>
+__device__ __forceinline__ void finish_block(const float (*X)[ft::kPt], int b, int64_t m, int64_t ldm, float* M,
+                                             int64_t p0, int64_t q0, unsigned char* slot, unsigned char* ops) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-  for (int i = 0; i < 8; ++i)
+  for (int v = 0; v < 2; ++v) {
+    const int r = 16 * warp + (lane & 15), cc = 4 * b + 2 * v + (lane >> 4);
+    float x[8];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) S[ty + 16 * i][tx + 16 * j] = acc[i][j];
-  __syncthreads();
-#pragma unroll 2
-  for (int u = 0; u < 2 * kBig * 8 / kThreads; ++u) {
-    const int e = tid + kThreads * u, kc = e >> 10, r = (e >> 3) & (kBig - 1), c8 = e & 7;
-    const float4 lo = *reinterpret_cast<const float4*>(&S[r][64 * kc + 8 * c8]);
-    const float4 hi = *reinterpret_cast<const float4*>(&S[r][64 * kc + 8 * c8 + 4]);
+    for (int e = 0; e < 8; ++e) x[e] = X[8 * cc + e][r];
+    if (p0 + r < m) {
+      float4* dst = reinterpret_cast<float4*>(M + (p0 + r) * ldm + q0 + 8 * cc);
+      dst[0] = make_float4(x[0], x[1], x[2], x[3]);
+      dst[1] = make_float4(x[4], x[5], x[6], x[7]);
+    }
     uint32_t w[3][4];
-    bf16x2_split3(lo.x, lo.y, w[0][0], w[1][0], w[2][0]);
-    bf16x2_split3(lo.z, lo.w, w[0][1], w[1][1], w[2][1]);
-    bf16x2_split3(hi.x, hi.y, w[0][2], w[1][2], w[2][2]);
-    bf16x2_split3(hi.z, hi.w, w[0][3], w[1][3], w[2][3]);
-    unsigned char* dst = slot + kc * kTcChunkBytes + r * 128 + ((c8 ^ (r & 7)) << 4);
 #pragma unroll
-    for (int sp = 0; sp < 3; ++sp)
-      *reinterpret_cast<uint4*>(dst + sp * kTcPlaneBytes) = make_uint4(w[sp][0], w[sp][1], w[sp][2], w[sp][3]);
+    for (int e = 0; e < 4; ++e) bf16x2_split3(x[2 * e], x[2 * e + 1], w[0][e], w[1][e], w[2][e]);
+    const int off = (cc >> 3) * kTcChunkBytes + r * 128 + (((cc & 7) ^ (r & 7)) << 4);
+#pragma unroll
+    for (int sp = 0; sp < 3; ++sp) {
+      const uint4 val = make_uint4(w[sp][0], w[sp][1], w[sp][2], w[sp][3]);
+      *reinterpret_cast<uint4*>(slot + off + sp * kTcPlaneBytes) = val;
+      if (OPS) *reinterpret_cast<uint4*>(ops + off + sp * kTcPlaneBytes) = val;
+    }
   }
-  asm volatile("fence.proxy.async.global;" ::: "memory");  // read next by bulk copies (async proxy)
+  // The MMAs read ops through the async proxy.  (The slot's readers fence after
+  // their acquire of the tile's counter, before their bulk copies: a fence here
+  // would wait for the stores to reach global memory.)
+  if (OPS) tc::fence_proxy_async();
 }
 
-// One thread: the 24 MMAs of a K chunk (A planes at ops, B planes after them
-// or, on a diagonal tile, the A planes again).
-__device__ __forceinline__ void tc_issue(uint32_t ops, bool diag, uint32_t tmem, bool first) {
+// One thread: the MMAs of K steps ks0 .. ks1 - 1 (16 each) of a K chunk of 64 (A
+// planes at ops, B planes after them or, on a diagonal tile, the A planes
+// again); first: the chunk's step 0 starts the sums.
+__device__ __forceinline__ void tc_issue(uint32_t ops, bool diag, uint32_t tmem, bool first, int ks0 = 0, int ks1 = 4) {
   const uint32_t a0 = ops, a1 = ops + kTcPlaneBytes, a2 = ops + 2 * kTcPlaneBytes;
   const uint32_t b0 = diag ? ops : ops + kTcChunkBytes, b1 = b0 + kTcPlaneBytes, b2 = b0 + 2 * kTcPlaneBytes;
-#pragma unroll
-  for (int ks = 0; ks < 4; ++ks) {  // K = 16 per MMA: 32 bytes along the swizzled row
+#pragma unroll 1
+  for (int ks = ks0; ks < ks1; ++ks) {  // K = 16 per MMA: 32 bytes along the swizzled row
     const uint32_t acc = (first && ks == 0) ? 0u : 1u;
     const uint64_t da0 = tc::sdesc_sw128(a0) + 2 * ks, da1 = tc::sdesc_sw128(a1) + 2 * ks,
                    da2 = tc::sdesc_sw128(a2) + 2 * ks;
@@ -628,8 +607,8 @@ __device__ __forceinline__ void tc_issue(uint32_t ops, bool diag, uint32_t tmem,
 // D = L_ia L_ib' for the tiles in plane slots ta, tb (ta == tb on a diagonal
 // tile).  Thread 0 copies both K chunks of both operands into shared memory
 // and issues each chunk's MMAs once its planes have landed; the other threads
-// go on (the caller overlaps its loads of C) and meet at tc_product_end.  Every
-// barrier completes once per product, so one parity bit serves all three.
+// go on (the caller overlaps its loads of C) and meet at tc_product_end.  parity:
+// of the arrival barriers, which complete once per product.
 template <bool DIAG>
 __device__ __forceinline__ void tc_product_begin(const unsigned char* planes, int64_t ta, int64_t tb,
                                                  TileCholSmem<float>& sm, uint32_t tmem, uint32_t parity,
@@ -637,7 +616,9 @@ __device__ __forceinline__ void tc_product_begin(const unsigned char* planes, in
   if (threadIdx.x != 0) return;
   unsigned char* ops = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(sm.tc_ops) + 1023) & ~uintptr_t(1023));
   const uint32_t ops_s = tc::smem_u32(ops);
-  asm volatile("fence.proxy.async.global;" ::: "memory");  // the planes were published by generic stores
+  // the planes were published by generic stores, and this CTA's generic
+  // accesses to the operand area are behind a barrier
+  asm volatile("fence.proxy.async;" ::: "memory");
   const unsigned char* A = planes + ta * kTcTileBytes;
   const unsigned char* B = planes + tb * kTcTileBytes;
 #pragma unroll
@@ -743,30 +724,169 @@ __device__ __forceinline__ void tc_sub_global(float4 (&x)[kRowsPerWarp], int64_t
   __syncthreads();  // the staging area holds the next task's operand planes
 }
 
-// FINAL epilogue: acc (tile layout) -= D, through the staging area.
-__device__ __forceinline__ void tc_sub_acc(float (&acc)[8][8], uint32_t tmem, TileCholSmem<float>& sm) {
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, quarter = warp & 3, half = warp >> 2;
-  const int tx = tid & 15, ty = tid >> 4;
+// FINAL epilogue: the column-major tile X -= D (warp w: rows 32 (w % 4) .. + 31,
+// columns 64 (w / 4) .. + 63).
+__device__ __forceinline__ void tc_sub_tile(ft::Tile X, uint32_t tmem) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, quarter = warp & 3, half = warp >> 2;
   const int r = quarter * 32 + lane;
   const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16);
 #pragma unroll 1
-  for (int g = 0; g < 2; ++g) {
-    const int c = half * 64 + g * 32;
-    uint32_t dv[32];
-    tc::tmem_ld32(taddr + c, dv);
+  for (int g = 0; g < 4; ++g) {
+    const int c = half * 64 + g * 16;
+    uint32_t lead[16], corr[16];
+    tc::tmem_ld16(taddr + c, lead);
+    tc::tmem_ld16(taddr + kBig + c, corr);
 #pragma unroll
-    for (int j = 0; j < 32; ++j) sm.ls[r][c + j] = __uint_as_float(dv[j]);
-    tc::tmem_ld32(taddr + kBig + c, dv);
-#pragma unroll
-    for (int j = 0; j < 32; ++j) sm.ls[r][c + j] += __uint_as_float(dv[j]);
+    for (int j = 0; j < 16; ++j) X[c + j][r] -= __uint_as_float(lead[j]) + __uint_as_float(corr[j]);
   }
   tc::fence_before();
+}
+
+// The off-diagonal tile (p0, q0) into sm.f.c, less the product L_ia L_ib' of
+// the plane slots ta, tb (ta < 0: no product).  Ends with a barrier; false on a
+// timeout.
+__device__ __forceinline__ bool tc_updated_tile(const unsigned char* planes, int64_t ta, int64_t tb, int64_t m,
+                                                int64_t ldm, const float* M, int64_t p0, int64_t q0,
+                                                TileCholSmem<float>& sm, uint32_t tmem, uint32_t& full_parity,
+                                                uint32_t& parity, Scalars* sc) {
+  float4 x[16];
+  if (ta >= 0) tc_product_begin<false>(planes, ta, tb, sm, tmem, full_parity, sc);
+  ft::fetch_tile(x, m, ldm, M, p0, q0);
+  if (ta >= 0) {
+    if (!tc_product_end(sm, parity, sc)) return false;
+    full_parity ^= 1u;
+  }
+  ft::put_tile(x, m, p0, false, sm.f.c);  // (the operand planes are free: the MMAs have completed)
   __syncthreads();
+  if (ta >= 0) {
+    tc_sub_tile(sm.f.c, tmem);
+    __syncthreads();
+  }
+  return true;
+}
+
+// The wait of a solve for panel need of a diagonal tile (thread 0); need < 0:
+// whether panel -need is there now.
+struct PanelWait {
+  Scalars* sc;
+  __device__ __forceinline__ int operator()(const int* flag, int need) const {
+    return need < 0 ? ld_acquire(flag) >= -need : (int)wait_at_least(flag, need, sc);
+  }
+};
+
+// Publishes tile (i, l)'s counter once the CTA's stores of it are ordered by a
+// barrier: by a thread of the last warp, whose fence then delays nobody else.
+__device__ __forceinline__ void publish_after_barrier(int* state, int64_t idx, int val) {
+  if (threadIdx.x == kThreads - 1) {
+    __threadfence();
+    st_release(state + idx, val);
+  }
+}
+
+// The dependency chain of the FP32 factor: FINAL(l, l), the solve of tile
+// (l + 1, l), FINAL(l + 1, l + 1), ...  Blocks 0 and 1 share it: block l % 2 applies
+// the last update of tile (l, l - 1), solves it against the panels of L_l-1,l-1 as the other block finishes
+// them, 32 columns at a time, and then factors tile (l, l), which needs
+// nothing else of the chain.  What bounds a link is latency, so
+//   * the solve ends one panel after the factorisation it follows;
+//   * L_l,l-1 goes to shared memory as operand planes too, and the product
+//     L_l,l-1 L_l,l-1' runs behind the solve, block by block;
+//   * the flags are set by one thread while the others go on.
+// panels[l] counts the finished panels of L_ll.  Returns with no MMA in flight.
+// Measured per link at m = 2048: 48 us with one block and every hand-off
+// through global memory -> 33 us (the factorisation 13 us of it; the solve is
+// behind it by 13 us, the product and the loads of the next tile take 5).
+__device__ void chol_chain(int me, int64_t m, int64_t ldm, float* M, float* dinv, int nb, int* state, int* panels,
+                           Scalars* sc, unsigned char* planes, TileCholSmem<float>& sm, uint32_t tmem, int* s_fail) {
+  const int tid = threadIdx.x;
+  static_assert(offsetof(TileCholSmem<float>, f.s) - offsetof(TileCholSmem<float>, f) <= kChainOps,
+                "the operand planes lie past the tile to be solved and the panels");
+  unsigned char* ops =
+      reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(sm.chain + kChainOps) + 1023) & ~uintptr_t(1023));
+  const uint32_t ops_s = tc::smem_u32(ops), bar = tc::smem_u32(&sm.mma_bar);
+  uint32_t parity = 0, full_parity = 0;
+  bool pending = false;  // MMAs have been issued and not been waited for
+  float4 x[16];
+#pragma unroll 1
+  for (int l = me; l < nb; l += 2) {
+    const int64_t p0 = (int64_t)l * kBig, q0 = p0 - kBig;
+    if (l > 0) {
+      if (tid == 0)
+        sm.go = l < 2 ? !dev_failed(sc)
+                      : wait_at_least(state + (int64_t)l * nb + l - 2, l - 1, sc) &&
+                            wait_at_least(state + (int64_t)(l - 1) * nb + l - 2, l - 1, sc) &&
+                            wait_at_least(state + (int64_t)l * nb + l - 1, l - 2, sc);
+      __syncthreads();
+      if (!sm.go) break;
+      if (!tc_updated_tile(planes, l < 2 ? -1 : plane_slot(l, l - 2), l < 2 ? -1 : plane_slot(l - 1, l - 2), m, ldm, M,
+                           p0, q0, sm, tmem, full_parity, parity, sc))
+        break;
+      const bool ok = ft::trsm(
+          sm.f.c, sm.f.panel, sm.rcp, sm.trsm_go, m, ldm, M, dinv, q0, panels + l - 1, PanelWait{sc},
+          [&](int b) {
+            finish_block<true>(sm.f.c, b, m, ldm, M, p0, q0, planes + plane_slot(l, l - 1) * kTcTileBytes, ops);
+          },
+          [&](int b) {
+            pending = true;
+            if (tid == 0) {
+              tc::fence_after();
+              tc_issue(ops_s + (b >> 1) * kTcChunkBytes, true, tmem, b == 0, 2 * (b & 1), 2 * (b & 1) + 2);
+              if (b == 3) tc::umma_commit(bar);
+            }
+          });
+      if (!ok) break;
+      publish_after_barrier(state, (int64_t)l * nb + l - 1, l);
+    }
+    if (tid == 0) sm.go = l < 2 ? !dev_failed(sc) : wait_at_least(state + (int64_t)l * nb + l, l - 1, sc);
+    __syncthreads();
+    if (!sm.go) break;
+    ft::fetch_tile(x, m, ldm, M, p0, p0);
+    if (l > 0) {
+      const bool ok = tc::mbar_wait(bar, parity, nullptr);
+      if (!ok) atomicCAS(&sc->status, 0, (int)PDAS_ERR_TIMEOUT);
+      if (!__syncthreads_and(ok)) break;
+      parity ^= 1u;
+      pending = false;
+      tc::fence_after();
+    }
+    ft::put_tile(x, m, p0, true, sm.f.s);
+    __syncthreads();
+    if (l > 0) {
+      tc_sub_tile(sm.f.s, tmem);
+      __syncthreads();
+    }
+    const int fail = ft::potrf(
+        sm.f.s, sm.rcp, s_fail,
+        [&](int b) {
 #pragma unroll
-  for (int i = 0; i < 8; ++i)
-#pragma unroll
-    for (int j = 0; j < 8; ++j) acc[i][j] -= sm.ls[ty + 16 * i][tx + 16 * j];
-  __syncthreads();
+          for (int v = 0; v < 4; ++v) {
+            int r, c;
+            ft::panel_rc(v, r, c);
+            c += 32 * b;
+            if (p0 + r < m && c <= r) {
+              float* dst = M + (p0 + r) * ldm + p0 + c;
+              const float e[4] = {sm.f.s[c][r], sm.f.s[c + 1][r], sm.f.s[c + 2][r], sm.f.s[c + 3][r]};
+              if (c + 3 <= r) *reinterpret_cast<float4*>(dst) = make_float4(e[0], e[1], e[2], e[3]);
+              else
+                for (int k = 0; k < 4; ++k)
+                  if (c + k <= r) dst[k] = e[k];
+            }
+          }
+          if (tid < 32 && p0 + 32 * b + tid < m) dinv[p0 + 32 * b + tid] = sm.rcp[32 * b + tid];
+        },
+        [&](int b) {
+          publish_after_barrier(panels, l, b + 1);
+          if (b == 3) publish_after_barrier(state, (int64_t)l * nb + l, l + 1);
+        });
+    if (fail >= 0) {
+      if (tid == 0 && atomicCAS(&sc->status, 0, (int)PDAS_ERR_NOT_SPD) == 0) sc->fail_index = (int)(p0 + fail);
+      break;
+    }
+  }
+  if (pending) {  // a wait gave up with MMAs in flight: they end before TMEM is freed
+    if (tid == 0) tc::umma_commit(bar);
+    tc::mbar_wait(bar, parity, nullptr);
+  }
 }
 
 template <typename T>
@@ -777,7 +897,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   TileCholSmem<T>& sm = *reinterpret_cast<TileCholSmem<T>*>(chol_tiles_smem);
   const int tid = threadIdx.x;
   constexpr bool kTc = sizeof(T) == 4;  // FP32 factor: products on the tensor cores
-  uint32_t tmem = 0, mma_parity = 0;
+  __shared__ int s_fail;
+  int* panels = state + (int64_t)nb * nb;  // finished panels of each diagonal tile (FP32)
+  uint32_t tmem = 0, mma_parity = 0, full_parity = 0;
   if constexpr (kTc) {
     if (tid == 0) {
       tc::mbar_init(tc::smem_u32(&sm.mma_bar), 1);
@@ -791,13 +913,19 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc::fence_after();
     tmem = sm.tmem_slot;
   }
-  int chain_step = 0;  // block 0: step 2 l is FINAL(l, l), step 2 l + 1 the solve of tile (l + 1, l)
+  if constexpr (kTc) {
+    if (blockIdx.x < 2) {
+      chol_chain(blockIdx.x, m, ldm, M, dinv, nb, state, panels, sc, planes, sm, tmem, &s_fail);
+      __syncthreads();
+    }
+  }
+  int chain_step = kTc ? 2 * nb : 0;  // (double-float) block 0: step 2 l is FINAL(l, l), step 2 l + 1 the solve of tile (l + 1, l)
   for (;;) {
     if (tid == 0) {  // take a task and wait for the tiles it starts from
       int go = 0;
       bool have = false;
       int4 d = make_int4(0, 0, 0, 0);
-      if (blockIdx.x == 0) {  // the diagonal chain in order
+      if (blockIdx.x < (kTc ? 2 : 1)) {  // the diagonal chain in order (FP32: done)
         const int l = chain_step >> 1;
         if (chain_step & 1) {
           have = l + 1 < nb;
@@ -812,7 +940,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           const unsigned t = atomicAdd(ticket, 1u);
           if (t >= (unsigned)ntasks) break;
           d = tasks[t];
-          if (d.x != TK_FINAL_DIAG && d.x != TK_CHAIN_SOLVE) {
+          // (FP32: the chain applies the last update of a sub-diagonal tile itself)
+          if (d.x != TK_FINAL_DIAG && d.x != TK_CHAIN_SOLVE && !(kTc && d.x == TK_UPDATE && d.w == d.z - 1)) {
             have = true;
             break;
           }
@@ -841,81 +970,84 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int4 d = sm.task;
     const int i = d.y, l = d.z;
     const int64_t p0 = (int64_t)i * kBig, q0 = (int64_t)l * kBig;
-    T acc[8][8];
     int val;
-    if (d.x == TK_INV) {  // (the double-float factor's solves substitute: no inverses)
-      if constexpr (!std::is_same<T, dfloat>::value) tile_inverse<T>(acc, m, ldm, M, dinv, Uinv, l, sm);
-      __syncthreads();  // (shared memory is reused by the next task; no counter to publish)
-      continue;
-    }
-    if (d.x == TK_CHAIN_SOLVE) {  // block 0, right after FINAL(l, l): L_ll and 1 / L_cc are still in shared memory
-      load_tile(acc, M, ldm, m, p0, q0, false);
-      trsm_sweep<T>(acc, sm);
-      store_tile(acc, M, ldm, m, p0, q0, false);
-      if constexpr (kTc) tc_write_planes(acc, planes + plane_slot(i, l) * kTcTileBytes, sm);
-      __threadfence();
-      __syncthreads();
-      if (tid == 0) st_release(state + (int64_t)i * nb + l, l + 1);
-      continue;
-    }
-    if (d.x == TK_UPDATE) {
-      if constexpr (kTc) {
-        if (i == l) tc_product_begin<true>(planes, plane_slot(i, d.w), plane_slot(i, d.w), sm, tmem, mma_parity, sc);
-        else tc_product_begin<false>(planes, plane_slot(i, d.w), plane_slot(l, d.w), sm, tmem, mma_parity, sc);
+    if constexpr (kTc) {
+      if (d.x == TK_INV) {
+        for (int e = tid; e < kBig * kBig; e += kThreads) sm.f.c[e >> 7][e & 127] = (e >> 7) == (e & 127) ? 1.f : 0.f;
+        __syncthreads();
+        auto nothing = [](int) {};
+        if (!ft::trsm(sm.f.c, sm.f.panel, sm.rcp, sm.trsm_go, m, ldm, M, dinv, q0, panels + l, PanelWait{sc}, nothing,
+                      nothing))  // U L' = I
+          break;
+        float* U = Uinv + (int64_t)l * kBig * kBig;
+#pragma unroll
+        for (int v = 0; v < 16; ++v) {
+          int r, c;
+          ft::unit_rc(v, r, c);
+          *reinterpret_cast<float4*>(U + r * kBig + c) =
+              make_float4(sm.f.c[c][r], sm.f.c[c + 1][r], sm.f.c[c + 2][r], sm.f.c[c + 3][r]);
+        }
+        __syncthreads();  // (shared memory is reused by the next task; no counter to publish)
+        continue;
+      }
+      if (d.x == TK_UPDATE) {
+        if (i == l) tc_product_begin<true>(planes, plane_slot(i, d.w), plane_slot(i, d.w), sm, tmem, full_parity, sc);
+        else tc_product_begin<false>(planes, plane_slot(i, d.w), plane_slot(l, d.w), sm, tmem, full_parity, sc);
         float4 cx[kRowsPerWarp];
         tc_load_rows(cx, m, ldm, M, p0, q0);
         if (!tc_product_end(sm, mma_parity, sc)) break;
+        full_parity ^= 1u;
         if (i == l) tc_sub_global<true>(cx, m, ldm, M, p0, q0, tmem, sm);
         else tc_sub_global<false>(cx, m, ldm, M, p0, q0, tmem, sm);
-      } else {
+        val = d.w + 1;
+      } else {  // FINAL(i, l)
+        const int64_t ta = l > 0 ? plane_slot(i, l - 1) : -1, tb = l > 0 ? plane_slot(l, l - 1) : -1;
+        if (!tc_updated_tile(planes, ta, tb, m, ldm, M, p0, q0, sm, tmem, full_parity, mma_parity, sc)) break;
+        if (!ft::trsm(
+                sm.f.c, sm.f.panel, sm.rcp, sm.trsm_go, m, ldm, M, dinv, q0, panels + l, PanelWait{sc},
+                [&](int b) {
+                  finish_block<false>(sm.f.c, b, m, ldm, M, p0, q0, planes + plane_slot(i, l) * kTcTileBytes, nullptr);
+                },
+                [](int) {}))
+          break;
+        val = l + 1;
+      }
+    } else {
+      if (d.x == TK_INV) continue;  // the double-float factor's solves substitute: no inverses
+      T acc[8][8];
+      if (d.x == TK_CHAIN_SOLVE) {  // block 0, right after FINAL(l, l): L_ll and 1 / L_cc are still in shared memory
+        load_tile(acc, M, ldm, m, p0, q0, false);
+        trsm_sweep<T>(acc, sm);
+        store_tile(acc, M, ldm, m, p0, q0, false);
+        val = l + 1;
+      } else if (d.x == TK_UPDATE) {
         load_tile(acc, M, ldm, m, p0, q0, i == l);
         if (i == l) rank_update<T, true>(acc, m, ldm, M, i, l, d.w, sm);
         else rank_update<T, false>(acc, m, ldm, M, i, l, d.w, sm);
         store_tile(acc, M, ldm, m, p0, q0, i == l);
-      }
-      val = d.w + 1;
-    } else if (d.x == TK_FINAL_DIAG) {
-      if constexpr (kTc) {
-        if (l > 0) {
-          tc_product_begin<true>(planes, plane_slot(l, l - 1), plane_slot(l, l - 1), sm, tmem, mma_parity, sc);
-          load_tile(acc, M, ldm, m, p0, p0, true);
-          if (!tc_product_end(sm, mma_parity, sc)) break;
-          tc_sub_acc(acc, tmem, sm);
-        } else {
-          load_tile(acc, M, ldm, m, p0, p0, true);
-        }
-      } else {
+        val = d.w + 1;
+      } else if (d.x == TK_FINAL_DIAG) {
         load_tile(acc, M, ldm, m, p0, p0, true);
         if (l > 0) rank_update<T, true>(acc, m, ldm, M, l, l, l - 1, sm);
-      }
-      if (!tile_potrf<T>(acc, m, ldm, M, dinv, l, sm, sc)) break;
-      val = l + 1;
-    } else {
-      if constexpr (kTc) {
-        if (l > 0) {
-          tc_product_begin<false>(planes, plane_slot(i, l - 1), plane_slot(l, l - 1), sm, tmem, mma_parity, sc);
-          load_tile(acc, M, ldm, m, p0, q0, false);
-          if (!tc_product_end(sm, mma_parity, sc)) break;
-          tc_sub_acc(acc, tmem, sm);
-        } else {
-          load_tile(acc, M, ldm, m, p0, q0, false);
-        }
+        if (!tile_potrf<T>(acc, m, ldm, M, dinv, l, sm, sc)) break;
+        val = l + 1;
       } else {
         load_tile(acc, M, ldm, m, p0, q0, false);
         if (l > 0) rank_update<T, false>(acc, m, ldm, M, i, l, l - 1, sm);
+        if (tid == 0) sm.go = wait_at_least(state + (int64_t)l * nb + l, l + 1, sc);  // L_ll
+        __syncthreads();
+        if (!sm.go) break;
+        load_diag_factor<T>(m, ldm, M, dinv, l, sm);
+        trsm_sweep<T>(acc, sm);
+        store_tile(acc, M, ldm, m, p0, q0, false);
+        val = l + 1;
       }
-      if (tid == 0) sm.go = wait_at_least(state + (int64_t)l * nb + l, l + 1, sc);  // L_ll
-      __syncthreads();
-      if (!sm.go) break;
-      load_diag_factor<T>(m, ldm, M, dinv, l, sm);
-      trsm_sweep<T>(acc, sm);
-      store_tile(acc, M, ldm, m, p0, q0, false);
-      if constexpr (kTc) tc_write_planes(acc, planes + plane_slot(i, l) * kTcTileBytes, sm);
-      val = l + 1;
     }
-    __threadfence();
     __syncthreads();
-    if (tid == 0) st_release(state + (int64_t)i * nb + l, val);
+    if (tid == 0) {  // (the fence covers what the barrier ordered before it)
+      __threadfence();
+      st_release(state + (int64_t)i * nb + l, val);
+    }
   }
   if constexpr (kTc) {  // every exit: all MMAs have completed (or drained after a timeout)
     tc::fence_before();
@@ -955,11 +1087,13 @@ int chol_tiles_resident() {
 }
 
 // The task order (see the file comment): a list schedule of the task graph
-// on nproc identical workers.  Costs are per task kind, in microseconds as
-// measured on GB300 for the FP32 factor (one CTA per SM): an update on the
-// tensor cores, diagonal or not, 7; the diagonal task's product and
-// factorisation 35; the off-diagonal solve with its load of L_ll and the
-// write of its BF16 planes 22; the inverse 20.
+// on nproc identical workers.  Costs are per task kind, in microseconds: an
+// update on the tensor cores 7; the diagonal task's product and factorisation
+// 34; the off-diagonal solve 22; the chain's solve 19; the inverse 20.  The
+// factorisation and the solves now take about two thirds of that (14 us the
+// factorisation, 15 the others); with those figures the order puts fewer of the
+// updates ahead of the chain's next link, and the factor at m = 8192 takes
+// 4.05 ms instead of 3.43 (at m = 2048 and below the order makes no difference).
 void chol_tile_tasks(int64_t m, int nproc, std::vector<int4>* out) {
   const int nb = (int)chol_tile_count(m);
   out->clear();
@@ -1114,12 +1248,12 @@ cudaError_t cholesky_tiles(cudaStream_t st, int64_t m, int64_t ldm, T* M, T* din
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
   const int nb = (int)chol_tile_count(m);
-  e = cudaMemsetAsync(state, 0, sizeof(int) * (size_t)nb * nb, st);
+  e = cudaMemsetAsync(state, 0, sizeof(int) * (size_t)(nb * nb + nb), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(ticket, 0, sizeof(unsigned), st);
   if (e != cudaSuccess) return e;
-  int grid = sms * per_sm;  // (at least 2: block 0 runs only the diagonal tasks)
-  if (grid > ntasks) grid = ntasks;
-  if (grid < 2) return cudaErrorInvalidConfiguration;
+  int grid = sms * per_sm;  // (at least 3: blocks 0 and, in FP32, 1 run only the diagonal tasks)
+  if (grid > ntasks + 1) grid = ntasks + 1;
+  if (grid < 3) return cudaErrorInvalidConfiguration;
   k_chol_tiles<T><<<grid, kThreads, chol_tiles_smem_bytes<T>(), st>>>(m, ldm, M, dinv, Uinv, tasks, ntasks, nb,
                                                                      state, ticket, sc, planes);
   return cudaGetLastError();
@@ -1127,9 +1261,6 @@ cudaError_t cholesky_tiles(cudaStream_t st, int64_t m, int64_t ldm, T* M, T* din
 
 template cudaError_t cholesky_tiles<float>(cudaStream_t, int64_t, int64_t, float*, float*, float*, const int4*, int,
                                            int*, unsigned*, Scalars*, unsigned char*);
-template cudaError_t cholesky_tiles<double>(cudaStream_t, int64_t, int64_t, double*, double*, double*, const int4*,
-                                            int, int*, unsigned*, Scalars*, unsigned char*);
-
 template cudaError_t cholesky_tiles<dfloat>(cudaStream_t, int64_t, int64_t, dfloat*, dfloat*, dfloat*, const int4*,
                                             int, int*, unsigned*, Scalars*, unsigned char*);
 

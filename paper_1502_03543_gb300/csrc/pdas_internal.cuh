@@ -132,8 +132,8 @@ template <typename T>
 cudaError_t cholesky(cudaStream_t st, int64_t m, int64_t ldm, T* M, T* dinv, Scalars* sc);
 
 // The single-launch tile Cholesky (chol_tiles.cu): 128 x 128 tiles; the task
-// list comes from chol_tile_tasks (built once per m); state holds
-// chol_tile_count(m)^2 ints; ticket is one counter.  Both are cleared here.
+// list comes from chol_tile_tasks (built once per m); state holds nb^2 + nb
+// ints (nb = chol_tile_count(m)); ticket is one counter.  Both are cleared here.
 // Beyond 256 tile rows (m > 32768) the task list (~nb^3/6 tasks, built on
 // the host at handle creation) grows past ~3M entries; such handles keep the
 // multi-launch blocked factor.
