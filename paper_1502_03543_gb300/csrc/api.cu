@@ -23,6 +23,7 @@
 
 #include "pdas_internal.cuh"
 #include "chol_dig.cuh"
+#include "passes.cuh"
 #include "syrk_dig.cuh"
 #include "syrk_simt.cuh"
 #include "syrk_tc.cuh"
@@ -30,21 +31,26 @@
 using namespace pdas;
 
 struct pdas_ctx {
+  std::vector<void*> allocs;  // every device allocation of the handle itself
   int64_t m = 0, n = 0, ldm = 0;
   pdas_options opt{};
   cudaStream_t st = nullptr;
   // FP64 vectors
   double *D = nullptr, *r = nullptr, *dy = nullptr, *dx = nullptr, *ds = nullptr, *w = nullptr, *u = nullptr;
   double *z = nullptr, *rho = nullptr, *delta = nullptr, *kp = nullptr, *kq = nullptr, *kz = nullptr;
+  double* kp2 = nullptr;      // the search direction of every other step
+  double* zb = nullptr;       // hand-off of the blocked FP32 solves (all unset between them)
+  bool solve_dirty = false;   // a call failed: zb and the tickets have to be set again
   double* rd = nullptr;       // infeasible-start variant: dual residual c - A'y - s (n)
   double* part = nullptr;     // reduction partials (kPartMax)
-  double* gt_part = nullptr;  // gemv_t partials, gt_chunks x n
-  int gt_chunks = 1;
-  int64_t gt_rows = 1;
+  double* gt_part = nullptr;  // partial column sums of A'u
+  unsigned* ctickets = nullptr;  // ... and its column blocks' tickets, zero between launches
   unsigned* tickets = nullptr;
   int* flags = nullptr;
   Scalars* sc = nullptr;
-  Scalars* sc_host = nullptr;  // pinned
+  Scalars* sc_host = nullptr;  // pinned; written by the device (read_scalars)
+  unsigned* sc_seq = nullptr;  // ... and the number of the snapshot in it
+  unsigned seq = 0;            // number of the last snapshot asked for
   int wait_us = 0;             // limit of the bounded inter-block waits (0: the 2 s default)
   int* wait_pinned = nullptr;  // pinned copy of wait_us, the source of its copy into sc
   double* M64 = nullptr;      // FP64 form; mixed forms: the FP64 tier's matrix (allocated at create)
@@ -78,7 +84,7 @@ struct pdas_ctx {
   int* chol_state = nullptr;    // counters of the tile Cholesky: per tile, then panels per diagonal tile
   float* uinv32 = nullptr;      // L_ll^{-T} of every diagonal tile of the FP32 tile factor
   unsigned char* chol_planes = nullptr;  // BF16 operand planes of the tile factor's off-diagonal tiles
-  float2* pairs = nullptr;      // the vector of a double-float pass as FP32 pairs (max(m, n))
+  float* pairs = nullptr;       // the vector of a double-float pass as FP32 pairs (n, two planes)
   int switch_reason = 0;  // pdas_iter_info.fp64_reason of that switch
   bool last_factor_df = false;    // the last factor was a fast FP64-tier factor (tensor-core or double-float)
   double last_rel_gap = HUGE_VAL;  // relative gap of the iterate after the last step
@@ -195,21 +201,42 @@ pdas_status with_dtype(int dt, F&& f) {
   return PDAS_ERR_ARG;
 }
 
-// Reads the device scalars (one small copy + stream sync).
+// Reads the device scalars: a one-warp launch writes them to pinned host memory,
+// then the snapshot's number, for which the host polls.  A copy and a stream
+// synchronisation take 12-15 us from the last kernel's end to the next launch
+// (two to five times per direction), this about 7 (512 x 2048: 499 -> 475 us
+// a direction).  Nothing is left running: the snapshot is the stream's last launch.
 pdas_status read_scalars(pdas_ctx* h) {
-  CK(cudaMemcpyAsync(h->sc_host, h->sc, sizeof(Scalars), cudaMemcpyDeviceToHost, h->st));
-  CK(cudaStreamSynchronize(h->st));
-  return PDAS_OK;
+  const unsigned want = ++h->seq;
+  KL(launch_snapshot(h->st, h->sc, h->sc_host, h->sc_seq, want), 1);
+  for (unsigned spin = 1;; ++spin) {
+    if (__atomic_load_n(h->sc_seq, __ATOMIC_ACQUIRE) == want) return PDAS_OK;
+    if ((spin & 0xfff) == 0) {  // an error on the stream (or a capture) never writes it
+      const cudaError_t e = cudaStreamQuery(h->st);
+      if (e == cudaErrorNotReady) continue;
+      CK(e);
+      if (__atomic_load_n(h->sc_seq, __ATOMIC_ACQUIRE) == want) return PDAS_OK;
+      CK(cudaStreamSynchronize(h->st));
+      if (__atomic_load_n(h->sc_seq, __ATOMIC_ACQUIRE) == want) return PDAS_OK;
+      return cuda_fail(h, cudaErrorUnknown, "scalars not written");
+    }
+  }
 }
 
 pdas_status device_status(pdas_ctx* h) {
   const Scalars& s = *h->sc_host;
+  if (s.status != 0) h->solve_dirty = true;  // launches may have stopped between a ticket and its reset
   if (s.status == PDAS_ERR_NOT_SPD) h->err_index = s.fail_index;
   return (pdas_status)s.status;
 }
 
 pdas_status reset_status(pdas_ctx* h) {
   CK(cudaMemsetAsync(h->sc, 0, sizeof(Scalars), h->st));
+  if (h->solve_dirty) {
+    CK(cudaMemsetAsync(h->tickets, 0, sizeof(unsigned) * T_COUNT, h->st));
+    if (h->zb) CK(cudaMemsetAsync(h->zb, 0xff, sizeof(double) * h->m, h->st));
+    h->solve_dirty = false;
+  }
   if (h->wait_us > 0)  // a limit of the handle's own (pdas_set_wait_limit)
     CK(cudaMemcpyAsync(&h->sc->wait_us, h->wait_pinned, sizeof(int), cudaMemcpyHostToDevice, h->st));
   return PDAS_OK;
@@ -228,47 +255,35 @@ pdas_status reset_status(pdas_ctx* h) {
 // pdas_gemv_t of a mixed handle expose the double-float pass itself.
 bool df_passes(const pdas_ctx* h) { return is_mixed(h) && h->opt.a_dtype != PDAS_A_F64 && !h->opt.exact_passes; }
 
+// df: h->pairs holds the FP32 pairs of v, or (v given) receives them first.
+// dot: also sum_p dot_p out_p into sc->dot_b.
 pdas_status gemv(pdas_ctx* h, const void* A, const double* v, const double* base, double* out, int norm_slot,
-                 bool df = false) {
-  if (df) {
-    KL(launch_split_pairs(h->st, h->n, v, h->pairs), 1);
-    if (h->opt.a_dtype == PDAS_A_F32)
-      KL(launch_gemv_df<float>(h->st, h->m, h->n, (const float*)A, h->pairs, base, out, h->part, h->tickets, h->sc,
-                               norm_slot), 1);
-    else
-      KL(launch_gemv_df<__nv_bfloat16>(h->st, h->m, h->n, (const __nv_bfloat16*)A, h->pairs, base, out, h->part,
-                                       h->tickets, h->sc, norm_slot), 1);
-    return PDAS_OK;
-  }
+                 bool df = false, const double* dot = nullptr) {
+  if (df && v) KL(launch_split_pairs(h->st, h->n, v, h->pairs), 1);
   return with_dtype(h->opt.a_dtype, [&](auto tag) -> pdas_status {
     using T = std::remove_const_t<std::remove_pointer_t<decltype(tag)>>;
-    KL(launch_gemv<T>(h->st, h->m, h->n, (const T*)A, v, base, out, h->part, h->tickets, h->sc, norm_slot), 1);
+    KL(launch_pass<T>(h->st, h->m, h->n, (const T*)A, v, df ? h->pairs : nullptr, base, out, h->part, h->tickets,
+                      h->sc, norm_slot, dot), 1);
     return PDAS_OK;
   });
 }
 
-// w = A' u, then the finish mode (see launch_gemv_t_finish).
-pdas_status gemv_t(pdas_ctx* h, const void* A, const double* u, int mode, const double* x, double* o0, double* o1,
-                   double* o2, bool df = false, const double* rd = nullptr) {
-  if (df) {
-    KL(launch_split_pairs(h->st, h->m, u, h->pairs), 1);
-    if (h->opt.a_dtype == PDAS_A_F32)
-      KL(launch_gemv_t_df<float>(h->st, h->m, h->n, (const float*)A, h->pairs, h->gt_part, h->gt_chunks, h->gt_rows),
-         1);
-    else
-      KL(launch_gemv_t_df<__nv_bfloat16>(h->st, h->m, h->n, (const __nv_bfloat16*)A, h->pairs, h->gt_part,
-                                         h->gt_chunks, h->gt_rows), 1);
-    KL(launch_gemv_t_finish(h->st, h->n, h->gt_chunks, h->gt_part, mode, x, h->D, o0, o1, o2, h->sc, rd), 1);
-    return PDAS_OK;
-  }
-  pdas_status s = with_dtype(h->opt.a_dtype, [&](auto tag) -> pdas_status {
+// w = A'(src), then the mode of launch_pass_t; pairs: the FP32 pairs of D w to
+// h->pairs (mode 2).
+pdas_status gemv_t(pdas_ctx* h, const void* A, const PassTSrc& src, int mode, const double* x, double* o0, double* o1,
+                   double* o2, bool df = false, const double* rd = nullptr, bool pairs = false) {
+  return with_dtype(h->opt.a_dtype, [&](auto tag) -> pdas_status {
     using T = std::remove_const_t<std::remove_pointer_t<decltype(tag)>>;
-    KL(launch_gemv_t<T>(h->st, h->m, h->n, (const T*)A, u, h->gt_part, h->gt_chunks, h->gt_rows), 1);
+    KL(launch_pass_t<T>(h->st, h->m, h->n, (const T*)A, df, src, h->gt_part, h->part + 3 * kPartMax, h->ctickets, mode,
+                        x, h->D, o0, o1, o2, pairs ? h->pairs : nullptr, h->sc, rd), 1);
     return PDAS_OK;
   });
-  if (s != PDAS_OK) return s;
-  KL(launch_gemv_t_finish(h->st, h->n, h->gt_chunks, h->gt_part, mode, x, h->D, o0, o1, o2, h->sc, rd), 1);
-  return PDAS_OK;
+}
+pdas_status gemv_t(pdas_ctx* h, const void* A, const double* u, int mode, const double* x, double* o0, double* o1,
+                   double* o2, bool df = false, const double* rd = nullptr) {
+  PassTSrc src;
+  src.u = u;
+  return gemv_t(h, A, src, mode, x, o0, o1, o2, df, rd);
 }
 
 bool want_fp64(const pdas_ctx* h) { return !is_mixed(h) || h->refactored; }
@@ -416,8 +431,20 @@ pdas_status factor(pdas_ctx* h) {
   return PDAS_OK;
 }
 
-// out = (L L')^{-1} rhs with the current factor (via h->z).
-pdas_status factor_solve(pdas_ctx* h, const double* rhs, double* out) {
+// out = (L L')^{-1} rhs with the current factor.  upd: first that step of the
+// conjugate gradients on rhs = h->rho; *nrz: then rhs'out as *nrz parts at
+// rz_part(h).
+double* rz_part(pdas_ctx* h) { return h->part + 2 * kPartMax; }
+
+pdas_status factor_solve(pdas_ctx* h, double* rhs, double* out, const CgStep* upd = nullptr, int* nrz = nullptr) {
+  if (!h->cur_f64 && h->chol_ntasks > 0) {  // the tile factor, with the inverses of its diagonal tiles
+    KL(trsv_blk_solve(h->st, h->m, h->ldm, h->M32, h->uinv32, rhs, h->zb, out, upd, nrz ? rz_part(h) : nullptr,
+                      h->part, h->tickets + T_TRSVB, h->sc),
+       2);
+    if (nrz) *nrz = (int)chol_tile_count(h->m);
+    return PDAS_OK;
+  }
+  if (upd) KL(launch_cg_update(h->st, h->m, *upd, rhs, h->part, h->tickets, h->sc), 1);
   if (h->cur_f64) {
     KL(trsv_lower<double>(h->st, h->m, h->ldm, h->M64, h->dinv64, rhs, h->z, h->flags, h->tickets, h->sc,
                           is_mixed(h)),
@@ -425,36 +452,16 @@ pdas_status factor_solve(pdas_ctx* h, const double* rhs, double* out) {
     KL(trsv_upper_t<double>(h->st, h->m, h->ldm, h->M64, h->dinv64, h->z, out, h->flags, h->tickets, h->sc,
                             is_mixed(h)),
        1);
-  } else if (h->chol_ntasks > 0) {  // the tile factor, with the inverses of its diagonal tiles
-    KL(trsv_lower_blk(h->st, h->m, h->ldm, h->M32, h->uinv32, rhs, h->z, h->tickets + T_TRSV, h->sc), 1);
-    KL(trsv_upper_blk(h->st, h->m, h->ldm, h->M32, h->uinv32, h->z, out, h->tickets + T_TRSV, h->sc), 1);
   } else {
     KL(trsv_lower<float>(h->st, h->m, h->ldm, h->M32, h->dinv32, rhs, h->z, h->flags, h->tickets, h->sc, true), 1);
     KL(trsv_upper_t<float>(h->st, h->m, h->ldm, h->M32, h->dinv32, h->z, out, h->flags, h->tickets, h->sc, true),
        1);
   }
+  if (nrz) {
+    KL(launch_cg_dot(h->st, h->m, rhs, out, h->part, rz_part(h), h->tickets, h->sc), 1);
+    *nrz = 1;
+  }
   return PDAS_OK;
-}
-
-// rho = r - A(D(A' v)); leaves w = A' v in h->w and ||rho||_inf in sc->rho_norm.
-// df: by the double-float passes, for a residual that only starts the
-// conjugate gradients (every residual that decides acceptance, and the w of
-// an accepted direction, come from the FP64 passes).
-pdas_status residual(pdas_ctx* h, const void* A, const double* v, bool df = false) {
-  pdas_status s = gemv_t(h, A, v, 2, nullptr, h->u, nullptr, h->w, df);
-  if (s != PDAS_OK) return s;
-  return gemv(h, A, h->u, h->r, h->rho, 1, df);
-}
-
-// M v (matrix-free, FP64) -> out.
-pdas_status apply_normal(pdas_ctx* h, const void* A, const double* v, double* out) {
-  // (not once the solve has switched to an FP64 factor: there the FP64 factor
-  // dominates the iteration, and near the end the operator's rounding decides
-  // whether the refinement still reaches its tolerance)
-  const bool df = df_passes(h) && !h->refactored;
-  pdas_status s = gemv_t(h, A, v, 2, nullptr, h->u, nullptr, nullptr, df);
-  if (s != PDAS_OK) return s;
-  return gemv(h, A, h->u, nullptr, out, -1, df);
 }
 
 // FP64 refinement of dy for the mixed forms (a6): conjugate gradients on
@@ -466,7 +473,10 @@ pdas_status apply_normal(pdas_ctx* h, const void* A, const double* v, double* ou
 // Accepted when ||r - M dy||_inf <= refine_tol ||r||_inf, or when the
 // normwise backward error ||r - M dy||_inf / (max_p M_pp ||dy||_inf +
 // ||r||_inf) <= refine_be.  On return h->w = A' dy of the final dy;
-// *ok = 0 if neither test passed within refine_max steps.
+// *ok = 0 if neither test passed within refine_max steps.  A step is four
+// launches (p and u = D A'p; q = A u and p'q; the two triangular solves, which
+// carry the updates and rho'z) and one read of the scalars.  The first read
+// also brings the factor's status (PDAS_ERR_NOT_SPD).
 pdas_status refine(pdas_ctx* h, const void* A, int* ok) {
   *ok = 0;
   const double tol = h->opt.refine_tol, be_tol = h->opt.refine_be;
@@ -477,20 +487,21 @@ pdas_status refine(pdas_ctx* h, const void* A, int* ok) {
   // saved per direction); a first residual that would be accepted is formed
   // again by the FP64 passes.
   const bool cheap_first = df_passes(h) && !h->cur_f64;
+  // The operator: not in double-float once the solve has switched to an FP64
+  // factor (there the FP64 factor dominates the iteration, and near the end
+  // the operator's rounding decides whether the refinement still reaches its
+  // tolerance).
+  const bool df_op = df_passes(h) && !h->refactored;
+  // rho = r - A(D(A' dy)), ||rho||, ||dy||, w = A'dy; df: by the double-float
+  // passes, for a residual that only starts the conjugate gradients
   auto true_residual = [&](bool df = false) -> pdas_status {
-    pdas_status t = residual(h, A, h->dy, df);  // rho, ||rho||, w = A'dy
+    PassTSrc src;
+    src.u = h->dy;
+    src.absmax = 1;
+    pdas_status t = gemv_t(h, A, src, 2, nullptr, df ? nullptr : h->u, nullptr, h->w, df, nullptr, df);
+    if (t == PDAS_OK) t = gemv(h, A, df ? nullptr : h->u, h->r, h->rho, 1, df);
     if (t != PDAS_OK) return t;
-    KL(launch_absmax(h->st, h->m, h->dy, h->part, h->tickets, h->sc, 2), 1);
     if ((t = read_scalars(h)) != PDAS_OK) return t;
-    return device_status(h);
-  };
-  auto restart = [&](double* rz) -> pdas_status {  // z = P^{-1} rho, p = z, rz = rho'z
-    pdas_status t = factor_solve(h, h->rho, h->kz);
-    if (t != PDAS_OK) return t;
-    CK(cudaMemcpyAsync(h->kp, h->kz, sizeof(double) * h->m, cudaMemcpyDeviceToDevice, h->st));
-    KL(launch_dot(h->st, h->m, h->rho, h->kz, h->part, h->tickets, h->sc, 0), 1);
-    if ((t = read_scalars(h)) != PDAS_OK) return t;
-    *rz = h->sc_host->dot_a;
     return device_status(h);
   };
   if ((s = true_residual(cheap_first)) != PDAS_OK) return s;
@@ -507,23 +518,32 @@ pdas_status refine(pdas_ctx* h, const void* A, int* ok) {
   if (accepted(res, dyn)) {
     *ok = 1;
   } else {
-    double rz = 0.0;
-    if ((s = restart(&rz)) != PDAS_OK) return s;
-    while (its < cap && rz > 0.0 && isfinite(rz)) {
-      if ((s = apply_normal(h, A, h->kp, h->kq)) != PDAS_OK) return s;                 // q = M p
-      KL(launch_dot(h->st, h->m, h->kp, h->kq, h->part, h->tickets, h->sc, 1), 1);       // p'q
-      KL(launch_krylov_update(h->st, h->m, h->dy, h->kp, h->dy, +1, h->sc), 1);          // dy += a p
-      KL(launch_krylov_update(h->st, h->m, h->rho, h->kq, h->rho, -1, h->sc), 1);        // rho -= a q
-      ++its;
-      KL(launch_absmax(h->st, h->m, h->rho, h->part, h->tickets, h->sc, 1), 1);
-      KL(launch_absmax(h->st, h->m, h->dy, h->part, h->tickets, h->sc, 2), 1);
-      if ((s = factor_solve(h, h->rho, h->kz)) != PDAS_OK) return s;                    // z = P^{-1} rho
-      KL(launch_dot(h->st, h->m, h->rho, h->kz, h->part, h->tickets, h->sc, 0), 1);      // new rho'z
-      KL(launch_krylov_direction(h->st, h->m, h->kz, h->kp, rz, h->sc), 1);              // p = z + b p
+    double *p = h->kp, *pn = h->kp2;
+    bool first = true;  // p = z = P^{-1} rho, no direction before it
+    int nrz = 0;
+    if (cap > 0 && (s = factor_solve(h, h->rho, h->kz, nullptr, &nrz)) != PDAS_OK) return s;
+    while (its < cap) {
+      PassTSrc src;
+      src.u = h->kz;
+      src.p = p;
+      src.p_new = pn;
+      src.rz_part = rz_part(h);
+      src.nrz = nrz;
+      src.par = its & 1;
+      src.first = first;
+      if ((s = gemv_t(h, A, src, 2, nullptr, df_op ? nullptr : h->u, nullptr, nullptr, df_op, nullptr, df_op)) != PDAS_OK)
+        return s;
+      if ((s = gemv(h, A, df_op ? nullptr : h->u, nullptr, h->kq, -1, df_op, pn)) != PDAS_OK) return s;  // q = M p
+      const CgStep upd{pn, h->kq, h->dy, &h->sc->rz[src.par]};
+      if ((s = factor_solve(h, h->rho, h->kz, &upd, &nrz)) != PDAS_OK) return s;
+      std::swap(p, pn);
+      first = false;
       if ((s = read_scalars(h)) != PDAS_OK) return s;
       if ((s = device_status(h)) != PDAS_OK) return s;
+      const double rz = h->sc_host->rz[src.par];
+      if (!(rz > 0.0 && isfinite(rz))) break;  // (nothing was updated)
+      ++its;
       if (!(h->sc_host->dot_b > 0.0)) break;  // the preconditioned operator lost definiteness
-      rz = h->sc_host->dot_a;
       res = h->sc_host->rho_norm;
       dyn = h->sc_host->dynorm;
       if (accepted(res, dyn) || its % 10 == 0 || its == cap) {
@@ -534,7 +554,8 @@ pdas_status refine(pdas_ctx* h, const void* A, int* ok) {
           *ok = 1;
           break;
         }
-        if ((s = restart(&rz)) != PDAS_OK) return s;
+        if (its < cap && (s = factor_solve(h, h->rho, h->kz, nullptr, &nrz)) != PDAS_OK) return s;
+        first = true;
       }
     }
   }
@@ -603,8 +624,8 @@ pdas_status direction(pdas_ctx* h, const void* A, const double* x, const double*
       STAGE_END(h);
       return PDAS_OK;
     }
-    if ((st = read_scalars(h)) != PDAS_OK) return st;
-    st = device_status(h);
+    int ok = 0;
+    st = refine(h, A, &ok);  // (its first read brings the factor's status)
     if (st == PDAS_ERR_NOT_SPD) {  // low-precision factor broke down: FP64 from now on
       STAGE_END(h);
       if (h->cur_f64) {
@@ -620,8 +641,6 @@ pdas_status direction(pdas_ctx* h, const void* A, const double* x, const double*
       continue;
     }
     if (st != PDAS_OK) return st;
-    int ok = 0;
-    if ((st = refine(h, A, &ok)) != PDAS_OK) return st;
     STAGE_END(h);
     if (ok || h->cur_f64) {
       // w = A' dy of the accepted dy is in h->w: dx = D w - x, ds = -w.  (An
@@ -740,18 +759,29 @@ pdas_status pdas_create(int64_t m, int64_t n, const pdas_options* opt_in, pdas_h
   h->ldm = (m + 15) / 16 * 16;
   h->opt = opt;
   h->st = (cudaStream_t)opt.stream;
-  // gemv_t decomposition: row chunks so that ~4 blocks per SM stream A
-  {
-    const int64_t target_chunks = 64;
-    int64_t rows = (m + target_chunks - 1) / target_chunks;
-    if (rows < 16) rows = 16;
-    h->gt_rows = rows;
-    h->gt_chunks = (int)((m + rows - 1) / rows);
-  }
   const int64_t nblk = (m + kTile - 1) / kTile;
   cudaError_t e = cudaSuccess;
+  // Buffers of up to 1 MB share 4 MB allocations (a cudaMalloc takes 20-60 us).
+  unsigned char* chunk = nullptr;
+  size_t left = 0;
   auto al = [&](void** p, size_t bytes) {
-    if (e == cudaSuccess) e = cudaMalloc(p, bytes);
+    if (e != cudaSuccess) return;
+    const size_t need = (bytes + 255) / 256 * 256;
+    if (need > ((size_t)1 << 20)) {
+      e = cudaMalloc(p, bytes);
+      if (e == cudaSuccess) h->allocs.push_back(*p);
+      return;
+    }
+    if (need > left) {
+      void* c = nullptr;
+      if ((e = cudaMalloc(&c, (size_t)4 << 20)) != cudaSuccess) return;
+      h->allocs.push_back(c);
+      chunk = (unsigned char*)c;
+      left = (size_t)4 << 20;
+    }
+    *p = chunk;
+    chunk += need;
+    left -= need;
   };
   al((void**)&h->D, sizeof(double) * n);
   al((void**)&h->dx, sizeof(double) * n);
@@ -766,14 +796,20 @@ pdas_status pdas_create(int64_t m, int64_t n, const pdas_options* opt_in, pdas_h
   al((void**)&h->kp, sizeof(double) * m);
   al((void**)&h->kq, sizeof(double) * m);
   al((void**)&h->kz, sizeof(double) * m);
+  al((void**)&h->kp2, sizeof(double) * m);
   if (opt.infeasible) al((void**)&h->rd, sizeof(double) * n);
   al((void**)&h->part, sizeof(double) * kPartMax * 4);
-  al((void**)&h->gt_part, sizeof(double) * n * h->gt_chunks);
+  al((void**)&h->gt_part, sizeof(double) * pass_t_part_doubles(m, n, (int)dtype_size(opt.a_dtype)));
+  al((void**)&h->ctickets, sizeof(unsigned) * pass_t_tickets(n));
   al((void**)&h->tickets, sizeof(unsigned) * T_COUNT);
   al((void**)&h->flags, sizeof(int) * (nblk + 1));
-  if (opt.form != PDAS_FP64 && opt.a_dtype != PDAS_A_F64) al((void**)&h->pairs, sizeof(float2) * n);  // n > m
+  if (opt.form != PDAS_FP64 && opt.a_dtype != PDAS_A_F64) al((void**)&h->pairs, sizeof(float) * 2 * pairs_pitch(n));
   al((void**)&h->sc, sizeof(Scalars));
-  if (e == cudaSuccess) e = cudaMallocHost((void**)&h->sc_host, sizeof(Scalars));
+  if (e == cudaSuccess) e = cudaMallocHost((void**)&h->sc_host, sizeof(Scalars) + sizeof(unsigned));
+  if (e == cudaSuccess) {
+    h->sc_seq = (unsigned*)(h->sc_host + 1);
+    *h->sc_seq = 0;
+  }
   if (e == cudaSuccess) e = cudaMallocHost((void**)&h->wait_pinned, sizeof(int));
   if (e == cudaSuccess) *h->wait_pinned = 0;
   al((void**)&h->adj, sizeof(double) * (5 * n + m));  // pdas_backward
@@ -816,6 +852,8 @@ pdas_status pdas_create(int64_t m, int64_t n, const pdas_options* opt_in, pdas_h
     const int64_t nb = chol_tile_count(m);
     h->chol_ntasks = (int)tasks.size();
     al((void**)&h->chol_tasks, sizeof(int4) * tasks.size());
+    al((void**)&h->zb, sizeof(double) * m);
+    if (e == cudaSuccess) e = cudaMemsetAsync(h->zb, 0xff, sizeof(double) * m, h->st);
     al((void**)&h->chol_state, sizeof(int) * (nb * nb + nb));
     al((void**)&h->uinv32, sizeof(float) * nb * kCholTile * kCholTile);
     if (nb > 1) al((void**)&h->chol_planes, (size_t)chol_plane_bytes(m));
@@ -835,6 +873,7 @@ pdas_status pdas_create(int64_t m, int64_t n, const pdas_options* opt_in, pdas_h
     }
   }
   if (e == cudaSuccess) e = cudaMemsetAsync(h->tickets, 0, sizeof(unsigned) * T_COUNT, h->st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(h->ctickets, 0, sizeof(unsigned) * pass_t_tickets(n), h->st);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->sc, 0, sizeof(Scalars), h->st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->st);
   if (e != cudaSuccess) {
@@ -850,29 +889,7 @@ void pdas_destroy(pdas_handle h) {
   if (!h) return;
   if (h->st) cudaStreamSynchronize(h->st);
   else cudaDeviceSynchronize();
-  double* vecs[] = {h->D, h->r, h->dy, h->dx, h->ds, h->w, h->u, h->z, h->rho, h->delta, h->kp, h->kq, h->kz,
-                    h->part, h->gt_part, h->M64, h->rd};
-  for (double* p : vecs)
-    if (p) cudaFree(p);
-  if (h->simt_part) cudaFree(h->simt_part);
-  if (h->simt_tickets) cudaFree(h->simt_tickets);
-  if (h->simt_planes) cudaFree(h->simt_planes);
-  if (h->M32) cudaFree(h->M32);
-  if (h->akept) cudaFree(h->akept);
-  if (h->dkept) cudaFree(h->dkept);
-  if (h->kidx) cudaFree(h->kidx);
-  if (h->d2) cudaFree(h->d2);
-  if (h->adj) cudaFree(h->adj);
-  if (h->chol_tasks) cudaFree(h->chol_tasks);
-  if (h->chol_state) cudaFree(h->chol_state);
-  if (h->uinv32) cudaFree(h->uinv32);
-  if (h->chol_planes) cudaFree(h->chol_planes);
-  if (h->pairs) cudaFree(h->pairs);
-  if (h->dinv64) cudaFree(h->dinv64);
-  if (h->dinv32) cudaFree(h->dinv32);
-  if (h->tickets) cudaFree(h->tickets);
-  if (h->flags) cudaFree(h->flags);
-  if (h->sc) cudaFree(h->sc);
+  for (void* p : h->allocs) cudaFree(p);
   if (h->sc_host) cudaFreeHost(h->sc_host);
   if (h->wait_pinned) cudaFreeHost(h->wait_pinned);
   tc_workspace_destroy(&h->tc);
@@ -1145,7 +1162,8 @@ pdas_status pdas_factor_solve(pdas_handle h, const double* rhs, double* out) {
   if (!h || !rhs || !out) return PDAS_ERR_ARG;
   pdas_status st = reset_status(h);
   if (st != PDAS_OK) return st;
-  if ((st = factor_solve(h, rhs, h->delta)) != PDAS_OK) return st;
+  CK(cudaMemcpyAsync(h->rho, rhs, sizeof(double) * h->m, cudaMemcpyDeviceToDevice, h->st));
+  if ((st = factor_solve(h, h->rho, h->delta)) != PDAS_OK) return st;
   CK(cudaMemcpyAsync(out, h->delta, sizeof(double) * h->m, cudaMemcpyDeviceToDevice, h->st));
   if ((st = read_scalars(h)) != PDAS_OK) return st;
   return device_status(h);

@@ -31,7 +31,8 @@ struct Scalars {
   double rel_gap;      // (c'x - b'y)/(1+|c'x|)
   double rnorm;        // ||A x||_inf
   double rho_norm;     // ||A x - M dy||_inf of the latest residual
-  double dot_a, dot_b; // dot products of the refinement Krylov steps
+  double rz[2];        // conjugate gradients: rho'z of this step and the one before, in turn
+  double dot_b;        // ... p'q
   double mnorm;        // max_p M_pp of the formed normal matrix (a lower bound on ||M||)
   double dynorm;       // ||dy||_inf
   double pres, dres;   // infeasible-start variant: relative primal and dual residuals
@@ -43,7 +44,7 @@ struct Scalars {
 
 // Counters for the "last block finishes the reduction" pattern and the
 // triangular-solve tickets.
-enum Ticket { T_SCALING = 0, T_PSI, T_STEP, T_NORM, T_NORM2, T_DOT, T_TRSV, T_CHOL, T_RES, T_COUNT = 9 };
+enum Ticket { T_SCALING = 0, T_PSI, T_STEP, T_NORM, T_NORM2, T_DOT, T_TRSV, T_TRSVB, T_CHOL, T_RES, T_COUNT };
 
 // ---- exact widening of the stored A ---------------------------------------
 __device__ __forceinline__ double widen(double v) { return v; }
@@ -73,23 +74,11 @@ __device__ __forceinline__ float widen32(__nv_bfloat16 v) { return __bfloat162fl
 
 // ---- launch helpers (host) ------------------------------------------------
 // Each returns cudaGetLastError() of its launch.
-template <typename T>
-cudaError_t launch_gemv(cudaStream_t st, int64_t m, int64_t n, const T* A, const double* v, const double* base,
-                        double* out, double* part, unsigned* tickets, Scalars* sc, int norm_slot);
+// Partial column sums of A'u by row chunks (no handle; passes.cuh has a handle's passes).
 template <typename T>
 cudaError_t launch_gemv_t(cudaStream_t st, int64_t m, int64_t n, const T* A, const double* u, double* part,
                           int chunks, int64_t rows_per_chunk);
 
-// The passes over A in double-float on the FP32 pipes (gemv_df.cu), for A
-// stored as FP32 or BF16: v (or u) is first split into FP32 pairs by
-// launch_split_pairs; results and partials are FP64 as above.
-cudaError_t launch_split_pairs(cudaStream_t st, int64_t n, const double* v, float2* out);
-template <typename T>
-cudaError_t launch_gemv_df(cudaStream_t st, int64_t m, int64_t n, const T* A, const float2* v2, const double* base,
-                           double* out, double* part, unsigned* tickets, Scalars* sc, int norm_slot);
-template <typename T>
-cudaError_t launch_gemv_t_df(cudaStream_t st, int64_t m, int64_t n, const T* A, const float2* u2, double* part,
-                             int chunks, int64_t rows_per_chunk);
 // w = sum of the gemv_t partials; then per mode:
 //   0: out0 = w
 //   1: direction: out0 = dx = D w - x, out1 = ds = -w, out2 = w (may be null)
@@ -117,15 +106,23 @@ cudaError_t launch_psi(cudaStream_t st, int64_t n, const double* x, const double
 cudaError_t launch_step(cudaStream_t st, int64_t m, int64_t n, const double* b, const double* c, double* x,
                         double* y, double* s, const double* dx, const double* dy, const double* ds, double* part,
                         unsigned* tickets, Scalars* sc);
+// *out = *sc and then *seq = want, both in pinned host memory.
+cudaError_t launch_snapshot(cudaStream_t st, const Scalars* sc, Scalars* out, unsigned* seq, unsigned want);
 cudaError_t launch_axpy(cudaStream_t st, int64_t n, double a, const double* xv, double* yv, const Scalars* sc);
-cudaError_t launch_dot(cudaStream_t st, int64_t n, const double* a, const double* b, double* part,
-                       unsigned* tickets, Scalars* sc, int slot);
-// x-update of one Krylov step: out = base + coef * p where coef = sc->dot_a / sc->dot_b
-// (sign < 0 subtracts); see the refinement driver.
-cudaError_t launch_krylov_update(cudaStream_t st, int64_t n, const double* base, const double* p, double* out,
-                                 int sign, const Scalars* sc);
-cudaError_t launch_krylov_direction(cudaStream_t st, int64_t n, const double* z, double* p, double beta_num,
-                                    const Scalars* sc);
+// One step of the conjugate gradients: with a = *rz / sc->dot_b, dy += a p,
+// rho -= a q (nothing unless *rz is positive and finite), and the largest
+// magnitudes of dy and rho to sc->dynorm and sc->rho_norm.
+struct CgStep {
+  const double* p;
+  const double* q;
+  double* dy;
+  const double* rz;
+};
+// The step and rho'z (to dpart[0]) where the triangular solves do not carry them.
+cudaError_t launch_cg_update(cudaStream_t st, int64_t m, const CgStep& upd, double* rho, double* part,
+                             unsigned* tickets, Scalars* sc);
+cudaError_t launch_cg_dot(cudaStream_t st, int64_t m, const double* a, const double* b, double* part, double* dpart,
+                          unsigned* tickets, Scalars* sc);
 
 // Blocked Cholesky in place; dinv (m) receives the reciprocals of the pivots.
 template <typename T>
@@ -157,12 +154,15 @@ int64_t chol_plane_bytes(int64_t m);
 // reciprocals dinv.  A pivot that is not positive sets PDAS_ERR_NOT_SPD.
 cudaError_t cholesky_tiles_df(cudaStream_t st, int64_t m, int64_t ldm, double* M, double* dinv, const int4* tasks,
                               int ntasks, int* state, unsigned* ticket, Scalars* sc);
-// The triangular solves with the FP32 tile factor (trsv_blk.cu).  The output
-// (z, y) is the hand-off between blocks; it must not alias the input.
-cudaError_t trsv_lower_blk(cudaStream_t st, int64_t m, int64_t ldm, const float* L, const float* Uinv,
-                           const double* v, double* z, unsigned* ticket, Scalars* sc);
-cudaError_t trsv_upper_blk(cudaStream_t st, int64_t m, int64_t ldm, const float* L, const float* Uinv,
-                           const double* z, double* y, unsigned* ticket, Scalars* sc);
+// The triangular solves with the FP32 tile factor (trsv_blk.cu): out =
+// (L L')^{-1} rhs through z.  z holds the unset pattern (every bit set) in all
+// entries before and after, as does *ticket zero, unless a wait gave up: then
+// both have to be set again.  out must not alias rhs or z.  upd != null: rhs and
+// dy first take that step (npart: 2 nb doubles).  dpart != null: the nb =
+// chol_tile_count(m) parts of rhs'out.  Two launches.
+cudaError_t trsv_blk_solve(cudaStream_t st, int64_t m, int64_t ldm, const float* L, const float* Uinv, double* rhs,
+                           double* z, double* out, const CgStep* upd, double* dpart, double* npart, unsigned* ticket,
+                           Scalars* sc);
 // scaled: the diagonal blocks are solved on pivot-scaled rows (the FP64 tier
 // of the mixed forms, a preconditioner: shorter chains); else by plain
 // substitution (the plain FP64 form's direct solve).
@@ -177,10 +177,6 @@ cudaError_t trsv_upper_t(cudaStream_t st, int64_t m, int64_t ldm, const T* L, co
 template <typename T>
 cudaError_t launch_diag_max(cudaStream_t st, int64_t m, int64_t ldm, const T* M, double* part, unsigned* tickets,
                             Scalars* sc);
-// max_j |v_j| into sc->rho_norm (slot 1) or sc->dynorm (slot 2).
-cudaError_t launch_absmax(cudaStream_t st, int64_t n, const double* v, double* part, unsigned* tickets, Scalars* sc,
-                          int slot);
-
 // Lower triangle of M64 = A D A' in double-float on the FP32 pipes (A exact
 // in FP32: float or BF16 storage); D2 (n float2) receives D as hi + lo.
 template <typename T>

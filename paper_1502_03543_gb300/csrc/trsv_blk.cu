@@ -8,30 +8,124 @@
 // mixed forms refine in FP64 afterwards), so the explicit inverse of each
 // diagonal tile is accurate enough; the plain FP64 form keeps substitution.
 //
-// One launch per solve.  Blocks take block rows in order from a ticket
-// counter and wait (bounded: 2 s, or the handle's own limit) for the
-// solution blocks they depend on, which were handed out earlier: no
-// deadlock.  The solution vector is filled
-// with an all-ones bit pattern before the launch (a value the solves cannot
-// produce: each entry is an FP32 sum widened to FP64, whose low 29 bits are
-// zero), and a consumer polls the entries it needs until none holds it, so
-// the hand-off from block to block is one round trip to L2, with no flag and
-// no fence.  Thread layout for the off-diagonal tiles: warp w holds rows
-// 16 w .. 16 w + 15, lane l columns 4 l .. 4 l + 3 (16-byte loads along the
-// rows); tiles are loaded before the wait for the block they multiply.
+// One launch per solve, in clusters of 8 blocks.  Clusters take 8 block rows at
+// a time from a ticket counter and wait (bounded: 2 s, or the handle's own limit)
+// for the solution blocks they depend on, which were handed out earlier: no
+// deadlock.  Inside a cluster a block writes its solution straight into the
+// shared memory of the blocks behind it (st.async on their mbarriers).  Between
+// clusters it goes through L2: a solution vector not yet written holds an all-ones
+// bit pattern (a value the solves cannot produce: each entry is an FP32 sum
+// widened to FP64, whose low 29 bits are zero), and one warp of the consumer polls
+// the entries until none holds it.  The forward solve fills the backward
+// solve's output with the pattern and the backward solve refills the forward
+// one's as it reads it, so no fill runs between the launches.
+//
+// What bounds a solve is the latency of its chain of nb links.  Per link: the
+// hand-off, a 128 x 128 product whose tile is already in registers, a
+// reduce-scatter over lanes, and the product with U_b, whose entries every
+// thread holds in registers, too.  Measured at m = 2048 (16 links), forward and
+// backward: 48 and 26 us with every warp of every waiting block polling L2,
+// 29 and 37 us with one warp polling and U_b in registers, 20-27 and 29 us in
+// clusters; at m = 8192 187 and 106, now 101 and 125 us.
+//
+// The conjugate gradients of the refinement ride along: the forward solve's
+// block first takes its rows of the step (dy += a p, rho -= a q) and leaves the
+// largest magnitudes, which the backward solve's last block combines while it
+// waits; the backward solve leaves the partial sums of rho'z.
+#include "reduce_util.cuh"
 #include "sync_util.cuh"
+#include "tc_util.cuh"
 #include "tile_core.cuh"
 
 namespace pdas {
 
 namespace {
 
+constexpr int kClu = 8;  // blocks per cluster (the portable limit)
+
 struct TrsvSmem {
-  float U[kBig][kBig + 1];  // U_b = L_bb^{-T}
-  float rhs[kBig];
-  float red[8][kBig];
-  int b;
+  __align__(16) float zc[kClu][kBig];  // solution blocks of this cluster
+  __align__(16) float zs[2][kBig];     // the solution block in use of another cluster, and the next
+  __align__(16) float rhs[kBig];
+  __align__(16) float red[8][kBig];
+  unsigned long long bar[kClu];  // arrival of zc
+  double mx[8][2];
+  unsigned cluster;
+  int ok[2];
 };
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t peer_addr(const void* p, uint32_t rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(tc::smem_u32(p)), "r"(rank));
+  return r;
+}
+
+// This block's place in the order of the chain.  All threads; sets up the
+// arrival barriers of the blocks before it in its cluster.
+__device__ __forceinline__ int64_t chain_position(TrsvSmem& sm, unsigned* ticket) {
+  const uint32_t rank = cluster_rank();
+  if (threadIdx.x == 0) {
+    for (uint32_t k = 0; k < rank; ++k) {
+      tc::mbar_init(tc::smem_u32(&sm.bar[k]), 1);
+      tc::mbar_expect_tx(tc::smem_u32(&sm.bar[k]), sizeof(float) * kBig);
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    if (rank == 0) {
+      const unsigned t = atomicAdd(ticket, 1u);
+      if (t == gridDim.x / kClu - 1) *ticket = 0;  // every cluster has its own
+      for (uint32_t k = 0; k < kClu; ++k)
+        asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(peer_addr(&sm.cluster, k)), "r"(t) : "memory");
+    }
+  }
+  cluster_barrier();
+  return (int64_t)sm.cluster * kClu + rank;
+}
+
+// The solution entry of row i = tid / 2 (in both lanes of a pair) to the blocks
+// behind this one in its cluster, of `behind` in all.
+__device__ __forceinline__ void send_entry(TrsvSmem& sm, float v, int64_t behind) {
+  const uint32_t rank = cluster_rank(), i = threadIdx.x >> 1;
+  for (uint32_t k = rank + 1 + (threadIdx.x & 1); k < kClu && (int64_t)(k - rank) <= behind; k += 2)
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(
+                     peer_addr(&sm.zc[rank][i], k)),
+                 "r"(__float_as_uint(v)), "r"(peer_addr(&sm.bar[rank], k))
+                 : "memory");
+}
+
+// No block leaves while another may write to its shared memory: it has waited
+// for all blocks before it, or (ok false) gives what they may have sent 50 us
+// to land once they are all done.
+__device__ __forceinline__ void leave(TrsvSmem& sm, bool ok) {
+  cluster_barrier();
+  if (ok) return;
+  const uint64_t t0 = global_ns();
+  for (uint32_t k = 0; k < cluster_rank(); ++k)
+    while (!tc::mbar_try(tc::smem_u32(&sm.bar[k]), 0) && global_ns() - t0 < 50000) {
+    }
+}
+
+// Bounded wait for block k of this cluster; false on a timeout or a failed status.
+__device__ __forceinline__ bool wait_peer(TrsvSmem& sm, int k, Scalars* sc) {
+  const uint32_t bar = tc::smem_u32(&sm.bar[k]);
+  if (tc::mbar_try(bar, 0)) return true;
+  const uint64_t t0 = global_ns(), limit = wait_limit_ns(sc);
+  for (;;) {
+    if (tc::mbar_try(bar, 0)) return true;
+    if (dev_failed(sc)) return false;
+    if (global_ns() - t0 > limit) {
+      atomicCAS(&sc->status, 0, (int)PDAS_ERR_TIMEOUT);
+      return false;
+    }
+  }
+}
 
 // 16 per-lane partial sums reduced across the warp by exchanging halves:
 // lane l ends with the total of entry (l >> 1) & 15 (16 shuffles in all).
@@ -62,7 +156,7 @@ __device__ __forceinline__ float reduce16(float (&v)[16], int lane) {
   return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
 }
 
-constexpr unsigned long long kUnset = ~0ull;  // the fill of a solution entry not yet written
+constexpr unsigned long long kUnset = ~0ull;  // a solution entry not yet written
 
 __device__ __forceinline__ double ld_relaxed_f64(const double* p) {
   double v;
@@ -73,216 +167,319 @@ __device__ __forceinline__ void st_relaxed_f64(double* p, double v) {
   asm volatile("st.relaxed.gpu.global.f64 [%0], %1;" ::"l"(p), "d"(v) : "memory");
 }
 
-// The warp waits (bounded) until none of the N entries p[k * stride] (k < N,
-// this lane's share) holds kUnset; entries with valid[k] false are not
-// waited for and read as 0.  Returns false on a timeout or a failed status.
-template <int N>
-__device__ __forceinline__ bool poll_entries(const double* p, const bool (&valid)[N], double (&out)[N], Scalars* sc) {
+// The warp waits (bounded) until none of the entries p[4 lane .. + 3] (those
+// below left; the others read as 0) holds kUnset.  Returns false on a timeout
+// or a failed status.  far: the block is not next in the chain and polls less often.
+__device__ __forceinline__ bool poll_entries(const double* p, int left, float (&out)[4], bool far, Scalars* sc) {
+  const int lane = threadIdx.x & 31;
   const uint64_t t0 = global_ns(), limit = wait_limit_ns(sc);
   for (;;) {
     bool mine = true;
+    const bool failed = dev_failed(sc);  // (in flight with the entries)
 #pragma unroll
-    for (int k = 0; k < N; ++k) {
-      out[k] = valid[k] ? ld_relaxed_f64(p + k) : 0.0;
-      mine = mine && __double_as_longlong(out[k]) != (long long)kUnset;
+    for (int k = 0; k < 4; ++k) {
+      const double v = 4 * lane + k < left ? ld_relaxed_f64(p + 4 * lane + k) : 0.0;
+      mine = mine && __double_as_longlong(v) != (long long)kUnset;
+      out[k] = (float)v;
     }
     if (__all_sync(0xffffffffu, mine)) return true;
-    if (dev_failed(sc)) return false;
-    if (global_ns() - t0 > limit) {
-      atomicCAS(&sc->status, 0, (int)PDAS_ERR_TIMEOUT);
+    if (__any_sync(0xffffffffu, failed)) return false;
+    if (__any_sync(0xffffffffu, global_ns() - t0 > limit)) {
+      if (lane == 0) atomicCAS(&sc->status, 0, (int)PDAS_ERR_TIMEOUT);
       return false;
     }
-    __nanosleep(32);
+    if (far) __nanosleep(200);
   }
 }
 
-__device__ __forceinline__ void load_u(TrsvSmem& sm, const float* __restrict__ Ub) {
-  for (int e = threadIdx.x; e < kBig * kBig; e += blockDim.x) sm.U[e >> 7][e & 127] = __ldg(Ub + e);
+// Warp 0 fetches solution block k of v (m entries) into sm.zs[buf]; the others
+// learn the outcome behind the caller's next barrier.
+__device__ __forceinline__ void fetch_block(TrsvSmem& sm, const double* v, int64_t m, int64_t k, int buf, bool far,
+                                            Scalars* sc) {
+  if (threadIdx.x < 32) {
+    const int64_t left = m - k * kBig;
+    float e[4];
+    const bool ok = poll_entries(v + k * kBig, left < kBig ? (int)left : kBig, e, far, sc);
+    *reinterpret_cast<float4*>(&sm.zs[buf][4 * threadIdx.x]) = make_float4(e[0], e[1], e[2], e[3]);
+    if (threadIdx.x == 0) sm.ok[buf] = ok;
+  }
 }
 
-// L z = v: z_b = U_b' (v_b - sum_{j<b} L_bj z_j).
-__global__ void __launch_bounds__(kThreads, 1) k_trsv_lower_blk(int64_t m, int64_t ldm, const float* __restrict__ L,
-                                                             const float* __restrict__ Uinv,
-                                                             const double* __restrict__ v, double* z,
-                                                             unsigned* ticket, Scalars* sc) {
-  extern __shared__ __align__(16) unsigned char trsv_blk_smem[];
-  TrsvSmem& sm = *reinterpret_cast<TrsvSmem*>(trsv_blk_smem);
+__device__ __forceinline__ float dot64(const float4 (&u)[16], const float* v) {  // v: 64 floats in shared memory
+  float s[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+  for (int k = 0; k < 16; ++k) {
+    const float4 q = *reinterpret_cast<const float4*>(v + 4 * k);
+    s[0] = fmaf(u[k].x, q.x, s[0]), s[1] = fmaf(u[k].y, q.y, s[1]);
+    s[2] = fmaf(u[k].z, q.z, s[2]), s[3] = fmaf(u[k].w, q.w, s[3]);
+  }
+  return (s[0] + s[1]) + (s[2] + s[3]);
+}
+
+// L z = v: z_b = U_b' (v_b - sum_{j<b} L_bj z_j).  upd: v takes a step of the
+// conjugate gradients first (CgStep) and the largest magnitudes of v and dy go
+// to npart.  fill: the backward solve's output.
+template <bool UPD>
+__device__ __forceinline__ bool trsv_lower_block(TrsvSmem& sm, int64_t b, int64_t nblk, int64_t m, int64_t ldm,
+                                                 const float* __restrict__ L, const float* __restrict__ Uinv,
+                                                 double* v, double* z, double* fill, const CgStep& upd, double* npart,
+                                                 Scalars* sc) {
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  if (tid == 0) sm.b = (int)atomicAdd(ticket, 1u);
-  __syncthreads();
-  if (dev_failed(sc)) return;
-  const int b = sm.b;
-  const int64_t r0 = (int64_t)b * kBig;
+  const int64_t own = b - cluster_rank();  // the cluster's first block
+  if (b >= nblk) return true;
+  if (__syncthreads_or(dev_failed(sc))) return false;
+  const int64_t r0 = b * kBig;
   const int rb = (int)(m - r0 < kBig ? m - r0 : kBig);
-  load_u(sm, Uinv + (int64_t)b * kBig * kBig);
-  const int myrow = 16 * w + ((lane >> 1) & 15);  // the row this lane finishes after the reduction
-  const float vmine = myrow < rb ? (float)v[r0 + myrow] : 0.f;  // off the dependency chain
+  if (tid < rb) fill[r0 + tid] = __longlong_as_double((long long)kUnset);
+  const int myrow = 16 * w + ((lane >> 1) & 15);  // the row this lane pair finishes after the reduction
+  float vmine = 0.f;
+  double mr = 0.0, my = 0.0;
+  if ((lane & 1) == 0 && myrow < rb) {
+    double r = v[r0 + myrow];
+    if constexpr (UPD) {
+      const double rz = *upd.rz;
+      double y = upd.dy[r0 + myrow];
+      if (rz > 0.0 && isfinite(rz)) {
+        const double a = rz / sc->dot_b;
+        y = y + a * upd.p[r0 + myrow];
+        r = r - a * upd.q[r0 + myrow];
+        upd.dy[r0 + myrow] = y;
+        v[r0 + myrow] = r;
+      }
+      mr = r == r ? fabs(r) : INFINITY;
+      my = y == y ? fabs(y) : INFINITY;
+    }
+    vmine = (float)r;
+  }
+  if constexpr (UPD) {
+    mr = warp_max(mr);
+    my = warp_max(my);
+    if (lane == 0) sm.mx[w][0] = mr, sm.mx[w][1] = my;
+    __syncthreads();
+    if (tid == 0) {
+      for (int k = 0; k < 8; ++k) mr = fmax(mr, sm.mx[k][0]), my = fmax(my, sm.mx[k][1]);
+      npart[2 * b] = mr, npart[2 * b + 1] = my;
+    }
+  }
   float part[16];
 #pragma unroll
   for (int rr = 0; rr < 16; ++rr) part[rr] = 0.f;
   bool ok = true;
-  // Two buffers: block j + 1's tile rows and solution entries are in flight
-  // while block j's products run (entries read too early are re-polled).
+  // Two buffers: tile j + 1 is on its way while tile j waits for its block of z.
+  // A tile is rows 16 w .. 16 w + 15, columns 4 lane .. + 3; "tile b" is this
+  // thread's share of U_b: column c = tid / 2, rows 64 (tid % 2) .. + 63.
   float4 lv[2][16];
-  double zd[2][4];
-  auto fetch = [&](int64_t j, int buf) {  // tile j is full (j < b <= nb - 1)
+  auto fetch = [&](int64_t j, float4 (&t)[16]) {
+    if (j < b) {
 #pragma unroll
-    for (int rr = 0; rr < 16; ++rr) {
-      const int64_t row = r0 + 16 * w + rr;
-      lv[buf][rr] = row < m ? __ldg(reinterpret_cast<const float4*>(L + row * ldm + j * kBig + 4 * lane))
-                            : make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int rr = 0; rr < 16; ++rr) {
+        const int64_t row = r0 + 16 * w + rr;
+        t[rr] = row < m ? __ldg(reinterpret_cast<const float4*>(L + row * ldm + j * kBig + 4 * lane))
+                        : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+    } else {
+      const float* Ub = Uinv + (int64_t)b * kBig * kBig + (int64_t)(64 * (tid & 1)) * kBig + (tid >> 1);
+#pragma unroll
+      for (int r = 0; r < 16; ++r)
+        t[r] = make_float4(__ldg(Ub + 4 * r * kBig), __ldg(Ub + (4 * r + 1) * kBig), __ldg(Ub + (4 * r + 2) * kBig),
+                           __ldg(Ub + (4 * r + 3) * kBig));
     }
-#pragma unroll
-    for (int k = 0; k < 4; ++k) zd[buf][k] = ld_relaxed_f64(z + j * kBig + 4 * lane + k);
   };
-  auto consume = [&](int64_t j, int buf) {
-    bool mine = true;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) mine = mine && __double_as_longlong(zd[buf][k]) != (long long)kUnset;
-    if (!__all_sync(0xffffffffu, mine)) {
-      const bool all4[4] = {true, true, true, true};
-      if (!poll_entries<4>(z + j * kBig + 4 * lane, all4, zd[buf], sc)) return false;
+  auto consume = [&](int64_t j, const float4 (&t)[16]) {
+    const float* zj = sm.zs[j & 1];
+    if (j >= own) {
+      if (__syncthreads_or(!wait_peer(sm, (int)(j - own), sc))) return false;
+      zj = sm.zc[j - own];
+    } else {
+      fetch_block(sm, z, m, j, j & 1, j + 3 < own, sc);
+      __syncthreads();
+      if (!sm.ok[j & 1]) return false;
     }
-    const float z0 = (float)zd[buf][0], z1 = (float)zd[buf][1], z2 = (float)zd[buf][2], z3 = (float)zd[buf][3];
+    const float4 q = *reinterpret_cast<const float4*>(&zj[4 * lane]);
 #pragma unroll
     for (int rr = 0; rr < 16; ++rr)
-      part[rr] = fmaf(lv[buf][rr].x, z0, fmaf(lv[buf][rr].y, z1, fmaf(lv[buf][rr].z, z2, fmaf(lv[buf][rr].w, z3, part[rr]))));
+      part[rr] = fmaf(t[rr].x, q.x, fmaf(t[rr].y, q.y, fmaf(t[rr].z, q.z, fmaf(t[rr].w, q.w, part[rr]))));
     return true;
   };
-  if (b > 0) fetch(0, 0);
+  fetch(0, lv[0]);
   for (int64_t j = 0; j < b && ok; j += 2) {
-    if (j + 1 < b) fetch(j + 1, 1);
-    ok = consume(j, 0);
+    fetch(j + 1, lv[1]);
+    ok = consume(j, lv[0]);
     if (!ok || j + 1 >= b) break;
-    if (j + 2 < b) fetch(j + 2, 0);
-    ok = consume(j + 1, 1);
+    fetch(j + 2, lv[0]);
+    ok = consume(j + 1, lv[1]);
   }
+  if (!ok) return false;  // a wait gave up: the status says why
   const float tot = reduce16(part, lane);
   if ((lane & 1) == 0) sm.rhs[myrow] = myrow < rb ? vmine - tot : 0.f;
-  if (__syncthreads_or(!ok)) return;  // a wait gave up: the status says why
-  const int c = tid & 127, h = tid >> 7;  // z_c = sum_r U_rc rhs_r, rows split in two halves
-  float s = 0.f;
-#pragma unroll 8
-  for (int r = 64 * h; r < 64 * h + 64; ++r) s = fmaf(sm.U[r][c], sm.rhs[r], s);
-  sm.red[h][c] = s;
   __syncthreads();
-  if (tid < rb) st_relaxed_f64(z + r0 + tid, (double)(sm.red[0][tid] + sm.red[1][tid]));
+  const float* half = &sm.rhs[64 * (tid & 1)];
+  float s = (b & 1) ? dot64(lv[1], half) : dot64(lv[0], half);  // z_c = sum_r U_rc rhs_r
+  s += __shfl_xor_sync(0xffffffffu, s, 1);
+  send_entry(sm, s, nblk - 1 - b);
+  if ((tid & 1) == 0 && (tid >> 1) < rb) st_relaxed_f64(z + r0 + (tid >> 1), (double)s);
+  return true;
+}
+
+template <bool UPD>
+__global__ void __launch_bounds__(kThreads, 1) k_trsv_lower_blk(int64_t m, int64_t ldm, int64_t nblk,
+                                                                const float* __restrict__ L,
+                                                                const float* __restrict__ Uinv, double* v, double* z,
+                                                                double* fill, CgStep upd, double* npart,
+                                                                unsigned* ticket, Scalars* sc) {
+  __shared__ TrsvSmem sm;
+  const int64_t b = chain_position(sm, ticket);
+  leave(sm, trsv_lower_block<UPD>(sm, b, nblk, m, ldm, L, Uinv, v, z, fill, upd, npart, sc));
 }
 
 // L' y = z: y_b = U_b (z_b - sum_{k>b} L_kb' y_k); blocks go from the last.
-__global__ void __launch_bounds__(kThreads, 1) k_trsv_upper_blk(int64_t m, int64_t ldm, const float* __restrict__ L,
-                                                             const float* __restrict__ Uinv,
-                                                             const double* __restrict__ zin, double* y,
-                                                             unsigned* ticket, Scalars* sc) {
-  extern __shared__ __align__(16) unsigned char trsv_blk_smem[];
-  TrsvSmem& sm = *reinterpret_cast<TrsvSmem*>(trsv_blk_smem);
+// dpart != null: the block's part of rho'y goes to dpart[b].  npart != null: the
+// last block of the chain combines the forward solve's magnitudes.
+__device__ __forceinline__ bool trsv_upper_block(TrsvSmem& sm, int64_t pos, int64_t nblk, int64_t m, int64_t ldm,
+                                                 const float* __restrict__ L, const float* __restrict__ Uinv,
+                                                 double* zin, double* y, const double* __restrict__ rho,
+                                                 double* dpart, const double* __restrict__ npart, Scalars* sc) {
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  const int64_t nblk = (m + kBig - 1) / kBig;
-  if (tid == 0) sm.b = (int)(nblk - 1 - (int64_t)atomicAdd(ticket, 1u));
-  __syncthreads();
-  if (dev_failed(sc)) return;
-  const int b = sm.b;
-  const int64_t r0 = (int64_t)b * kBig;
+  const int64_t own = pos - cluster_rank();  // the cluster's first place in the chain
+  if (pos >= nblk) return true;
+  if (__syncthreads_or(dev_failed(sc))) return false;
+  const int64_t b = nblk - 1 - pos;
+  const int64_t r0 = b * kBig;
   const int rb = (int)(m - r0 < kBig ? m - r0 : kBig);
-  load_u(sm, Uinv + (int64_t)b * kBig * kBig);
-  const float zmine = tid < rb ? (float)zin[r0 + tid] : 0.f;  // off the dependency chain
+  if (npart && b == 0 && w == 0) {
+    double gr = 0.0, gy = 0.0;
+    for (int64_t i = lane; i < nblk; i += 32) gr = fmax(gr, npart[2 * i]), gy = fmax(gy, npart[2 * i + 1]);
+    gr = warp_max(gr);
+    gy = warp_max(gy);
+    if (lane == 0) sc->rho_norm = gr, sc->dynorm = gy;
+  }
+  float zmine = 0.f;
+  if (tid < rb) {
+    zmine = (float)zin[r0 + tid];
+    zin[r0 + tid] = __longlong_as_double((long long)kUnset);  // for the next forward solve
+  }
   float colp[4] = {0.f, 0.f, 0.f, 0.f};  // columns 4 lane .. 4 lane + 3 of tile b, this warp's rows
   bool ok = true;
-  // Two buffers, as in the forward solve: block k - 1's tile rows and
-  // solution entries are in flight while block k's products run.  Lane l
-  // holds entry 16 w + (l & 15) of a block of y; the warp shares them.
+  // Two buffers, as in the forward solve; after the tiles this thread's share of
+  // U_b: row r = tid / 2, columns 64 (tid % 2) .. + 63.
   float4 lv[2][16];
-  double yd[2];
-  auto fetch = [&](int64_t k, int buf) {  // tile column b is full (b < k)
-    const int64_t k0 = k * kBig;
+  auto fetch = [&](int64_t k, float4 (&t)[16]) {
+    if (k > b) {
 #pragma unroll
-    for (int rr = 0; rr < 16; ++rr) {
-      const int64_t row = k0 + 16 * w + rr;
-      lv[buf][rr] = row < m ? __ldg(reinterpret_cast<const float4*>(L + row * ldm + r0 + 4 * lane))
-                            : make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int rr = 0; rr < 16; ++rr) {
+        const int64_t row = k * kBig + 16 * w + rr;
+        t[rr] = row < m ? __ldg(reinterpret_cast<const float4*>(L + row * ldm + r0 + 4 * lane))
+                        : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+    } else {
+      const float4* Ub = reinterpret_cast<const float4*>(Uinv + (int64_t)b * kBig * kBig + (int64_t)(tid >> 1) * kBig +
+                                                         64 * (tid & 1));
+#pragma unroll
+      for (int r = 0; r < 16; ++r) t[r] = __ldg(Ub + r);
     }
-    const int64_t mine = k0 + 16 * w + (lane & 15);
-    yd[buf] = mine < m ? ld_relaxed_f64(y + mine) : 0.0;
   };
-  auto consume = [&](int64_t k, int buf) {
-    const int64_t k0 = k * kBig, mine = k0 + 16 * w + (lane & 15);
-    if (!__all_sync(0xffffffffu, __double_as_longlong(yd[buf]) != (long long)kUnset)) {
-      const bool inside[1] = {mine < m};
-      double one[1];
-      if (!poll_entries<1>(y + mine, inside, one, sc)) return false;
-      yd[buf] = one[0];
+  auto consume = [&](int64_t k, const float4 (&t)[16]) {
+    const int64_t at = nblk - 1 - k;  // its place in the chain
+    const float* yk = sm.zs[k & 1];
+    if (at >= own) {
+      if (__syncthreads_or(!wait_peer(sm, (int)(at - own), sc))) return false;
+      yk = sm.zc[at - own];
+    } else {
+      fetch_block(sm, y, m, k, k & 1, at + 3 < own, sc);
+      __syncthreads();
+      if (!sm.ok[k & 1]) return false;
     }
-    const float ymine = (float)yd[buf];
 #pragma unroll
-    for (int rr = 0; rr < 16; ++rr) {
-      const float yv = __shfl_sync(0xffffffffu, ymine, rr);
-      colp[0] = fmaf(lv[buf][rr].x, yv, colp[0]);
-      colp[1] = fmaf(lv[buf][rr].y, yv, colp[1]);
-      colp[2] = fmaf(lv[buf][rr].z, yv, colp[2]);
-      colp[3] = fmaf(lv[buf][rr].w, yv, colp[3]);
+    for (int rr = 0; rr < 16; rr += 4) {
+      const float4 q = *reinterpret_cast<const float4*>(&yk[16 * w + rr]);
+      const float yv[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        colp[0] = fmaf(t[rr + e].x, yv[e], colp[0]);
+        colp[1] = fmaf(t[rr + e].y, yv[e], colp[1]);
+        colp[2] = fmaf(t[rr + e].z, yv[e], colp[2]);
+        colp[3] = fmaf(t[rr + e].w, yv[e], colp[3]);
+      }
     }
     return true;
   };
-  if (nblk - 1 > b) fetch(nblk - 1, 0);
-  for (int64_t k = nblk - 1; k > b && ok; k -= 2) {
-    if (k - 1 > b) fetch(k - 1, 1);
-    ok = consume(k, 0);
-    if (!ok || k - 1 <= b) break;
-    if (k - 2 > b) fetch(k - 2, 0);
-    ok = consume(k - 1, 1);
+  const int64_t nk = nblk - 1 - b;  // tiles: k = nblk - 1 - i, i < nk
+  fetch(nblk - 1, lv[0]);
+  for (int64_t i = 0; i < nk && ok; i += 2) {
+    fetch(nblk - 2 - i, lv[1]);
+    ok = consume(nblk - 1 - i, lv[0]);
+    if (!ok || i + 1 >= nk) break;
+    fetch(nblk - 3 - i, lv[0]);
+    ok = consume(nblk - 2 - i, lv[1]);
   }
+  if (!ok) return false;  // a wait gave up: the status says why
   *reinterpret_cast<float4*>(&sm.red[w][4 * lane]) = make_float4(colp[0], colp[1], colp[2], colp[3]);
-  if (__syncthreads_or(!ok)) return;  // a wait gave up: the status says why
+  __syncthreads();
   if (tid < kBig) {
-    float s = 0.f;
+    float t = 0.f;
 #pragma unroll
-    for (int ww = 0; ww < 8; ++ww) s += sm.red[ww][tid];
-    sm.rhs[tid] = tid < rb ? zmine - s : 0.f;
+    for (int ww = 0; ww < 8; ++ww) t += sm.red[ww][tid];
+    sm.rhs[tid] = tid < rb ? zmine - t : 0.f;
   }
   __syncthreads();
-  const int r = tid & 127, h = tid >> 7;  // y_r = sum_c U_rc rhs_c, columns split in two halves
-  float s = 0.f;
-#pragma unroll 8
-  for (int c = 64 * h; c < 64 * h + 64; ++c) s = fmaf(sm.U[r][c], sm.rhs[c], s);
-  __syncthreads();  // (red is reused)
-  sm.red[h][r] = s;
-  __syncthreads();
-  if (tid < rb) st_relaxed_f64(y + r0 + tid, (double)(sm.red[0][tid] + sm.red[1][tid]));
+  const float* half = &sm.rhs[64 * (tid & 1)];
+  float s = (nk & 1) ? dot64(lv[1], half) : dot64(lv[0], half);  // y_r = sum_c U_rc rhs_c
+  s += __shfl_xor_sync(0xffffffffu, s, 1);
+  send_entry(sm, s, b);
+  const int r = tid >> 1;
+  const bool mine = (tid & 1) == 0 && r < rb;
+  if (mine) st_relaxed_f64(y + r0 + r, (double)s);
+  if (dpart) {
+    const double d = warp_sum(mine ? rho[r0 + r] * (double)s : 0.0);
+    if (lane == 0) sm.mx[w][0] = d;
+    __syncthreads();
+    if (tid == 0) {
+      double g = 0.0;
+      for (int k = 0; k < 8; ++k) g += sm.mx[k][0];
+      dpart[b] = g;
+    }
+  }
+  return true;
 }
 
-cudaError_t trsv_blk_prepare() {
-  static bool done = false;  // per process; the attribute is per function
-  if (done) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(k_trsv_lower_blk, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)sizeof(TrsvSmem));
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_trsv_upper_blk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TrsvSmem));
-  if (e == cudaSuccess) done = true;
-  return e;
+__global__ void __launch_bounds__(kThreads, 1) k_trsv_upper_blk(int64_t m, int64_t ldm, int64_t nblk,
+                                                                const float* __restrict__ L,
+                                                                const float* __restrict__ Uinv, double* zin, double* y,
+                                                                const double* __restrict__ rho, double* dpart,
+                                                                const double* __restrict__ npart, unsigned* ticket,
+                                                                Scalars* sc) {
+  __shared__ TrsvSmem sm;
+  const int64_t pos = chain_position(sm, ticket);
+  leave(sm, trsv_upper_block(sm, pos, nblk, m, ldm, L, Uinv, zin, y, rho, dpart, npart, sc));
+}
+
+template <class... Params, class... Args>
+cudaError_t launch_clusters(cudaStream_t st, int64_t nblk, void (*kernel)(Params...), Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)((nblk + kClu - 1) / kClu * kClu));
+  cfg.blockDim = dim3(kThreads);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = kClu;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
 }
 
 }  // namespace
 
-cudaError_t trsv_lower_blk(cudaStream_t st, int64_t m, int64_t ldm, const float* L, const float* Uinv,
-                           const double* v, double* z, unsigned* ticket, Scalars* sc) {
+cudaError_t trsv_blk_solve(cudaStream_t st, int64_t m, int64_t ldm, const float* L, const float* Uinv, double* rhs,
+                           double* z, double* out, const CgStep* upd, double* dpart, double* npart, unsigned* ticket,
+                           Scalars* sc) {
   const int64_t nblk = (m + kBig - 1) / kBig;
-  cudaError_t e = trsv_blk_prepare();
-  if (e == cudaSuccess) e = cudaMemsetAsync(z, 0xff, sizeof(double) * m, st);  // every entry kUnset
-  if (e == cudaSuccess) e = cudaMemsetAsync(ticket, 0, sizeof(unsigned), st);
-  if (e != cudaSuccess) return e;
-  k_trsv_lower_blk<<<(unsigned)nblk, kThreads, sizeof(TrsvSmem), st>>>(m, ldm, L, Uinv, v, z, ticket, sc);
-  return cudaGetLastError();
-}
-
-cudaError_t trsv_upper_blk(cudaStream_t st, int64_t m, int64_t ldm, const float* L, const float* Uinv,
-                           const double* z, double* y, unsigned* ticket, Scalars* sc) {
-  const int64_t nblk = (m + kBig - 1) / kBig;
-  cudaError_t e = trsv_blk_prepare();
-  if (e == cudaSuccess) e = cudaMemsetAsync(y, 0xff, sizeof(double) * m, st);  // every entry kUnset
-  if (e == cudaSuccess) e = cudaMemsetAsync(ticket, 0, sizeof(unsigned), st);
-  if (e != cudaSuccess) return e;
-  k_trsv_upper_blk<<<(unsigned)nblk, kThreads, sizeof(TrsvSmem), st>>>(m, ldm, L, Uinv, z, y, ticket, sc);
-  return cudaGetLastError();
+  cudaError_t e = launch_clusters(st, nblk, upd ? k_trsv_lower_blk<true> : k_trsv_lower_blk<false>, m, ldm, nblk, L,
+                                  Uinv, rhs, z, out, upd ? *upd : CgStep{}, npart, ticket, sc);
+  if (e == cudaSuccess)
+    e = launch_clusters(st, nblk, k_trsv_upper_blk, m, ldm, nblk, L, Uinv, z, out, rhs, dpart,
+                        upd ? npart : (double*)nullptr, ticket, sc);
+  return e;
 }
 
 }  // namespace pdas

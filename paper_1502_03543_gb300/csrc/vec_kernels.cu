@@ -1,8 +1,7 @@
 // vec_kernels.cu -- the bandwidth-bound steps of one PDAS iteration:
-//   scaling D = S^{-1} X (Eq. 4), the right-hand side r = A x and the
-//   refinement residual r - A(D(A' dy)) (Section V), the direction
-//   ds = -A' dy, dx = D(-ds) - x (Section V), the psi ratio test and the step
-//   (algorithm of Section III).
+//   scaling D = S^{-1} X (Eq. 4), the direction ds = -A' dy, dx = D(-ds) - x
+//   (Section V), the psi ratio test and the step (algorithm of Section III),
+//   the vector work of the refinement.  (passes.cu has the passes over A.)
 //
 // All sums are deterministic: every thread accumulates a fixed strided slice,
 // blocks reduce with a fixed shuffle tree, and the last block to finish
@@ -84,72 +83,6 @@ __global__ void __launch_bounds__(kThreads) k_scaling(int64_t n, const double* _
     sc->dmin = gmn;
     if (sc->bad_iterate && sc->status == 0) sc->status = PDAS_ERR_NOT_INTERIOR;
     tickets[T_SCALING] = 0;
-  }
-}
-
-// ---------------------------------------------------------------------------
-// a2 / a6: out_p = A_p. v  (base == null)  or  out_p = base_p - A_p. v.
-// ROWS rows per block; FP64 accumulation of exactly widened A.  With
-// norm_slot >= 0 also reduces max_p |out_p| into sc->rnorm (slot 0) or
-// sc->rho_norm (slot 1).
-template <typename T, int ROWS>
-__global__ void __launch_bounds__(kThreads) k_gemv(int64_t m, int64_t n, const T* __restrict__ A,
-                                                   const double* __restrict__ v, const double* __restrict__ base,
-                                                   double* __restrict__ out, int vec_ok, double* part,
-                                                   unsigned* tickets, Scalars* sc, int norm_slot) {
-  __shared__ double sm[32];
-  __shared__ double rowsum[ROWS];
-  if (failed(sc)) return;
-  constexpr int VN = Vec<T>::N;
-  const int64_t p0 = (int64_t)blockIdx.x * ROWS;
-  double acc[ROWS];
-#pragma unroll
-  for (int r = 0; r < ROWS; ++r) acc[r] = 0.0;
-  if (vec_ok) {
-    for (int64_t j = (int64_t)threadIdx.x * VN; j < n; j += (int64_t)blockDim.x * VN) {
-      double vv[VN];
-#pragma unroll
-      for (int k = 0; k < VN; ++k) vv[k] = __ldg(v + j + k);
-#pragma unroll
-      for (int r = 0; r < ROWS; ++r) {
-        if (p0 + r < m) {
-          double a[VN];
-          Vec<T>::load(A + (p0 + r) * n + j, a);
-#pragma unroll
-          for (int k = 0; k < VN; ++k) acc[r] = fma(a[k], vv[k], acc[r]);
-        }
-      }
-    }
-  } else {
-    for (int64_t j = threadIdx.x; j < n; j += blockDim.x) {
-      const double vj = __ldg(v + j);
-#pragma unroll
-      for (int r = 0; r < ROWS; ++r)
-        if (p0 + r < m) acc[r] = fma(widen(A[(p0 + r) * n + j]), vj, acc[r]);
-    }
-  }
-  double amax = 0.0;
-#pragma unroll
-  for (int r = 0; r < ROWS; ++r) {
-    double t = block_reduce<0>(acc[r], sm);
-    if (threadIdx.x == 0) rowsum[r] = t;
-  }
-  __syncthreads();
-  if (threadIdx.x < ROWS && p0 + threadIdx.x < m) {
-    const int64_t p = p0 + threadIdx.x;
-    const double o = base ? base[p] - rowsum[threadIdx.x] : rowsum[threadIdx.x];
-    out[p] = o;
-    amax = fabs(o);
-    if (!isfinite(o)) amax = INFINITY;
-  }
-  if (norm_slot < 0) return;
-  double bm = block_reduce<1>(amax, sm);
-  if (threadIdx.x == 0) part[blockIdx.x] = bm;
-  if (!last_block(tickets + T_NORM)) return;
-  double g = combine<1>(part, gridDim.x, sm);
-  if (threadIdx.x == 0) {
-    if (norm_slot == 0) sc->rnorm = g; else sc->rho_norm = g;
-    tickets[T_NORM] = 0;
   }
 }
 
@@ -356,16 +289,63 @@ __global__ void __launch_bounds__(kThreads) k_step(int64_t m, int64_t n, const d
   }
 }
 
+static_assert(sizeof(Scalars) % 8 == 0 && sizeof(Scalars) / 8 <= 32, "one 8-byte word per lane");
+__global__ void k_snapshot(const Scalars* sc, Scalars* out, unsigned* seq, unsigned want) {
+  if (threadIdx.x < sizeof(Scalars) / 8)
+    reinterpret_cast<volatile unsigned long long*>(out)[threadIdx.x] =
+        __ldcg(reinterpret_cast<const unsigned long long*>(sc) + threadIdx.x);
+  __threadfence_system();
+  __syncwarp();
+  if (threadIdx.x == 0) *(volatile unsigned*)seq = want;
+}
+
 __global__ void k_axpy(int64_t n, double a, const double* __restrict__ xv, double* yv, const Scalars* sc) {
   if (failed(sc)) return;
   for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x)
     yv[j] += a * xv[j];
 }
 
-// dot product into sc->dot_a (slot 0) or sc->dot_b (slot 1); fixed order.
-__global__ void __launch_bounds__(kThreads) k_dot(int64_t n, const double* __restrict__ a,
-                                                  const double* __restrict__ b, double* part, unsigned* tickets,
-                                                  Scalars* sc, int slot) {
+__global__ void __launch_bounds__(kThreads) k_cg_update(int64_t m, const CgStep upd, double* rho, double* part,
+                                                        unsigned* tickets, Scalars* sc) {
+  __shared__ double sm[32];
+  if (failed(sc)) return;
+  const double rz = *upd.rz;
+  const bool go = rz > 0.0 && isfinite(rz);
+  const double a = go ? rz / sc->dot_b : 0.0;
+  double mr = 0.0, my = 0.0;
+  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x) {
+    double y = upd.dy[j], r = rho[j];
+    if (go) {
+      y = y + a * upd.p[j];
+      r = r - a * upd.q[j];
+      upd.dy[j] = y;
+      rho[j] = r;
+    }
+    mr = r == r ? fmax(mr, fabs(r)) : INFINITY;
+    my = y == y ? fmax(my, fabs(y)) : INFINITY;
+  }
+  mr = block_reduce<1>(mr, sm);
+  my = block_reduce<1>(my, sm);
+  if (threadIdx.x == 0) {
+    part[2 * blockIdx.x] = mr;
+    part[2 * blockIdx.x + 1] = my;
+  }
+  if (!last_block(tickets + T_NORM2)) return;
+  if (threadIdx.x == 0) {
+    double gr = 0.0, gy = 0.0;
+    for (int i = 0; i < (int)gridDim.x; ++i) {
+      gr = fmax(gr, __ldcg(part + 2 * i));
+      gy = fmax(gy, __ldcg(part + 2 * i + 1));
+    }
+    sc->rho_norm = gr;
+    sc->dynorm = gy;
+    tickets[T_NORM2] = 0;
+  }
+}
+
+__global__ void __launch_bounds__(kThreads) k_cg_dot(int64_t n, const double* __restrict__ a,
+                                                     const double* __restrict__ b, double* part, double* dpart,
+                                                     unsigned* tickets, const Scalars* sc) {
   __shared__ double sm[32];
   if (failed(sc)) return;
   double acc = 0.0;
@@ -377,7 +357,7 @@ __global__ void __launch_bounds__(kThreads) k_dot(int64_t n, const double* __res
   if (threadIdx.x == 0) {
     double g = 0.0;
     for (int i = 0; i < (int)gridDim.x; ++i) g += __ldcg(part + i);
-    if (slot == 0) sc->dot_a = g; else sc->dot_b = g;
+    dpart[0] = g;
     tickets[T_DOT] = 0;
   }
 }
@@ -395,25 +375,6 @@ __global__ void __launch_bounds__(kThreads) k_diag_max(int64_t m, int64_t ldm, c
   double g = combine<1>(part, gridDim.x, sm);
   if (threadIdx.x == 0) {
     sc->mnorm = g;
-    tickets[T_NORM2] = 0;
-  }
-}
-
-__global__ void __launch_bounds__(kThreads) k_absmax(int64_t n, const double* __restrict__ v, double* part,
-                                                     unsigned* tickets, Scalars* sc, int slot) {
-  __shared__ double sm[32];
-  if (failed(sc)) return;
-  double mx = 0.0;
-  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x) {
-    const double a = fabs(v[j]);
-    mx = (a == a) ? fmax(mx, a) : INFINITY;
-  }
-  mx = block_reduce<1>(mx, sm);
-  if (threadIdx.x == 0) part[blockIdx.x] = mx;
-  if (!last_block(tickets + T_NORM2)) return;
-  double g = combine<1>(part, gridDim.x, sm);
-  if (threadIdx.x == 0) {
-    if (slot == 1) sc->rho_norm = g; else sc->dynorm = g;
     tickets[T_NORM2] = 0;
   }
 }
@@ -513,23 +474,6 @@ __global__ void k_adjoint_dA(int64_t m, int64_t n, const double* __restrict__ la
   }
 }
 
-__global__ void k_krylov_update(int64_t n, const double* base, const double* __restrict__ p, double* out, int sign,
-                                const Scalars* sc) {
-  if (failed(sc)) return;
-  const double coef = sc->dot_a / sc->dot_b;
-  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x)
-    out[j] = sign > 0 ? base[j] + coef * p[j] : base[j] - coef * p[j];
-}
-
-// p = z + (dot_a / beta_num) p
-__global__ void k_krylov_direction(int64_t n, const double* __restrict__ z, double* p, double beta_den,
-                                   const Scalars* sc) {
-  if (failed(sc)) return;
-  const double beta = sc->dot_a / beta_den;
-  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x)
-    p[j] = z[j] + beta * p[j];
-}
-
 __global__ void k_convert_matrix(int64_t m, int64_t ld_src, const void* src, int src_f64, int64_t ld_dst, void* dst,
                                  int dst_f64) {
   for (int64_t i = blockIdx.y; i < m; i += gridDim.y)
@@ -544,17 +488,6 @@ __global__ void k_convert_matrix(int64_t m, int64_t ld_src, const void* src, int
 }  // namespace
 
 // ---------------------------------------------------------------------------
-template <typename T>
-cudaError_t launch_gemv(cudaStream_t st, int64_t m, int64_t n, const T* A, const double* v, const double* base,
-                        double* out, double* part, unsigned* tickets, Scalars* sc, int norm_slot) {
-  constexpr int ROWS = 4;
-  const int64_t grid = (m + ROWS - 1) / ROWS;
-  if (norm_slot >= 0 && grid > kPartMax) return cudaErrorInvalidConfiguration;
-  k_gemv<T, ROWS><<<(unsigned)grid, kThreads, 0, st>>>(m, n, A, v, base, out, vec_aligned(A, n) ? 1 : 0, part,
-                                                         tickets, sc, norm_slot);
-  return cudaGetLastError();
-}
-
 template <typename T>
 cudaError_t launch_gemv_t(cudaStream_t st, int64_t m, int64_t n, const T* A, const double* u, double* part,
                           int chunks, int64_t rows_per_chunk) {
@@ -606,26 +539,25 @@ cudaError_t launch_step(cudaStream_t st, int64_t m, int64_t n, const double* b, 
   return cudaGetLastError();
 }
 
+cudaError_t launch_snapshot(cudaStream_t st, const Scalars* sc, Scalars* out, unsigned* seq, unsigned want) {
+  k_snapshot<<<1, 32, 0, st>>>(sc, out, seq, want);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_axpy(cudaStream_t st, int64_t n, double a, const double* xv, double* yv, const Scalars* sc) {
   k_axpy<<<grid_for(n), kThreads, 0, st>>>(n, a, xv, yv, sc);
   return cudaGetLastError();
 }
 
-cudaError_t launch_dot(cudaStream_t st, int64_t n, const double* a, const double* b, double* part,
-                       unsigned* tickets, Scalars* sc, int slot) {
-  k_dot<<<grid_for(n, 4), kThreads, 0, st>>>(n, a, b, part, tickets, sc, slot);
+cudaError_t launch_cg_update(cudaStream_t st, int64_t m, const CgStep& upd, double* rho, double* part,
+                             unsigned* tickets, Scalars* sc) {
+  k_cg_update<<<grid_for(m, 4), kThreads, 0, st>>>(m, upd, rho, part, tickets, sc);
   return cudaGetLastError();
 }
 
-cudaError_t launch_krylov_update(cudaStream_t st, int64_t n, const double* base, const double* p, double* out,
-                                 int sign, const Scalars* sc) {
-  k_krylov_update<<<grid_for(n), kThreads, 0, st>>>(n, base, p, out, sign, sc);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_krylov_direction(cudaStream_t st, int64_t n, const double* z, double* p, double beta_den,
-                                    const Scalars* sc) {
-  k_krylov_direction<<<grid_for(n), kThreads, 0, st>>>(n, z, p, beta_den, sc);
+cudaError_t launch_cg_dot(cudaStream_t st, int64_t m, const double* a, const double* b, double* part, double* dpart,
+                          unsigned* tickets, Scalars* sc) {
+  k_cg_dot<<<grid_for(m, 4), kThreads, 0, st>>>(m, a, b, part, dpart, tickets, sc);
   return cudaGetLastError();
 }
 
@@ -652,12 +584,6 @@ template cudaError_t launch_gather_columns<float>(cudaStream_t, int64_t, int64_t
                                                   const int*, float*, double*);
 template cudaError_t launch_gather_columns<__nv_bfloat16>(cudaStream_t, int64_t, int64_t, const __nv_bfloat16*,
                                                           const double*, int64_t, const int*, __nv_bfloat16*, double*);
-
-cudaError_t launch_absmax(cudaStream_t st, int64_t n, const double* v, double* part, unsigned* tickets, Scalars* sc,
-                          int slot) {
-  k_absmax<<<grid_for(n, 4), kThreads, 0, st>>>(n, v, part, tickets, sc, slot);
-  return cudaGetLastError();
-}
 
 template <typename T>
 cudaError_t launch_normal_diag(cudaStream_t st, int64_t m, int64_t n, const T* A, const double* D, double* out,
@@ -719,9 +645,7 @@ cudaError_t launch_convert_matrix(cudaStream_t st, int64_t m, int64_t ld_src, co
   return cudaGetLastError();
 }
 
-#define PDAS_INST(T)                                                                                          \
-  template cudaError_t launch_gemv<T>(cudaStream_t, int64_t, int64_t, const T*, const double*, const double*, \
-                                      double*, double*, unsigned*, Scalars*, int);                            \
+#define PDAS_INST(T)                                                                                           \
   template cudaError_t launch_gemv_t<T>(cudaStream_t, int64_t, int64_t, const T*, const double*, double*, int, \
                                         int64_t);
 PDAS_INST(double)
