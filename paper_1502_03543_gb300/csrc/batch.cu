@@ -15,6 +15,12 @@
 // All reductions are block-level with a fixed order, so results do not
 // depend on which CTA or in which order the LPs run.
 //
+// What bounds it: the makespan is the slowest LP, whose phases run one after
+// another in one CTA.  Cycles of the slowest of 512 LPs (239 x 956, 21 iterations to
+// a gap of 3e-2, 76 conjugate-gradient steps; before with 256 threads -> now with
+// 512), in millions: formation 18 -> 7, FP32 factor 2.7, preconditioner 1.6,
+// products of the refinement 35 -> 19, FP64 tier 47 -> 35 (6 iterations).
+//
 // GB300 issues FP64 at 1/64 of its FP32 rate; the passes A v (r = A x and
 // the outer product of M v) run in double-float (df_util.cuh), about FP64
 // accurate, while the passes A' v stay FP64 because D multiplies their result
@@ -66,7 +72,7 @@ struct BatchArgs {
 
 // Shared-memory layout for capacities (mc, nc): 16-byte aligned sections.
 struct BatchSmem {
-  size_t L, dinv, zf, vm, pm2, D, w, un2, kidx, stage, dc, scal, total;
+  size_t L, dinv, zf, vm, pm2, D, w, un2, kidx, stage, dc, pr, scal, total;
 };
 __host__ __device__ inline size_t al16(size_t v) { return (v + 15) & ~size_t(15); }
 __host__ __device__ inline BatchSmem batch_smem(int mc, int nc) {
@@ -81,8 +87,9 @@ __host__ __device__ inline BatchSmem batch_smem(int mc, int nc) {
   o.w = p;     p = al16(p + sizeof(double) * nc);
   o.un2 = p;   p = al16(p + sizeof(float2) * nc);
   o.kidx = p;  p = al16(p + sizeof(int) * nc);
-  o.stage = p; p = al16(p + sizeof(float) * mc * 34);  // (also an FP64 panel of 16 columns, pitch 17)
+  o.stage = p; p = al16(p + sizeof(float) * (mc * 34 + 64));  // (32 columns, pitch mc + 4; an FP64 panel of 16 columns, pitch 17)
   o.dc = p;    p = al16(p + sizeof(float) * 64);
+  o.pr = p;    p = al16(p + sizeof(float) * 32 * 16);
   o.scal = p;  p = al16(p + sizeof(double) * 32);
   o.total = p;
   return o;
@@ -112,8 +119,9 @@ struct Ctx {
   float2* un2;   // an n-vector as FP32 pairs
   float2* pm2;   // an m-vector as FP32 pairs
   int* kidx;     // FP64 tier: the columns kept for the normal matrix
-  float* stage;  // [m_cap][33]: 32 columns of A D^1/2
-  float* dc;     // 32 entries of D^1/2, or of D as FP32 pairs (64 floats)
+  float* stage;  // 32 columns of A D^1/2; a panel of the factor; then the inverses of its diagonal blocks
+  float* dc;     // 32 entries of D^1/2, or of D as FP32 pairs (64 floats); a block of the solves
+  float* pr;     // partial sums of the solves, 32 per warp
   double* scal;  // reduction scratch
   const float* A;
   int m, n;
@@ -140,167 +148,448 @@ __device__ __forceinline__ double bmax(double v, double* scal) {
   return r;
 }
 
-// out_p = [base_p -] A_p. v for the FP32-pair vector v2 (n); one warp per row.
+// v[0 .. 3] summed over the warp by halving exchanges (6 FP64 additions instead
+// of 20): lane l returns the sum of entry l / 8.
+__device__ __forceinline__ double warp_sum4(double (&v)[4], int lane) {
+  const bool h16 = lane & 16, h8 = lane & 8;
+  double a[2];
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const double keep = h16 ? v[i + 2] : v[i], give = h16 ? v[i] : v[i + 2];
+    a[i] = keep + __shfl_xor_sync(0xffffffffu, give, 16);
+  }
+  double s = (h8 ? a[1] : a[0]) + __shfl_xor_sync(0xffffffffu, h8 ? a[0] : a[1], 8);
+  s += __shfl_xor_sync(0xffffffffu, s, 4);
+  s += __shfl_xor_sync(0xffffffffu, s, 2);
+  s += __shfl_xor_sync(0xffffffffu, s, 1);
+  return s;
+}
+
+// out_p = [base_p -] A_p. v for the FP32-pair vector v2 (n); four rows per warp
+// at a time, 32 loads in flight per lane (the passes of a CTA are bound by the
+// latency of L2; with 8 in flight they took 130k cycles at 239 x 956).
 template <int T>
 __device__ void blk_gemv(const Ctx& c, const float2* v2, const double* base, double* out) {
   constexpr int NW = T / 32;
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-  for (int p = wp; p < c.m; p += NW) {
-    const float* row = c.A + (int64_t)p * c.n;
-    double acc = 0.0;
-    float hi = 0.f, lo = 0.f;
-    for (int j0 = lane; j0 < c.n; j0 += 32 * 8) {  // 8 loads in flight per lane
-      float av[8];
-      float2 vv[8];
+  for (int p = 4 * wp; p < c.m; p += 4 * NW) {
+    const float* row[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) row[i] = c.A + (int64_t)min(p + i, c.m - 1) * c.n;
+    double acc[4] = {0.0, 0.0, 0.0, 0.0};
+    float hi[4] = {0.f, 0.f, 0.f, 0.f}, lo[4] = {0.f, 0.f, 0.f, 0.f};
+    int it = 0;
+    for (int j0 = lane; j0 < c.n; j0 += 32 * 8) {
+      float av[4][8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) av[i][u] = j0 + 32 * u < c.n ? __ldg(row[i] + j0 + 32 * u) : 0.f;
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
-        const int j = j0 + 32 * u;
-        av[u] = j < c.n ? __ldg(row + j) : 0.f;
-        vv[u] = j < c.n ? v2[j] : make_float2(0.f, 0.f);
-      }
+        const float2 vv = j0 + 32 * u < c.n ? v2[j0 + 32 * u] : make_float2(0.f, 0.f);
 #pragma unroll
-      for (int u = 0; u < 8; ++u) df_madd(hi, lo, av[u], vv[u].x, vv[u].y);
-      df_flush(acc, hi, lo);
+        for (int i = 0; i < 4; ++i) df_madd(hi[i], lo[i], av[i][u], vv.x, vv.y);
+      }
+      if ((++it & 1) == 0 || j0 + 32 * 8 >= c.n) {  // at most 16 terms
+#pragma unroll
+        for (int i = 0; i < 4; ++i) df_flush(acc[i], hi[i], lo[i]);
+      }
     }
-    acc = warp_sum(acc);
-    if (lane == 0) out[p] = base ? base[p] - acc : acc;
+    const double s = warp_sum4(acc, lane);
+    const int r = p + (lane >> 3);
+    if ((lane & 7) == 0 && r < c.m) out[r] = base ? base[r] - s : s;
   }
 }
 
-// out_j = sum_p A_pj u_p in FP64 (exact widening of A on the integer pipes,
-// FP64 multiply-adds); one thread per column.  Every use of A' (.) here is
-// multiplied by D afterwards (dx = D w - x, u = D A' v), which spans many
+// A'u for U columns per thread, j0 + T q (q < U), with 32 loads of A in flight per
+// thread.  DF: double-float for the FP32-pair vector u2; else FP64 (exact
+// widening of A on the integer pipes, FP64 multiply-adds).
+template <int T, int U, bool DF>
+__device__ __forceinline__ void columns(const Ctx& c, int j0, const double* u, const float2* u2, double* out) {
+  constexpr int B = 32 / U;  // rows per batch
+  const float* col[U];
+  double acc[U];
+  float hi[U], lo[U];
+#pragma unroll
+  for (int q = 0; q < U; ++q) {
+    col[q] = c.A + min(j0 + T * q, c.n - 1);
+    acc[q] = 0.0;
+    hi[q] = lo[q] = 0.f;
+  }
+  int terms = 0;
+  for (int p0 = 0; p0 < c.m; p0 += B) {
+    float av[U][B];
+#pragma unroll
+    for (int k = 0; k < B; ++k)
+#pragma unroll
+      for (int q = 0; q < U; ++q) av[q][k] = p0 + k < c.m ? __ldg(col[q] + (int64_t)(p0 + k) * c.n) : 0.f;
+    if constexpr (DF) {
+#pragma unroll
+      for (int k = 0; k < B; ++k) {
+        const float2 v = p0 + k < c.m ? u2[p0 + k] : make_float2(0.f, 0.f);
+#pragma unroll
+        for (int q = 0; q < U; ++q) df_madd(hi[q], lo[q], av[q][k], v.x, v.y);
+      }
+      terms += B;
+      if (terms >= 16 || p0 + B >= c.m) {  // (a batch has at most 32 terms)
+        terms = 0;
+#pragma unroll
+        for (int q = 0; q < U; ++q) df_flush(acc[q], hi[q], lo[q]);
+      }
+    } else {
+#pragma unroll
+      for (int k = 0; k < B; ++k)
+        if (p0 + k < c.m) {
+          const double up = u[p0 + k];
+#pragma unroll
+          for (int q = 0; q < U; ++q) acc[q] = fma(widen_bits(__float_as_uint(av[q][k])), up, acc[q]);
+        }
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < U; ++q)
+    if (j0 + T * q < c.n) out[j0 + T * q] = acc[q];
+}
+
+template <int T, bool DF>
+__device__ void blk_columns(const Ctx& c, const double* u, const float2* u2, double* out) {
+  const int n = c.n;
+  for (int j0 = 0; j0 < n;) {
+    const int left = n - j0;
+    if (left > 2 * T) {
+      columns<T, 4, DF>(c, j0 + threadIdx.x, u, u2, out);
+      j0 += 4 * T;
+    } else if (left > T) {
+      columns<T, 2, DF>(c, j0 + threadIdx.x, u, u2, out);
+      j0 += 2 * T;
+    } else {
+      columns<T, 1, DF>(c, j0 + threadIdx.x, u, u2, out);
+      j0 += T;
+    }
+  }
+}
+
+// out_j = sum_p A_pj u_p in FP64; a thread per column.  Every use of A' (.)
+// here is multiplied by D afterwards (dx = D w - x, u = D A' v), which spans many
 // orders of magnitude near the optimum, so this pass keeps FP64 accuracy.
 template <int T>
 __device__ void blk_gemv_t(const Ctx& c, const double* u, double* out) {
-  for (int j = threadIdx.x; j < c.n; j += T) {
-    const float* col = c.A + j;
-    double acc = 0.0;
-    for (int p0 = 0; p0 < c.m; p0 += 8) {  // 8 loads in flight per thread
-      float av[8];
-#pragma unroll
-      for (int k = 0; k < 8; ++k) av[k] = p0 + k < c.m ? __ldg(col + (int64_t)(p0 + k) * c.n) : 0.f;
-#pragma unroll
-      for (int k = 0; k < 8; ++k)
-        if (p0 + k < c.m) acc = fma(widen_bits(__float_as_uint(av[k])), u[p0 + k], acc);
-    }
-    out[j] = acc;
-  }
+  blk_columns<T, false>(c, u, nullptr, out);
+}
+
+// The same in double-float for the FP32-pair vector u2 (m).  Used for the
+// conjugate-gradient operator and the first residual while the factor is FP32,
+// where D spans fewer orders of magnitude.
+template <int T>
+__device__ void blk_gemv_t_df(const Ctx& c, const float2* u2, double* out) {
+  blk_columns<T, true>(c, nullptr, u2, out);
 }
 
 // M = (A D^1/2)(A D^1/2)' into c.L (packed lower), FP32: 32-column chunks of
-// A D^1/2 staged in shared memory; warps take 32 x 32 lower tiles, a lane
-// holding rows lr + 8 i (i < 4) and columns lc + 4 j (j < 8) of its tile.
-// m_cap is a multiple of 32, so every staged row index is in range; rows past
-// m are staged as zero.
+// A D^1/2 staged in shared memory column by column (pitch m_cap + 4; rows past m
+// are zero), and every thread accumulates 8 x 8 units of the lower triangle in
+// registers over all chunks: four 16-byte reads for 64 multiply-adds.  (With 4 x 8
+// outputs a lane, 12 reads for 32 multiply-adds and a read-modify-write of the
+// triangle per chunk, a formation took 1.14M cycles at 239 x 956; the
+// multiply-adds alone take 0.23M.)  m_cap is a multiple of 32.
 template <int T>
 __device__ void blk_syrk(const Ctx& c, int m_cap) {
   constexpr int NW = T / 32;
-  const int m = c.m, n = c.n;
-  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, lr = lane >> 2, lc = lane & 3;
-  const int mt = (m + 31) >> 5, ntile = mt * (mt + 1) / 2;
-  for (int e = threadIdx.x; e < m * (m + 1) / 2; e += T) c.L[e] = 0.f;
-  for (int k0 = 0; k0 < n; k0 += 32) {
-    if (threadIdx.x < 32) c.dc[threadIdx.x] = k0 + threadIdx.x < n ? (float)sqrt(c.D[k0 + threadIdx.x]) : 0.f;
-    __syncthreads();
-    for (int e = threadIdx.x; e < m_cap * 32; e += T) {
-      const int r = e >> 5, kk = e & 31;
-      c.stage[r * 33 + kk] = (r < m && k0 + kk < n) ? __ldg(c.A + (int64_t)r * n + k0 + kk) * c.dc[kk] : 0.f;
-    }
-    __syncthreads();
-    for (int t = wp; t < ntile; t += NW) {
-      int tp = 0;
-      while ((tp + 1) * (tp + 2) / 2 <= t) ++tp;
-      const int tq = t - tp * (tp + 1) / 2;
-      float acc[4][8];
+  const int m = c.m, n = c.n, pm = m_cap + 4, lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  const int m8 = (m + 7) >> 3, units = m8 * (m8 + 1) / 2, mr = (m + 31) & ~31;
+  float* sq = reinterpret_cast<float*>(c.w);  // D^1/2 (A'v is not in use during a formation)
+  for (int j = threadIdx.x; j < n; j += T) sq[j] = (float)sqrt(c.D[j]);
+  __syncthreads();
+  for (int u0 = 0; u0 < units; u0 += T) {  // (one pass but for CTAs smaller than the triangle)
+    const int u = u0 + (int)threadIdx.x;
+    const bool mine = u < units;
+    int i = (int)((sqrtf(8.f * u + 1.f) - 1.f) * 0.5f);
+    while (i * (i + 1) / 2 > u) --i;
+    while ((i + 1) * (i + 2) / 2 <= u) ++i;
+    const int r = mine ? 8 * i : 0, q = mine ? 8 * (u - i * (i + 1) / 2) : 0;
+    float acc[8][8];
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+    for (int a = 0; a < 8; ++a)
 #pragma unroll
-        for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
-#pragma unroll 4
-      for (int kk = 0; kk < 32; ++kk) {
-        float a[4], bb[8];
+      for (int b = 0; b < 8; ++b) acc[a][b] = 0.f;
+    for (int k0 = 0; k0 < n; k0 += 32) {
+      const bool kin = k0 + lane < n;
+      const float d = kin ? sq[k0 + lane] : 0.f;
+      for (int r4 = 4 * wp; r4 < mr; r4 += 4 * NW) {
+        float v[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) a[i] = c.stage[(tp * 32 + lr + 8 * i) * 33 + kk];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) bb[j] = c.stage[(tq * 32 + lc + 4 * j) * 33 + kk];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i], bb[j], acc[i][j]);
+        for (int e = 0; e < 4; ++e) v[e] = (kin && r4 + e < m) ? __ldg(c.A + (int64_t)(r4 + e) * n + k0 + lane) : 0.f;
+        *reinterpret_cast<float4*>(c.stage + lane * pm + r4) = make_float4(v[0] * d, v[1] * d, v[2] * d, v[3] * d);
       }
+      __syncthreads();
+      if (mine) {
+#pragma unroll 2
+        for (int kk = 0; kk < 32; ++kk) {
+          float a[8], b[8];
+          const float* row = c.stage + kk * pm;
+          *reinterpret_cast<float4*>(a) = *reinterpret_cast<const float4*>(row + r);
+          *reinterpret_cast<float4*>(a + 4) = *reinterpret_cast<const float4*>(row + r + 4);
+          *reinterpret_cast<float4*>(b) = *reinterpret_cast<const float4*>(row + q);
+          *reinterpret_cast<float4*>(b + 4) = *reinterpret_cast<const float4*>(row + q + 4);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int pr = tp * 32 + lr + 8 * i;
+          for (int x = 0; x < 8; ++x)
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const int qc = tq * 32 + lc + 4 * j;
-          if (pr < m && qc <= pr) c.L[pk(pr, qc)] += acc[i][j];
+            for (int y = 0; y < 8; ++y) acc[x][y] = fmaf(a[x], b[y], acc[x][y]);
         }
       }
+      __syncthreads();
     }
-    __syncthreads();
-  }
-}
-
-// In-place Cholesky of the packed lower triangle (FP32), right-looking by
-// columns, two block barriers per column; the scaled column is read from a
-// contiguous copy (zf) in the trailing update.  Returns false on a pivot that is
-// not positive and finite (the same in every thread).
-template <int T>
-__device__ bool blk_chol(const Ctx& c) {
-  constexpr int NW = T / 32;
-  const int m = c.m, lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-  for (int k = 0; k < m; ++k) {
-    __syncthreads();
-    const float d = c.L[pk(k, k)];
-    if (!(d > 0.f) || !isfinite(d)) return false;
-    const float rs = inv_sqrt32(d);
-    for (int r = k + 1 + threadIdx.x; r < m; r += T) {  // the scaled column, also kept in zf
-      const float v = c.L[pk(r, k)] * rs;
-      c.L[pk(r, k)] = v;
-      c.zf[r] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      c.L[pk(k, k)] = d * rs;
-      c.dinv[k] = rs;
-    }
-    for (int r = k + 1 + wp; r < m; r += NW) {
-      const float lrk = c.zf[r];
-      float* row = c.L + pk(r, 0);
-      for (int q = k + 1 + lane; q <= r; q += 32) row[q] = fmaf(-lrk, c.zf[q], row[q]);
+    if (mine) {
+#pragma unroll
+      for (int x = 0; x < 8; ++x)
+#pragma unroll
+        for (int y = 0; y < 8; ++y)
+          if (r + x < m && q + y <= r + x) c.L[pk(r + x, q + y)] = acc[x][y];
     }
   }
   __syncthreads();
+}
+
+// t = chol(t) (lower triangle of an 8 x 8 block) with rs = 1 / L_cc, or false
+// for a pivot that is not positive and finite.
+__device__ __forceinline__ bool chol8_any(float (&t)[8][8], float (&rs)[8]) {
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    const float d = t[c][c];
+    if (!(d > 0.f) || !isfinite(d)) return false;
+    rs[c] = inv_sqrt32(d);
+#pragma unroll
+    for (int i = c; i < 8; ++i) t[i][c] *= rs[c];
+#pragma unroll
+    for (int j = c + 1; j < 8; ++j)
+#pragma unroll
+      for (int i = j; i < 8; ++i) t[i][j] = fmaf(-t[i][c], t[j][c], t[i][j]);
+  }
   return true;
 }
 
-// out = (L L')^{-1} v (FP64 in and out, FP32 solves by warp 0; the rows of
-// the vector are spread over the lanes, the pivot entry is read by all).
+// In-place Cholesky of the packed lower triangle (FP32) in panels of 32
+// columns.  The panel is copied column by column into the stage area (rows 32 at
+// a time hit 32 banks of the packed triangle) and factored in groups of 8
+// columns: every thread factors the group's 8 x 8 block in registers, then a
+// thread per row solves the row and applies the group to the panel's later
+// columns; the trailing triangle takes the whole panel in 4 x 4 units.  16
+// block barriers per panel.  Returns false on a pivot that is not positive and
+// finite (the same in every thread).  Column by column, with two barriers and a
+// read-modify-write of the triangle per column, it took about a fifth of an
+// iteration at m = 240.
 template <int T>
-__device__ void blk_precond(const Ctx& c, const double* v, double* out) {
-  const int m = c.m, lane = threadIdx.x & 31;
-  for (int i = threadIdx.x; i < m; i += T) c.zf[i] = (float)v[i];
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    for (int r = 0; r < m; ++r) {  // L z = v, row by row (contiguous packed rows)
-      const float* row = c.L + pk(r, 0);
-      float t = 0.f;
-      for (int k = lane; k < r; k += 32) t = fmaf(row[k], c.zf[k], t);
-      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-      if (lane == 0) c.zf[r] = (c.zf[r] - t) * c.dinv[r];
-      __syncwarp();
+__device__ bool blk_chol(const Ctx& c, int pm) {
+  const int m = c.m, mr = (m + 31) & ~31;  // pm: the pitch, m_cap >= mr
+  float* P = c.stage;                      // element (r, c0 + q) at P[q pm + r]
+  for (int c0 = 0; c0 < m; c0 += 32) {
+    const int R = mr - c0;
+    for (int e = threadIdx.x; e < 32 * R; e += T) {
+      const int q = e / R, r = c0 + e % R;
+      P[q * pm + r] = (r < m && c0 + q <= r) ? c.L[pk(r, c0 + q)] : (r == c0 + q ? 1.f : 0.f);
     }
-    for (int k = m - 1; k >= 0; --k) {  // L' y = z
-      const float yk = c.zf[k] * c.dinv[k];
-      for (int r = lane; r < k; r += 32) c.zf[r] = fmaf(-c.L[pk(k, r)], yk, c.zf[r]);
-      __syncwarp();
-      if (lane == 0) c.zf[k] = yk;
-      __syncwarp();
+    __syncthreads();
+#pragma unroll 1
+    for (int g = 0; g < 4; ++g) {
+      const int g0 = c0 + 8 * g;
+      if (g0 >= m) break;
+      float t[8][8], rs[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const float4 lo = *reinterpret_cast<const float4*>(P + (8 * g + j) * pm + g0);
+        const float4 hi = *reinterpret_cast<const float4*>(P + (8 * g + j) * pm + g0 + 4);
+        t[0][j] = lo.x, t[1][j] = lo.y, t[2][j] = lo.z, t[3][j] = lo.w;
+        t[4][j] = hi.x, t[5][j] = hi.y, t[6][j] = hi.z, t[7][j] = hi.w;
+      }
+      if (!chol8_any(t, rs)) return false;
+      if (threadIdx.x == 0) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+          if (g0 + k < m) c.dinv[g0 + k] = rs[k];
+      }
+      __syncthreads();  // every thread has read the block
+      for (int r = g0 + threadIdx.x; r < mr; r += T) {
+        float v[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] = P[(8 * g + k) * pm + r];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          float x = v[k];
+#pragma unroll
+          for (int l = 0; l < k; ++l) x = fmaf(-v[l], t[k][l], x);
+          v[k] = g0 + k <= r ? x * rs[k] : 0.f;
+          P[(8 * g + k) * pm + r] = v[k];
+        }
+      }
+      if (g == 3) break;
+      __syncthreads();  // the group's columns are in place
+      for (int r = g0 + 8 + threadIdx.x; r < mr; r += T) {
+        float v[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] = P[(8 * g + k) * pm + r];
+#pragma unroll 1
+        for (int q = 8 * g + 8; q < 32; q += 8) {
+          float x[8];
+#pragma unroll
+          for (int e = 0; e < 8; ++e) x[e] = P[(q + e) * pm + r];
+#pragma unroll
+          for (int k = 0; k < 8; ++k) {
+            const float4 lo = *reinterpret_cast<const float4*>(P + (8 * g + k) * pm + c0 + q);
+            const float4 hi = *reinterpret_cast<const float4*>(P + (8 * g + k) * pm + c0 + q + 4);
+            x[0] = fmaf(-v[k], lo.x, x[0]), x[1] = fmaf(-v[k], lo.y, x[1]);
+            x[2] = fmaf(-v[k], lo.z, x[2]), x[3] = fmaf(-v[k], lo.w, x[3]);
+            x[4] = fmaf(-v[k], hi.x, x[4]), x[5] = fmaf(-v[k], hi.y, x[5]);
+            x[6] = fmaf(-v[k], hi.z, x[6]), x[7] = fmaf(-v[k], hi.w, x[7]);
+          }
+#pragma unroll
+          for (int e = 0; e < 8; ++e) P[(q + e) * pm + r] = x[e];
+        }
+      }
+      __syncthreads();
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < 32 * R; e += T) {
+      const int q = e / R, r = c0 + e % R;
+      if (r < m && c0 + q <= r) c.L[pk(r, c0 + q)] = P[q * pm + r];
+    }
+    const int s0 = c0 + 32, n4 = (mr - s0) >> 2;  // trailing triangle: 4 x 4 units (i, j), j <= i
+    for (int u = threadIdx.x; u < n4 * (n4 + 1) / 2; u += T) {
+      int i = (int)((sqrtf(8.f * u + 1.f) - 1.f) * 0.5f);
+      while (i * (i + 1) / 2 > u) --i;
+      while ((i + 1) * (i + 2) / 2 <= u) ++i;
+      const int r = s0 + 4 * i, q = s0 + 4 * (u - i * (i + 1) / 2);
+      float x[4][4];
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) x[a][b] = 0.f;
+#pragma unroll 8
+      for (int k = 0; k < 32; ++k) {
+        const float4 a = *reinterpret_cast<const float4*>(P + k * pm + r);
+        const float4 b = *reinterpret_cast<const float4*>(P + k * pm + q);
+        const float aa[4] = {a.x, a.y, a.z, a.w}, bb[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+        for (int y = 0; y < 4; ++y)
+#pragma unroll
+          for (int z = 0; z < 4; ++z) x[y][z] = fmaf(aa[y], bb[z], x[y][z]);
+      }
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b)
+          if (r + a < m && q + b <= r + a) c.L[pk(r + a, q + b)] -= x[a][b];
+    }
+    __syncthreads();
+  }
+  return true;
+}
+
+// W_b = L_bb^{-1} of every 32 x 32 diagonal block to the stage area (row-major,
+// pitch 33, zero above the diagonal and past m), a warp per block, lane j its
+// column j: the triangular solves apply them instead of substituting.
+template <int T>
+__device__ void blk_invert_diag(const Ctx& c) {
+  constexpr int NW = T / 32;
+  const int m = c.m, lane = threadIdx.x & 31;
+  for (int b = threadIdx.x >> 5; 32 * b < m; b += NW) {
+    float* W = c.stage + b * 32 * 33;
+    const int r0 = 32 * b;
+#pragma unroll 1
+    for (int r = 0; r < 32; ++r) {
+      float t = 0.f;
+      if (r0 + r < m) {
+        const float* row = c.L + pk(r0 + r, r0);
+        float t0 = r == lane ? 1.f : 0.f, t1 = 0.f;
+        int k = 0;
+        for (; k + 1 < r; k += 2) {
+          t0 = fmaf(-row[k], W[k * 33 + lane], t0);
+          t1 = fmaf(-row[k + 1], W[(k + 1) * 33 + lane], t1);
+        }
+        if (k < r) t0 = fmaf(-row[k], W[k * 33 + lane], t0);
+        t = lane <= r ? (t0 + t1) * c.dinv[r0 + r] : 0.f;
+      }
+      W[r * 33 + lane] = t;  // (each lane reads its own column only)
     }
   }
   __syncthreads();
+}
+
+// out = (L L')^{-1} v (FP64 in and out, FP32 solves in blocks of 32 rows):
+// forward, the warps share a block's rows of the product with the entries solved
+// so far (a row per warp at a time, contiguous packed rows), then warp 0
+// applies W_b; backward, the warps share the rows below the block.  Row by row
+// by one warp it took a quarter of an iteration at m = 240.
+template <int T>
+__device__ void blk_precond(const Ctx& c, const double* v, double* out) {
+  constexpr int NW = T / 32;
+  const int m = c.m, lane = threadIdx.x & 31, wp = threadIdx.x >> 5, nb = (m + 31) >> 5;
+  float* tmp = c.dc;  // the block's right-hand side
+  for (int i = threadIdx.x; i < m; i += T) c.zf[i] = (float)v[i];
+  __syncthreads();
+  for (int b = 0; b < nb; ++b) {  // L z = v
+    const int r0 = 32 * b;
+    constexpr int PER = (32 + NW - 1) / NW;
+    float t[PER];
+#pragma unroll
+    for (int u = 0; u < PER; ++u) {
+      const int row = r0 + wp + NW * u;
+      t[u] = 0.f;
+      if (wp + NW * u < 32 && row < m) {
+        const float* L = c.L + pk(row, 0);
+        for (int k = lane; k < r0; k += 32) t[u] = fmaf(L[k], c.zf[k], t[u]);
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+      for (int u = 0; u < PER; ++u) t[u] += __shfl_xor_sync(0xffffffffu, t[u], o);
+#pragma unroll
+    for (int u = 0; u < PER; ++u) {
+      const int rr = wp + NW * u;
+      if (lane == 0 && rr < 32) tmp[rr] = r0 + rr < m ? c.zf[r0 + rr] - t[u] : 0.f;
+    }
+    __syncthreads();
+    if (wp == 0) {
+      const float* W = c.stage + b * 32 * 33 + lane * 33;
+      float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+#pragma unroll
+      for (int k = 0; k < 32; k += 4) {
+        s0 = fmaf(W[k], tmp[k], s0), s1 = fmaf(W[k + 1], tmp[k + 1], s1);
+        s2 = fmaf(W[k + 2], tmp[k + 2], s2), s3 = fmaf(W[k + 3], tmp[k + 3], s3);
+      }
+      if (r0 + lane < m) c.zf[r0 + lane] = (s0 + s1) + (s2 + s3);
+    }
+    __syncthreads();
+  }
+  for (int b = nb - 1; b >= 0; --b) {  // L' y = z
+    const int r0 = 32 * b;
+    float a0 = 0.f, a1 = 0.f;
+    int r = r0 + 32 + wp;
+    for (; r + NW < m; r += 2 * NW) {
+      a0 = fmaf(c.L[pk(r, r0) + lane], c.zf[r], a0);
+      a1 = fmaf(c.L[pk(r + NW, r0) + lane], c.zf[r + NW], a1);
+    }
+    if (r < m) a0 = fmaf(c.L[pk(r, r0) + lane], c.zf[r], a0);
+    c.pr[wp * 32 + lane] = a0 + a1;
+    __syncthreads();
+    if (wp == 0) {
+      float t = r0 + lane < m ? c.zf[r0 + lane] : 0.f;
+#pragma unroll
+      for (int w = 0; w < NW; ++w) t -= c.pr[w * 32 + lane];
+      tmp[lane] = t;
+      __syncwarp();
+      const float* W = c.stage + b * 32 * 33 + lane;
+      float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+#pragma unroll
+      for (int k = 0; k < 32; k += 4) {
+        s0 = fmaf(W[k * 33], tmp[k], s0), s1 = fmaf(W[(k + 1) * 33], tmp[k + 1], s1);
+        s2 = fmaf(W[(k + 2) * 33], tmp[k + 2], s2), s3 = fmaf(W[(k + 3) * 33], tmp[k + 3], s3);
+      }
+      if (r0 + lane < m) c.zf[r0 + lane] = (s0 + s1) + (s2 + s3);
+    }
+    __syncthreads();
+  }
   for (int i = threadIdx.x; i < m; i += T) out[i] = (double)c.zf[i];
   __syncthreads();
 }
@@ -445,55 +734,121 @@ __device__ bool blk_chol64(const Ctx& c, double* L, double* dinv) {
   return true;
 }
 
-// out = (L L')^{-1} v with the FP64 factor: forward substitution row by row
-// (a warp dot product over the contiguous packed row), back substitution by
-// rows of L (a warp sweep); out must not alias v.
+// The FP64 factor's diagonal blocks inverted (as blk_invert_diag, in FP64) into
+// the shared memory of the FP32 factor, which this tier does not use: column
+// c of block b at W[32 (32 b + c)], zero above the diagonal.  For m_cap > 96 (below
+// that it does not fit, and the row-by-row solves are short).
+constexpr int kMinBlk64 = 96;
 template <int T>
-__device__ void blk_precond64(const Ctx& c, const double* L, const double* dinv, const double* v, double* out) {
+__device__ void blk_invert_diag64(const Ctx& c, const double* L, const double* dinv) {
+  constexpr int NW = T / 32;
   const int m = c.m, lane = threadIdx.x & 31;
-  if (threadIdx.x < 32) {
-    for (int r = 0; r < m; ++r) {  // L z = v
-      const double* row = L + pk(r, 0);
+  double* Wall = reinterpret_cast<double*>(c.L);
+  for (int b = threadIdx.x >> 5; 32 * b < m; b += NW) {
+    double* W = Wall + b * 32 * 32 + lane * 32;  // this lane's column
+    const int r0 = 32 * b;
+#pragma unroll 1
+    for (int r = 0; r < 32; ++r) {
       double t = 0.0;
-      for (int k = lane; k < r; k += 32) t = fma(row[k], out[k], t);
-      t = warp_sum(t);
-      if (lane == 0) out[r] = (v[r] - t) * dinv[r];
-      __syncwarp();
-    }
-    for (int k = m - 1; k >= 0; --k) {  // L' y = z
-      const double yk = out[k] * dinv[k];
-      const double* row = L + pk(k, 0);
-      for (int r = lane; r < k; r += 32) out[r] = fma(-row[r], yk, out[r]);
-      __syncwarp();
-      if (lane == 0) out[k] = yk;
-      __syncwarp();
+      if (r0 + r < m) {
+        const double* row = L + pk(r0 + r, r0);
+        t = r == lane ? 1.0 : 0.0;
+        for (int k = 0; k < r; ++k) t = fma(-__ldcg(row + k), W[k], t);
+        t = lane <= r ? t * dinv[r0 + r] : 0.0;
+      }
+      W[r] = t;
     }
   }
   __syncthreads();
 }
 
-// out_j = sum_p A_pj u_p in double-float for the FP32-pair vector u2 (m);
-// one thread per column.  Used for the conjugate-gradient operator while the
-// factor is FP32, where D spans fewer orders of magnitude.
+// out = (L L')^{-1} v with the FP64 factor in global memory; out must not alias
+// v.  In blocks of 32 rows as blk_precond; for m_cap <= 96 row by row by one
+// warp.
 template <int T>
-__device__ void blk_gemv_t_df(const Ctx& c, const float2* u2, double* out) {
-  for (int j = threadIdx.x; j < c.n; j += T) {
-    const float* col = c.A + j;
-    double acc = 0.0;
-    float hi = 0.f, lo = 0.f;
-    for (int p0 = 0; p0 < c.m; p0 += 8) {  // 8 loads in flight per thread
-      float av[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) av[u] = p0 + u < c.m ? __ldg(col + (int64_t)(p0 + u) * c.n) : 0.f;
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const float2 q = p0 + u < c.m ? u2[p0 + u] : make_float2(0.f, 0.f);
-        df_madd(hi, lo, av[u], q.x, q.y);
+__device__ void blk_precond64(const Ctx& c, int m_cap, const double* L, const double* dinv, const double* v,
+                              double* out) {
+  const int m = c.m, lane = threadIdx.x & 31;
+  if (m_cap <= kMinBlk64) {
+    if (threadIdx.x < 32) {
+      for (int r = 0; r < m; ++r) {  // L z = v
+        const double* row = L + pk(r, 0);
+        double t = 0.0;
+        for (int k = lane; k < r; k += 32) t = fma(row[k], out[k], t);
+        t = warp_sum(t);
+        if (lane == 0) out[r] = (v[r] - t) * dinv[r];
+        __syncwarp();
       }
-      if ((p0 & 15) == 8) df_flush(acc, hi, lo);
+      for (int k = m - 1; k >= 0; --k) {  // L' y = z
+        const double yk = out[k] * dinv[k];
+        const double* row = L + pk(k, 0);
+        for (int r = lane; r < k; r += 32) out[r] = fma(-row[r], yk, out[r]);
+        __syncwarp();
+        if (lane == 0) out[k] = yk;
+        __syncwarp();
+      }
     }
-    df_flush(acc, hi, lo);
-    out[j] = acc;
+    __syncthreads();
+    return;
+  }
+  constexpr int NW = T / 32;
+  const int wp = threadIdx.x >> 5, nb = (m + 31) >> 5;
+  const double* Wall = reinterpret_cast<const double*>(c.L);
+  double* tmp = reinterpret_cast<double*>(c.dc);  // 32 doubles
+  double* pr = reinterpret_cast<double*>(c.stage);  // partial sums (the stage is free outside the formation)
+  for (int b = 0; b < nb; ++b) {  // L z = v
+    const int r0 = 32 * b;
+    for (int rr = 4 * wp; rr < 32; rr += 4 * NW) {  // four rows per warp at a time
+      double t[4] = {0.0, 0.0, 0.0, 0.0};
+      for (int k = lane; k < r0; k += 32) {
+        const double zk = out[k];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) t[i] = fma(L[pk(min(r0 + rr + i, m - 1), 0) + k], zk, t[i]);
+      }
+      const double s = warp_sum4(t, lane);
+      const int row = r0 + rr + (lane >> 3);
+      if ((lane & 7) == 0) tmp[rr + (lane >> 3)] = row < m ? v[row] - s : 0.0;
+    }
+    __syncthreads();
+    if (wp == 0) {
+      const double* W = Wall + b * 32 * 32 + lane;  // row lane: W[32 k]
+      double s0 = 0.0, s1 = 0.0;
+#pragma unroll 8
+      for (int k = 0; k < 32; k += 2) {
+        s0 = fma(W[32 * k], tmp[k], s0);
+        s1 = fma(W[32 * (k + 1)], tmp[k + 1], s1);
+      }
+      if (r0 + lane < m) out[r0 + lane] = s0 + s1;
+    }
+    __syncthreads();
+  }
+  for (int b = nb - 1; b >= 0; --b) {  // L' y = z
+    const int r0 = 32 * b;
+    double a0 = 0.0, a1 = 0.0;
+    int r = r0 + 32 + wp;
+    for (; r + NW < m; r += 2 * NW) {
+      a0 = fma(L[pk(r, r0) + lane], out[r], a0);
+      a1 = fma(L[pk(r + NW, r0) + lane], out[r + NW], a1);
+    }
+    if (r < m) a0 = fma(L[pk(r, r0) + lane], out[r], a0);
+    pr[wp * 32 + lane] = a0 + a1;
+    __syncthreads();
+    if (wp == 0) {
+      double t = r0 + lane < m ? out[r0 + lane] : 0.0;
+#pragma unroll
+      for (int w = 0; w < NW; ++w) t -= pr[w * 32 + lane];
+      tmp[lane] = t;
+      __syncwarp();
+      const double* W = Wall + b * 32 * 32 + lane * 32;  // column lane
+      double s0 = 0.0, s1 = 0.0;
+#pragma unroll 8
+      for (int k = 0; k < 32; k += 2) {
+        s0 = fma(W[k], tmp[k], s0);
+        s1 = fma(W[k + 1], tmp[k + 1], s1);
+      }
+      if (r0 + lane < m) out[r0 + lane] = s0 + s1;
+    }
+    __syncthreads();
   }
 }
 
@@ -532,9 +887,11 @@ __device__ bool factor_lp(const BatchArgs& a, Ctx& c, bool& tier2, double* M64, 
     double dm = 0.0;
     for (int i = threadIdx.x; i < m; i += T) dm = fmax(dm, (double)c.L[pk(i, i)]);
     mnorm = bmax<T>(dm, c.scal);
-    tier2 = !blk_chol<T>(c);
+    tier2 = !blk_chol<T>(c, a.m_cap);
+    if (!tier2) blk_invert_diag<T>(c);
   }
   if (!tier2) return true;
+  __syncthreads();
   // the significant columns: D_j >= 1e-10 max D, at least min(n, 1.25 m)
   // of them (the threshold drops by 16x until enough pass); the factor
   // of A_K D_K A_K' preconditions the exact M in the refinement
@@ -562,14 +919,16 @@ __device__ bool factor_lp(const BatchArgs& a, Ctx& c, bool& tier2, double* M64, 
   double dm = 0.0;
   for (int i = threadIdx.x; i < m; i += T) dm = fmax(dm, M64[pk(i, i)]);
   mnorm = bmax<T>(dm, c.scal);
-  return blk_chol64<T>(c, M64, dinv64);
+  if (!blk_chol64<T>(c, M64, dinv64)) return false;
+  if (a.m_cap > kMinBlk64) blk_invert_diag64<T>(c, M64, dinv64);
+  return true;
 }
 
 // out = (A D A')^{-1} rhs: out = P^-1 rhs, then preconditioned conjugate
 // gradients on the exact M (matrix-free), accepted when ||rhs - M out||_inf
 // <= refine_tol ||rhs||_inf or <= refine_tol (mnorm ||out||_inf +
-// ||rhs||_inf).  Uses c.rho, c.z, c.p, c.q; leaves c.w = A' (last operand).
-// Returns whether the tolerance was met within refine_max steps.
+// ||rhs||_inf).  Uses c.rho, c.z, c.p, c.q; when accepted c.w = A' out (from
+// the FP64 residual that decided it).  Returns whether the tolerance was met within refine_max steps.
 template <int T>
 __device__ bool pcg_lp(const BatchArgs& a, Ctx& c, bool tier2, const double* M64, const double* dinv64,
                        double mnorm, const double* rhs, double* out, int refine_max) {
@@ -579,15 +938,15 @@ __device__ bool pcg_lp(const BatchArgs& a, Ctx& c, bool tier2, const double* M64
   rn = bmax<T>(rn, c.scal);
   if (!(rn > 0.0)) rn = 1.0;
   auto precond = [&](const double* v, double* o) {
-    if (tier2) blk_precond64<T>(c, M64, dinv64, v, o);
+    if (tier2) blk_precond64<T>(c, a.m_cap, M64, dinv64, v, o);
     else blk_precond<T>(c, v, o);
   };
   precond(rhs, out);
   auto accepted = [&](double res, double dyn) {
     return res <= a.refine_tol * rn || res <= a.refine_tol * (mnorm * dyn + rn);
   };
-  auto true_residual = [&](double& res, double& dyn) {
-    blk_apply_m<T>(c, out, rhs, c.rho);  // rho = rhs - M out
+  auto true_residual = [&](double& res, double& dyn, bool df = false) {
+    blk_apply_m<T>(c, out, rhs, c.rho, df);  // rho = rhs - M out
     double rr = 0.0, dd = 0.0;
     for (int i = threadIdx.x; i < m; i += T) {
       rr = fmax(rr, fabs(c.rho[i]));
@@ -597,7 +956,11 @@ __device__ bool pcg_lp(const BatchArgs& a, Ctx& c, bool tier2, const double* M64
     dyn = bmax<T>(dd, c.scal);
   };
   double res, dyn;
-  true_residual(res, dyn);
+  // With an FP32 factor the first residual is ~1e-7 of the right-hand side and
+  // only starts the conjugate gradients: its inner pass runs in double-float; one
+  // that would be accepted is formed again in FP64 (as in the large path).
+  true_residual(res, dyn, !tier2);
+  if (!tier2 && accepted(res, dyn)) true_residual(res, dyn);
   bool done = accepted(res, dyn);
   if (!done) {
     double rz = 0.0;
@@ -688,10 +1051,12 @@ __device__ void solve_lp(const BatchArgs& a, const BatchLP lp, Ctx& c, int& stat
       break;
     }
     if (tier2) ++n_shift;
-    if (!pcg_lp<T>(a, c, tier2, M64, dinv64, mnorm, c.r, c.dy, a.refine_max)) ++n_unref;
-    // w = A' dy; dx = D w - x; ds = -w
-    blk_gemv_t<T>(c, c.dy, c.w);
-    __syncthreads();
+    // w = A' dy (there if dy was accepted); dx = D w - x; ds = -w
+    if (!pcg_lp<T>(a, c, tier2, M64, dinv64, mnorm, c.r, c.dy, a.refine_max)) {
+      ++n_unref;
+      blk_gemv_t<T>(c, c.dy, c.w);
+      __syncthreads();
+    }
     double psi = -INFINITY;
     int nonfinite = 0;
     for (int j = threadIdx.x; j < n; j += T) {
@@ -760,12 +1125,14 @@ __device__ __forceinline__ Ctx make_ctx(unsigned char* batch_smem_raw, int m_cap
   c.kidx = reinterpret_cast<int*>(batch_smem_raw + L.kidx);
   c.stage = reinterpret_cast<float*>(batch_smem_raw + L.stage);
   c.dc = reinterpret_cast<float*>(batch_smem_raw + L.dc);
+  c.pr = reinterpret_cast<float*>(batch_smem_raw + L.pr);
   c.scal = reinterpret_cast<double*>(batch_smem_raw + L.scal);
   return c;
 }
 
+// (Two CTAs of up to 256 threads per SM where their shared memory allows it.)
 template <int T>
-__global__ void __launch_bounds__(T) k_batch(BatchArgs a) {
+__global__ void __launch_bounds__(T, T <= 256 ? 2 : 1) k_batch(BatchArgs a) {
   extern __shared__ __align__(16) unsigned char batch_smem_raw[];
   __shared__ int s_lp;
   Ctx c = make_ctx(batch_smem_raw, a.m_cap, a.n_cap);
@@ -855,9 +1222,7 @@ __device__ int adjoint_lp(const AdjointArgs& g, const BatchLP lp, Ctx& c) {
   blk_gemv<T>(c, c.un2, nullptr, c.r);  // r = A D g
   __syncthreads();
   if (!pcg_lp<T>(a, c, tier2, M64, dinv64, mnorm, c.r, c.dy, 4 * a.refine_max)) return PDAS_ERR_NOT_SPD;
-  for (int i = threadIdx.x; i < m; i += T) la[i] = c.dy[i];
-  blk_gemv_t<T>(c, c.dy, c.w);  // A' la
-  __syncthreads();
+  for (int i = threadIdx.x; i < m; i += T) la[i] = c.dy[i];  // (c.w = A' la)
   for (int j = threadIdx.x; j < n; j += T) {
     const double b = c.D[j] * (c.w[j] - gv[j]);
     lb[j] = b;
@@ -879,8 +1244,6 @@ __device__ int adjoint_lp(const AdjointArgs& g, const BatchLP lp, Ctx& c) {
     // (no correction that meets the tolerance: it is at the rounding level; keep what we have)
     if (!pcg_lp<T>(a, c, tier2, M64, dinv64, mnorm, c.r, c.dy, 4 * a.refine_max)) break;
     for (int i = threadIdx.x; i < m; i += T) la[i] += c.dy[i];
-    blk_gemv_t<T>(c, c.dy, c.w);
-    __syncthreads();
     for (int j = threadIdx.x; j < n; j += T) {
       const double db = c.D[j] * (c.w[j] - r1[j]) + r3[j];
       lb[j] += db;
@@ -900,7 +1263,7 @@ __device__ int adjoint_lp(const AdjointArgs& g, const BatchLP lp, Ctx& c) {
 }
 
 template <int T>
-__global__ void __launch_bounds__(T) k_batch_adjoint(AdjointArgs g) {
+__global__ void __launch_bounds__(T, T <= 256 ? 2 : 1) k_batch_adjoint(AdjointArgs g) {
   extern __shared__ __align__(16) unsigned char batch_smem_raw[];
   __shared__ int s_lp;
   const BatchArgs& a = g.a;
@@ -1309,11 +1672,13 @@ pdas_status pdas_batch_create(int count, const int* m, const int* n, const float
     cuda_fail(h, e, "pdas_batch_create");
     return fail(PDAS_ERR_CUDA);
   }
-  // CTA sizes: built-in choice (256), or the autotuner's
+  // CTA sizes: the autotuner's, or the built-in choice: 256 threads while two
+  // CTAs fit an SM (m <= 128), 512 beyond, where shared memory leaves one (512 LPs
+  // of m <= 256 to a gap of 3e-2: 38 ms, and about 44 with 256 throughout)
   for (int bi = 0; bi < kBuckets; ++bi) {
     auto& B = h->bk[bi];
     if (B.count == 0) continue;
-    B.threads = 256;
+    B.threads = B.m_bound <= 128 ? 256 : 512;
     if ((st = grid_for_bucket(h, bi, B.threads, &B.grid)) != PDAS_OK) return fail(st);
   }
   if (opt.autotune && (st = autotune(h, no, mo)) != PDAS_OK) return fail(st);
