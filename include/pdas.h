@@ -116,7 +116,9 @@ typedef struct {
                               factor's trailing updates run on the tensor cores from digit
                               planes of each panel (FP64-grade at every gap);
                               0 = double-float formation (normal_form 2) and the factors of
-                              df_factor_floor                                                 (1) */
+                              df_factor_floor.  PDAS_FP64: 1 = the factor of (b) at every m (a
+                              matrix that it finds not positive definite is factored again on the
+                              SIMT pipes); 0 = the SIMT factor                                 (1) */
   double df_factor_floor;  /* mixed forms in the FP64 tier without the tensor-core factor: the
                               factor is the double-float tile factor (FP32 pipes) while the
                               relative gap of the iterate is above this, the FP64 SIMT factor

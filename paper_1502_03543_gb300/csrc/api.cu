@@ -88,6 +88,7 @@ struct pdas_ctx {
   int switch_reason = 0;  // pdas_iter_info.fp64_reason of that switch
   bool last_factor_df = false;    // the last factor was a fast FP64-tier factor (tensor-core or double-float)
   double last_rel_gap = HUGE_VAL;  // relative gap of the iterate after the last step
+  bool plain_simt = false;        // plain FP64 form: this call is a retry with the SIMT factor
   bool no_dffactor_once = false;  // this iteration: that factor failed, use the FP64 factor
   int64_t err_index = -1;
   char errmsg[256] = {0};
@@ -396,8 +397,8 @@ pdas_status form_normal(pdas_ctx* h, const void* A) {
 // the gap-1e-8 run of the 8192 x 32768 problem from 54 iterations to 80.
 pdas_status factor(pdas_ctx* h) {
   h->last_factor_df = false;
-  if (h->cur_f64 && is_mixed(h) && h->cdig.planes && !h->no_dffactor_once) {
-    // FP64 tier with fp64_tier_tc: the FP64 factor whose trailing updates run
+  if (h->cur_f64 && h->cdig.m > 0 && !h->no_dffactor_once) {
+    // The plain FP64 form and the FP64 tier with fp64_tier_tc: the FP64 factor whose trailing updates run
     // on the tensor cores from exact digit planes (FP64-grade at every gap);
     // on a failed pivot the next attempt uses the FP64 SIMT factor
     h->last_factor_df = true;
@@ -599,7 +600,7 @@ pdas_status direction(pdas_ctx* h, const void* A, const double* x, const double*
   }
   h->no_drop_once = false;
   h->no_df_once = false;
-  h->no_dffactor_once = false;
+  h->no_dffactor_once = h->plain_simt;
   for (int attempt = 0; attempt < 5; ++attempt) {
     STAGE(h, PDAS_STAGE_NORMAL);
     if ((st = form_normal(h, A)) != PDAS_OK) return st;
@@ -686,6 +687,54 @@ void fill_info(pdas_ctx* h, pdas_iter_info* info, bool stepped) {
       info->dres = s.dres;
     }
   }
+}
+
+// The plain FP64 form reads the device's status only at the end of a call:
+// where the factor with tensor-core updates met a pivot that is not positive,
+// the call is done over with the SIMT factor (nothing of the caller's has been
+// touched), so that a matrix at the edge is judged as by that factor.
+bool retry_simt(pdas_ctx* h, pdas_status st) {
+  if (st != PDAS_ERR_NOT_SPD || is_mixed(h) || h->last_factor_form != 4) return false;
+  h->plain_simt = true;
+  return true;
+}
+
+// One step in place, up to the device's status; *read: it was read.
+pdas_status step_once(pdas_ctx* h, const void* A, const double* b, const double* c, double* x, double* y, double* s,
+                      double alpha, const Infeasible* iv, bool* read) {
+  *read = false;
+  pdas_status st = direction(h, A, x, s, iv);
+  if (st != PDAS_OK) return st;
+  STAGE(h, PDAS_STAGE_STEP);
+  KL(launch_psi(h->st, h->n, x, s, h->dx, h->ds, alpha, h->part, h->tickets, h->sc, iv != nullptr), 1);
+  KL(launch_step(h->st, h->m, h->n, b, c, x, y, s, h->dx, h->dy, h->ds, h->part, h->tickets, h->sc), 1);
+  if (iv) {  // residuals of the new iterate: b - A x and c - A'y - s
+    if ((st = gemv(h, A, x, b, h->rho, -1)) != PDAS_OK) return st;
+    if ((st = gemv_t(h, A, y, 0, nullptr, h->w, nullptr, nullptr)) != PDAS_OK) return st;
+    KL(launch_residual_norms(h->st, h->m, h->n, b, h->rho, c, h->w, s, h->part, h->tickets, h->sc), 1);
+  }
+  STAGE_END(h);
+  if ((st = read_scalars(h)) != PDAS_OK) return st;
+  *read = true;
+  return device_status(h);
+}
+
+// Newton direction to the caller's arrays, synchronous.
+pdas_status direction_out(pdas_ctx* h, const void* A, const double* x, const double* s, const Infeasible* iv, double* dx,
+                          double* dy, double* ds, pdas_iter_info* info) {
+  pdas_status st;
+  do {
+    h->err_index = -1;
+    if ((st = direction(h, A, x, s, iv)) != PDAS_OK) break;
+    CK(cudaMemcpyAsync(dx, h->dx, sizeof(double) * h->n, cudaMemcpyDeviceToDevice, h->st));
+    CK(cudaMemcpyAsync(ds, h->ds, sizeof(double) * h->n, cudaMemcpyDeviceToDevice, h->st));
+    CK(cudaMemcpyAsync(dy, h->dy, sizeof(double) * h->m, cudaMemcpyDeviceToDevice, h->st));
+    if ((st = read_scalars(h)) != PDAS_OK) break;
+    st = device_status(h);
+    fill_info(h, info, false);
+  } while (retry_simt(h, st));
+  h->plain_simt = false;
+  return st;
 }
 
 }  // namespace
@@ -862,7 +911,7 @@ pdas_status pdas_create(int64_t m, int64_t n, const pdas_options* opt_in, pdas_h
   }
   if (e == cudaSuccess && opt.form != PDAS_FP64 && opt.a_dtype == PDAS_A_BF16 && opt.fp64_tier_tc)
     e = dig_workspace_create(&h->dig, m, n);
-  if (e == cudaSuccess && opt.form != PDAS_FP64 && opt.fp64_tier_tc && m > kCholDigMinM)
+  if (e == cudaSuccess && opt.fp64_tier_tc && (opt.form == PDAS_FP64 || m > kCholDigMinM))
     e = chol_dig_create(&h->cdig, m);
   if (e == cudaSuccess && (opt.form == PDAS_BF16_IR || opt.form == PDAS_TF32_IR)) {
     e = tc_workspace_create(&h->tc, opt.form, opt.a_dtype, opt.splits, m, n);
@@ -943,16 +992,7 @@ pdas_status pdas_profile_read(pdas_handle h, pdas_profile* out) {
 pdas_status pdas_direction(pdas_handle h, const void* A, const double* x, const double* s, double* dx, double* dy,
                            double* ds, pdas_iter_info* info) {
   if (!h || check_vec_args(A, x, s) != PDAS_OK || !dx || !dy || !ds) return PDAS_ERR_ARG;
-  h->err_index = -1;
-  pdas_status st = direction(h, A, x, s);
-  if (st != PDAS_OK) return st;
-  CK(cudaMemcpyAsync(dx, h->dx, sizeof(double) * h->n, cudaMemcpyDeviceToDevice, h->st));
-  CK(cudaMemcpyAsync(ds, h->ds, sizeof(double) * h->n, cudaMemcpyDeviceToDevice, h->st));
-  CK(cudaMemcpyAsync(dy, h->dy, sizeof(double) * h->m, cudaMemcpyDeviceToDevice, h->st));
-  if ((st = read_scalars(h)) != PDAS_OK) return st;
-  st = device_status(h);
-  fill_info(h, info, false);
-  return st;
+  return direction_out(h, A, x, s, nullptr, dx, dy, ds, info);
 }
 
 pdas_status pdas_direction_infeasible(pdas_handle h, const void* A, const double* b, const double* c,
@@ -960,40 +1000,24 @@ pdas_status pdas_direction_infeasible(pdas_handle h, const void* A, const double
                                       double* ds, pdas_iter_info* info) {
   if (!h || check_vec_args(A, x, s) != PDAS_OK || !b || !c || !y || !dx || !dy || !ds) return PDAS_ERR_ARG;
   if (!h->opt.infeasible) return PDAS_ERR_ARG;
-  h->err_index = -1;
   const Infeasible iv{y, b, c};
-  pdas_status st = direction(h, A, x, s, &iv);
-  if (st != PDAS_OK) return st;
-  CK(cudaMemcpyAsync(dx, h->dx, sizeof(double) * h->n, cudaMemcpyDeviceToDevice, h->st));
-  CK(cudaMemcpyAsync(ds, h->ds, sizeof(double) * h->n, cudaMemcpyDeviceToDevice, h->st));
-  CK(cudaMemcpyAsync(dy, h->dy, sizeof(double) * h->m, cudaMemcpyDeviceToDevice, h->st));
-  if ((st = read_scalars(h)) != PDAS_OK) return st;
-  st = device_status(h);
-  fill_info(h, info, false);
-  return st;
+  return direction_out(h, A, x, s, &iv, dx, dy, ds, info);
 }
 
 pdas_status pdas_step(pdas_handle h, const void* A, const double* b, const double* c, double* x, double* y,
                       double* s, double alpha, pdas_iter_info* info) {
   if (!h || check_vec_args(A, x, s) != PDAS_OK || !b || !c || !y) return PDAS_ERR_ARG;
   if (!(alpha > 0.0 && alpha < 1.0)) return PDAS_ERR_ARG;
-  h->err_index = -1;
   const bool variant = h->opt.infeasible != 0;
   const Infeasible iv{y, b, c};
-  pdas_status st = direction(h, A, x, s, variant ? &iv : nullptr);
-  if (st != PDAS_OK) return st;
-  STAGE(h, PDAS_STAGE_STEP);
-  KL(launch_psi(h->st, h->n, x, s, h->dx, h->ds, alpha, h->part, h->tickets, h->sc, variant), 1);
-  KL(launch_step(h->st, h->m, h->n, b, c, x, y, s, h->dx, h->dy, h->ds, h->part, h->tickets, h->sc), 1);
-  if (variant) {  // residuals of the new iterate: b - A x and c - A'y - s
-    if ((st = gemv(h, A, x, b, h->rho, -1)) != PDAS_OK) return st;
-    if ((st = gemv_t(h, A, y, 0, nullptr, h->w, nullptr, nullptr)) != PDAS_OK) return st;
-    KL(launch_residual_norms(h->st, h->m, h->n, b, h->rho, c, h->w, s, h->part, h->tickets, h->sc), 1);
-  }
-  STAGE_END(h);
-  if ((st = read_scalars(h)) != PDAS_OK) return st;
-  st = device_status(h);
-  fill_info(h, info, st == PDAS_OK);
+  pdas_status st;
+  bool read = false;
+  do {
+    h->err_index = -1;
+    st = step_once(h, A, b, c, x, y, s, alpha, variant ? &iv : nullptr, &read);
+  } while (retry_simt(h, st));
+  h->plain_simt = false;
+  if (read) fill_info(h, info, st == PDAS_OK);
   if (st != PDAS_OK) return st;
   h->last_rel_gap = variant ? fmax(fabs(h->sc_host->rel_gap), fmax(h->sc_host->pres, h->sc_host->dres))
                             : h->sc_host->rel_gap;

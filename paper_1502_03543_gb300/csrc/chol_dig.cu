@@ -779,6 +779,7 @@ cudaError_t chol_dig_create(CholDigWorkspace* w, int64_t m) {
   if (ea == cudaSuccess) ea = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (ea != cudaSuccess) return ea;
   w->sub_partitions = 4 * sms;
+  if (m <= UK) return cudaSuccess;  // one diagonal block: no panel, no planes
   CholDigHost* hs = new (std::nothrow) CholDigHost();
   if (!hs) return cudaErrorMemoryAllocation;
   w->host = hs;

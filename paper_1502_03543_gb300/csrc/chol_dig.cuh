@@ -7,12 +7,13 @@
 
 namespace pdas {
 
-// Smallest m whose FP64 tier takes this factor (below it the FP64 factor's
-// SIMT updates are small and the double-float tile factor is as fast).
+// Smallest m whose FP64 tier takes this factor (below it the double-float tile
+// factor is as fast).  The plain FP64 form takes it at every m: against the
+// SIMT factor 52 to 96 us at m = 64, 1.15 to 5.96 ms at m = 1000.
 constexpr int64_t kCholDigMinM = 256;
 
 struct CholDigWorkspace {
-  int64_t m = 0;
+  int64_t m = 0;           // 0: not created
   int64_t mpad = 0;        // m rounded up to 128
   int sub_partitions = 0;  // SM sub-partitions of the device (4 per SM): the row solve's launch shape
   void* planes = nullptr;  // 7 BF16 digit planes of mpad rows x 64 columns (the current panel)
