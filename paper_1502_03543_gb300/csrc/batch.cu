@@ -937,76 +937,69 @@ __device__ bool pcg_lp(const BatchArgs& a, Ctx& c, bool tier2, const double* M64
   for (int i = threadIdx.x; i < m; i += T) rn = fmax(rn, fabs(rhs[i]));
   rn = bmax<T>(rn, c.scal);
   if (!(rn > 0.0)) rn = 1.0;
-  auto precond = [&](const double* v, double* o) {
-    if (tier2) blk_precond64<T>(c, a.m_cap, M64, dinv64, v, o);
-    else blk_precond<T>(c, v, o);
-  };
-  precond(rhs, out);
   auto accepted = [&](double res, double dyn) {
     return res <= a.refine_tol * rn || res <= a.refine_tol * (mnorm * dyn + rn);
   };
-  auto true_residual = [&](double& res, double& dyn, bool df = false) {
-    blk_apply_m<T>(c, out, rhs, c.rho, df);  // rho = rhs - M out
-    double rr = 0.0, dd = 0.0;
-    for (int i = threadIdx.x; i < m; i += T) {
-      rr = fmax(rr, fabs(c.rho[i]));
-      dd = fmax(dd, fabs(out[i]));
+  // One loop, so that each solve and each product is compiled once: a round
+  // applies the preconditioner (but for kTrue), then M to a vector.
+  //   kFirst    out = P^-1 rhs, rho = rhs - M out.  With an FP32 factor this
+  //             residual is ~1e-7 of rhs and only starts the conjugate gradients:
+  //             its inner pass runs in double-float, and one that would be
+  //             accepted is formed again in FP64 (as in the large path)
+  //   kTrue     rho = rhs - M out in FP64, which decides acceptance
+  //   kRestart  z = P^-1 rho, p = z, then the step
+  //   kStep     z = P^-1 rho, p = z + beta p, then the step
+  enum { kFirst, kTrue, kRestart, kStep } state = kFirst;
+  double rz = 0.0;
+  for (int k = 0;;) {
+    if (state != kTrue) {
+      const double* v = state == kFirst ? rhs : c.rho;
+      double* o = state == kFirst ? out : c.z;
+      if (tier2) blk_precond64<T>(c, a.m_cap, M64, dinv64, v, o);
+      else blk_precond<T>(c, v, o);
     }
-    res = bmax<T>(rr, c.scal);
-    dyn = bmax<T>(dd, c.scal);
-  };
-  double res, dyn;
-  // With an FP32 factor the first residual is ~1e-7 of the right-hand side and
-  // only starts the conjugate gradients: its inner pass runs in double-float; one
-  // that would be accepted is formed again in FP64 (as in the large path).
-  true_residual(res, dyn, !tier2);
-  if (!tier2 && accepted(res, dyn)) true_residual(res, dyn);
-  bool done = accepted(res, dyn);
-  if (!done) {
-    double rz = 0.0;
-    auto restart = [&]() {
-      precond(c.rho, c.z);
+    const bool step = state == kRestart || state == kStep;
+    if (step) {
       double t = 0.0;
-      for (int i = threadIdx.x; i < m; i += T) {
-        c.p[i] = c.z[i];
-        t += c.rho[i] * c.z[i];
-      }
-      rz = bsum<T>(t, c.scal);
-    };
-    restart();
-    for (int k = 0; k < refine_max && rz > 0.0 && isfinite(rz); ++k) {
-      blk_apply_m<T>(c, c.p, nullptr, c.q, !tier2);
+      for (int i = threadIdx.x; i < m; i += T) t += c.rho[i] * c.z[i];
+      const double rz2 = bsum<T>(t, c.scal);
+      const double beta = state == kStep ? rz2 / rz : 0.0;
+      for (int i = threadIdx.x; i < m; i += T) c.p[i] = state == kStep ? c.z[i] + beta * c.p[i] : c.z[i];
+      __syncthreads();
+      rz = rz2;
+      if (!(k < refine_max && rz > 0.0 && isfinite(rz))) return false;
+    }
+    const bool df = state != kTrue && !tier2;
+    blk_apply_m<T>(c, step ? c.p : out, step ? nullptr : rhs, step ? c.q : c.rho, df);
+    double al = 0.0;
+    if (step) {
       double t = 0.0;
       for (int i = threadIdx.x; i < m; i += T) t += c.p[i] * c.q[i];
       const double pq = bsum<T>(t, c.scal);
-      if (!(pq > 0.0)) break;
-      const double al = rz / pq;
-      double rr = 0.0, dd = 0.0;
-      for (int i = threadIdx.x; i < m; i += T) {
+      if (!(pq > 0.0)) return false;
+      al = rz / pq;
+    }
+    double rr = 0.0, dd = 0.0;
+    for (int i = threadIdx.x; i < m; i += T) {
+      if (step) {
         out[i] += al * c.p[i];
         c.rho[i] -= al * c.q[i];
-        rr = fmax(rr, fabs(c.rho[i]));
-        dd = fmax(dd, fabs(out[i]));
       }
-      res = bmax<T>(rr, c.scal);
-      dyn = bmax<T>(dd, c.scal);
-      if (accepted(res, dyn) || k % 10 == 9) {
-        true_residual(res, dyn);
-        if ((done = accepted(res, dyn))) break;
-        restart();
-        continue;
-      }
-      precond(c.rho, c.z);
-      t = 0.0;
-      for (int i = threadIdx.x; i < m; i += T) t += c.rho[i] * c.z[i];
-      const double rz2 = bsum<T>(t, c.scal);
-      const double beta = rz2 / rz;
-      for (int i = threadIdx.x; i < m; i += T) c.p[i] = c.z[i] + beta * c.p[i];
-      __syncthreads();
-      rz = rz2;
+      rr = fmax(rr, fabs(c.rho[i]));
+      dd = fmax(dd, fabs(out[i]));
+    }
+    const double res = bmax<T>(rr, c.scal);
+    const double dyn = bmax<T>(dd, c.scal);
+    if (step) {
+      state = accepted(res, dyn) || k % 10 == 9 ? kTrue : kStep;
+      ++k;
+    } else if (accepted(res, dyn)) {
+      if (!df) return true;
+      state = kTrue;
+    } else {
+      state = kRestart;
     }
   }
-  return done;
 }
 
 // The whole PDAS loop of one LP; returns its status, iterations and gap.
@@ -1219,36 +1212,40 @@ __device__ int adjoint_lp(const AdjointArgs& g, const BatchLP lp, Ctx& c) {
   bool tier2 = false;
   double mnorm = 0.0;
   if (!factor_lp<T>(a, c, tier2, M64, dinv64, mnorm)) return PDAS_ERR_NOT_SPD;
-  blk_gemv<T>(c, c.un2, nullptr, c.r);  // r = A D g
-  __syncthreads();
-  if (!pcg_lp<T>(a, c, tier2, M64, dinv64, mnorm, c.r, c.dy, 4 * a.refine_max)) return PDAS_ERR_NOT_SPD;
-  for (int i = threadIdx.x; i < m; i += T) la[i] = c.dy[i];  // (c.w = A' la)
-  for (int j = threadIdx.x; j < n; j += T) {
-    const double b = c.D[j] * (c.w[j] - gv[j]);
-    lb[j] = b;
-    lc[j] = -b / x[j];
-    wt[j] = c.w[j];
-  }
-  __syncthreads();
-  for (int it = 0; it < 2; ++it) {
-    for (int j = threadIdx.x; j < n; j += T) {
-      const double e1 = gv[j] - wt[j] - s[j] * lc[j];
-      const double e3 = -lb[j] - x[j] * lc[j];
-      r1[j] = e1;
-      r3[j] = e3;
-      c.un2[j] = df_split(c.D[j] * e1 - e3 - lb[j]);
+  for (int it = 0; it < 3; ++it) {  // the solve, then two corrections
+    if (it > 0) {
+      for (int j = threadIdx.x; j < n; j += T) {
+        const double e1 = gv[j] - wt[j] - s[j] * lc[j];
+        const double e3 = -lb[j] - x[j] * lc[j];
+        r1[j] = e1;
+        r3[j] = e3;
+        c.un2[j] = df_split(c.D[j] * e1 - e3 - lb[j]);
+      }
+      __syncthreads();
     }
+    blk_gemv<T>(c, c.un2, nullptr, c.r);  // r = A D g, then A (D r1 - r3 - lb)
     __syncthreads();
-    blk_gemv<T>(c, c.un2, nullptr, c.r);  // r = A (D r1 - r3 - lb)
-    __syncthreads();
-    // (no correction that meets the tolerance: it is at the rounding level; keep what we have)
-    if (!pcg_lp<T>(a, c, tier2, M64, dinv64, mnorm, c.r, c.dy, 4 * a.refine_max)) break;
-    for (int i = threadIdx.x; i < m; i += T) la[i] += c.dy[i];
-    for (int j = threadIdx.x; j < n; j += T) {
-      const double db = c.D[j] * (c.w[j] - r1[j]) + r3[j];
-      lb[j] += db;
-      lc[j] += (r3[j] - db) / x[j];
-      wt[j] += c.w[j];
+    if (!pcg_lp<T>(a, c, tier2, M64, dinv64, mnorm, c.r, c.dy, 4 * a.refine_max)) {
+      if (it == 0) return PDAS_ERR_NOT_SPD;
+      break;  // (no correction that meets the tolerance: it is at the rounding level; keep what we have)
+    }
+    // (c.w = A' dy)
+    if (it == 0) {
+      for (int i = threadIdx.x; i < m; i += T) la[i] = c.dy[i];
+      for (int j = threadIdx.x; j < n; j += T) {
+        const double b = c.D[j] * (c.w[j] - gv[j]);
+        lb[j] = b;
+        lc[j] = -b / x[j];
+        wt[j] = c.w[j];
+      }
+    } else {
+      for (int i = threadIdx.x; i < m; i += T) la[i] += c.dy[i];
+      for (int j = threadIdx.x; j < n; j += T) {
+        const double db = c.D[j] * (c.w[j] - r1[j]) + r3[j];
+        lb[j] += db;
+        lc[j] += (r3[j] - db) / x[j];
+        wt[j] += c.w[j];
+      }
     }
     __syncthreads();
   }
