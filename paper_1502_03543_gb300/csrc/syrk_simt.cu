@@ -129,19 +129,43 @@ __global__ void __launch_bounds__(kThreads) k_syrk_fp64(int64_t m, int64_t n, co
 // FP64, and A itself, m x ldk FP32 each, so that the product loads 16 bytes
 // whatever the alignment of A's rows.  The planes hold columns c0 .. c0 + ldk - 1
 // (zero past column n); only where both would exceed 4 GB is that not all of A.
+// An FP64 product and two conversions per element hold the FP64 pipe for most of
+// the pass (31 us at 1001 x 3003), so where A is exact in FP32 the product is
+// formed from D as an FP32 pair, a dh + (a dl + the exact error of a dh), which
+// rounds as the FP64 product does but for ties 2^-24 apart; D outside
+// 2^(-100 .. 100) keeps the FP64 product.  A block takes 16 rows of 256 columns.
+constexpr int kPlaneRows = 16;
 template <typename T>
 __global__ void __launch_bounds__(kThreads) k_simt_planes(int64_t m, int64_t n, int64_t c0, int64_t ldk,
                                                           const T* __restrict__ A, const double* __restrict__ D,
                                                           float* __restrict__ Bp, float* __restrict__ Ap,
                                                           const Scalars* sc) {
   if (*(volatile const int*)&sc->status != 0) return;
-  for (int64_t p = blockIdx.y; p < m; p += gridDim.y)
-    for (int64_t k = blockIdx.x * (int64_t)kThreads + threadIdx.x; k < ldk; k += (int64_t)gridDim.x * kThreads) {
-      const bool in = c0 + k < n;
+  const int64_t k = blockIdx.x * (int64_t)kThreads + threadIdx.x;
+  if (k >= ldk) return;
+  const bool in = c0 + k < n;
+  const double d = in ? __ldg(D + c0 + k) : 0.0;
+  const float dh = (float)d, dl = (float)(d - (double)dh);
+  const bool pair = sizeof(T) < 8 && fabs(d) < 0x1p100 && (fabs(d) > 0x1p-100 || d == 0.0);
+  for (int64_t p0 = (int64_t)blockIdx.y * kPlaneRows; p0 < m; p0 += (int64_t)gridDim.y * kPlaneRows) {
+#pragma unroll 8
+    for (int r = 0; r < kPlaneRows; ++r) {
+      const int64_t p = p0 + r;
+      if (p >= m) break;
       const T a = in ? A[p * n + c0 + k] : T(0.f);
-      Bp[p * ldk + k] = in ? (float)(widen(a) * __ldg(D + c0 + k)) : 0.f;
-      Ap[p * ldk + k] = widen32(a);
+      const float af = widen32(a);
+      float b;
+      if (pair) {
+        const float h = af * dh;
+        b = h + fmaf(af, dl, fmaf(af, dh, -h));
+        if (!isfinite(h)) b = h;
+      } else {
+        b = (float)(widen(a) * d);
+      }
+      Bp[p * ldk + k] = b;
+      Ap[p * ldk + k] = af;
     }
+  }
 }
 
 // M = B A' on 128 x 128 tiles, 8 x 8 outputs per thread, K chunks of 16 in two
@@ -149,7 +173,7 @@ __global__ void __launch_bounds__(kThreads) k_simt_planes(int64_t m, int64_t n, 
 // Thread (tx, ty) owns rows 4 ty .. + 3 and 64 + 4 ty .. + 3 and the same of
 // columns by tx, so a step reads four 16-byte vectors for 64 multiply-adds.
 // Bound by the FP32 pipe.  Measured at 1001 x 3003 (36 tiles): 774 us as 36 CTAs
-// with the FP64 products in the loads -> 127 us with the planes and 8 K slices
+// with the FP64 products in the loads -> 120 us with the planes and 8 K slices
 // (288 CTAs; the multiply-adds alone take 46 us).
 constexpr int kPitch = kBig + 4;
 
@@ -311,7 +335,8 @@ cudaError_t launch_syrk_fp32(cudaStream_t st, int64_t m, int64_t n, const T* A, 
                              float* M, int64_t ldm, void* part, unsigned* tickets, const Scalars* sc, int* launches) {
   const SimtPlan p = simt_plan_fp32(m, n);
   float* Ap = planes + m * p.ldk;
-  const dim3 pg((unsigned)std::min<int64_t>((p.ldk + kThreads - 1) / kThreads, 64), (unsigned)std::min<int64_t>(m, 4096));
+  const dim3 pg((unsigned)((p.ldk + kThreads - 1) / kThreads),
+                (unsigned)std::min<int64_t>((m + kPlaneRows - 1) / kPlaneRows, 4096));
   const dim3 grid((unsigned)p.tiles, (unsigned)p.slices);
   for (int64_t c0 = 0; c0 < n; c0 += p.ldk) {
     k_simt_planes<T><<<pg, kThreads, 0, st>>>(m, n, c0, p.ldk, A, D, planes, Ap, sc);
