@@ -414,8 +414,7 @@ pdas_status factor(pdas_ctx* h) {
     // while the iterate is not yet close to the optimum
     h->last_factor_df = true;
     h->last_factor_form = 2;
-    KL(cholesky_tiles_df(h->st, h->m, h->ldm, h->M64, h->dinv64, h->chol_tasks, h->chol_ntasks, h->chol_state,
-                         h->tickets + T_CHOL, h->sc),
+    KL(cholesky_tiles_df(h->st, h->m, h->ldm, h->M64, h->dinv64, h->chol_tasks, h->chol_ntasks, h->chol_state, h->sc),
        4);
   } else if (h->cur_f64) {
     h->last_factor_form = 3;
@@ -426,7 +425,7 @@ pdas_status factor(pdas_ctx* h) {
   } else {
     h->last_factor_form = 0;
     KL(cholesky_tiles<float>(h->st, h->m, h->ldm, h->M32, h->dinv32, h->uinv32, h->chol_tasks, h->chol_ntasks,
-                             h->chol_state, h->tickets + T_CHOL, h->sc, h->chol_planes),
+                             h->chol_state, h->sc, h->chol_planes),
        1);
   }
   return PDAS_OK;
@@ -447,15 +446,15 @@ pdas_status factor_solve(pdas_ctx* h, double* rhs, double* out, const CgStep* up
   }
   if (upd) KL(launch_cg_update(h->st, h->m, *upd, rhs, h->part, h->tickets, h->sc), 1);
   if (h->cur_f64) {
-    KL(trsv_lower<double>(h->st, h->m, h->ldm, h->M64, h->dinv64, rhs, h->z, h->flags, h->tickets, h->sc,
+    KL(trsv_lower<double>(h->st, h->m, h->ldm, h->M64, h->dinv64, rhs, h->z, h->flags, h->sc,
                           is_mixed(h)),
        1);
-    KL(trsv_upper_t<double>(h->st, h->m, h->ldm, h->M64, h->dinv64, h->z, out, h->flags, h->tickets, h->sc,
+    KL(trsv_upper_t<double>(h->st, h->m, h->ldm, h->M64, h->dinv64, h->z, out, h->flags, h->sc,
                             is_mixed(h)),
        1);
   } else {
-    KL(trsv_lower<float>(h->st, h->m, h->ldm, h->M32, h->dinv32, rhs, h->z, h->flags, h->tickets, h->sc, true), 1);
-    KL(trsv_upper_t<float>(h->st, h->m, h->ldm, h->M32, h->dinv32, h->z, out, h->flags, h->tickets, h->sc, true),
+    KL(trsv_lower<float>(h->st, h->m, h->ldm, h->M32, h->dinv32, rhs, h->z, h->flags, h->sc, true), 1);
+    KL(trsv_upper_t<float>(h->st, h->m, h->ldm, h->M32, h->dinv32, h->z, out, h->flags, h->sc, true),
        1);
   }
   if (nrz) {
@@ -903,7 +902,7 @@ pdas_status pdas_create(int64_t m, int64_t n, const pdas_options* opt_in, pdas_h
     al((void**)&h->chol_tasks, sizeof(int4) * tasks.size());
     al((void**)&h->zb, sizeof(double) * m);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->zb, 0xff, sizeof(double) * m, h->st);
-    al((void**)&h->chol_state, sizeof(int) * (nb * nb + nb));
+    al((void**)&h->chol_state, sizeof(int) * (nb * nb + nb + 1));
     al((void**)&h->uinv32, sizeof(float) * nb * kCholTile * kCholTile);
     if (nb > 1) al((void**)&h->chol_planes, (size_t)chol_plane_bytes(m));
     if (e == cudaSuccess)

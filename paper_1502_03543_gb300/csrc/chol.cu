@@ -447,41 +447,41 @@ cudaError_t cholesky(cudaStream_t st, int64_t m, int64_t ldm, T* M, T* dinv, Sca
 
 template <typename T>
 cudaError_t trsv_lower(cudaStream_t st, int64_t m, int64_t ldm, const T* L, const T* dinv, const double* v, double* z,
-                       int* flags, unsigned* tickets, Scalars* sc, bool scaled) {
+                       int* flags, Scalars* sc, bool scaled) {
   const int64_t nblk = (m + kTile - 1) / kTile;
-  cudaError_t e = cudaMemsetAsync(flags, 0, sizeof(int) * nblk, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(tickets + T_TRSV, 0, sizeof(unsigned), st);
+  unsigned* ticket = reinterpret_cast<unsigned*>(flags + nblk);  // (cleared with the flags)
+  const cudaError_t e = cudaMemsetAsync(flags, 0, sizeof(int) * (nblk + 1), st);
   if (e != cudaSuccess) return e;
   if (scaled)
-    k_trsv_lower<T, true><<<(unsigned)nblk, kThreads, 0, st>>>(m, ldm, L, dinv, v, z, flags, tickets + T_TRSV, sc);
+    k_trsv_lower<T, true><<<(unsigned)nblk, kThreads, 0, st>>>(m, ldm, L, dinv, v, z, flags, ticket, sc);
   else
-    k_trsv_lower<T, false><<<(unsigned)nblk, kThreads, 0, st>>>(m, ldm, L, dinv, v, z, flags, tickets + T_TRSV, sc);
+    k_trsv_lower<T, false><<<(unsigned)nblk, kThreads, 0, st>>>(m, ldm, L, dinv, v, z, flags, ticket, sc);
   return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t trsv_upper_t(cudaStream_t st, int64_t m, int64_t ldm, const T* L, const T* dinv, const double* z,
-                         double* y, int* flags, unsigned* tickets, Scalars* sc, bool scaled) {
+                         double* y, int* flags, Scalars* sc, bool scaled) {
   const int64_t nblk = (m + kTile - 1) / kTile;
-  cudaError_t e = cudaMemsetAsync(flags, 0, sizeof(int) * nblk, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(tickets + T_TRSV, 0, sizeof(unsigned), st);
+  unsigned* ticket = reinterpret_cast<unsigned*>(flags + nblk);  // (cleared with the flags)
+  const cudaError_t e = cudaMemsetAsync(flags, 0, sizeof(int) * (nblk + 1), st);
   if (e != cudaSuccess) return e;
   if (scaled)
-    k_trsv_upper_t<T, true><<<(unsigned)nblk, kThreads, 0, st>>>(m, ldm, L, dinv, z, y, flags, tickets + T_TRSV, sc);
+    k_trsv_upper_t<T, true><<<(unsigned)nblk, kThreads, 0, st>>>(m, ldm, L, dinv, z, y, flags, ticket, sc);
   else
-    k_trsv_upper_t<T, false><<<(unsigned)nblk, kThreads, 0, st>>>(m, ldm, L, dinv, z, y, flags, tickets + T_TRSV, sc);
+    k_trsv_upper_t<T, false><<<(unsigned)nblk, kThreads, 0, st>>>(m, ldm, L, dinv, z, y, flags, ticket, sc);
   return cudaGetLastError();
 }
 
 template cudaError_t cholesky<double>(cudaStream_t, int64_t, int64_t, double*, double*, Scalars*);
 template cudaError_t cholesky<float>(cudaStream_t, int64_t, int64_t, float*, float*, Scalars*);
 template cudaError_t trsv_lower<double>(cudaStream_t, int64_t, int64_t, const double*, const double*, const double*,
-                                        double*, int*, unsigned*, Scalars*, bool);
+                                        double*, int*, Scalars*, bool);
 template cudaError_t trsv_lower<float>(cudaStream_t, int64_t, int64_t, const float*, const float*, const double*,
-                                       double*, int*, unsigned*, Scalars*, bool);
+                                       double*, int*, Scalars*, bool);
 template cudaError_t trsv_upper_t<double>(cudaStream_t, int64_t, int64_t, const double*, const double*, const double*,
-                                          double*, int*, unsigned*, Scalars*, bool);
+                                          double*, int*, Scalars*, bool);
 template cudaError_t trsv_upper_t<float>(cudaStream_t, int64_t, int64_t, const float*, const float*, const double*,
-                                         double*, int*, unsigned*, Scalars*, bool);
+                                         double*, int*, Scalars*, bool);
 
 }  // namespace pdas

@@ -1231,7 +1231,7 @@ void chol_tile_tasks(int64_t m, int nproc, std::vector<int4>* out) {
 
 template <typename T>
 cudaError_t cholesky_tiles(cudaStream_t st, int64_t m, int64_t ldm, T* M, T* dinv, T* Uinv, const int4* tasks,
-                           int ntasks, int* state, unsigned* ticket, Scalars* sc, unsigned char* planes) {
+                           int ntasks, int* state, Scalars* sc, unsigned char* planes) {
   if (sizeof(T) == 4 && !planes && chol_tile_count(m) > 1) return cudaErrorInvalidValue;
   static int per_sm = 0;  // resident CTAs per SM (per process; the attribute is per function)
   if (per_sm == 0) {
@@ -1248,8 +1248,8 @@ cudaError_t cholesky_tiles(cudaStream_t st, int64_t m, int64_t ldm, T* M, T* din
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
   const int nb = (int)chol_tile_count(m);
-  e = cudaMemsetAsync(state, 0, sizeof(int) * (size_t)(nb * nb + nb), st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(ticket, 0, sizeof(unsigned), st);
+  unsigned* ticket = reinterpret_cast<unsigned*>(state + (int64_t)nb * nb + nb);
+  e = cudaMemsetAsync(state, 0, sizeof(int) * ((size_t)nb * nb + nb + 1), st);
   if (e != cudaSuccess) return e;
   int grid = sms * per_sm;  // (at least 3: blocks 0 and, in FP32, 1 run only the diagonal tasks)
   if (grid > ntasks + 1) grid = ntasks + 1;
@@ -1260,9 +1260,9 @@ cudaError_t cholesky_tiles(cudaStream_t st, int64_t m, int64_t ldm, T* M, T* din
 }
 
 template cudaError_t cholesky_tiles<float>(cudaStream_t, int64_t, int64_t, float*, float*, float*, const int4*, int,
-                                           int*, unsigned*, Scalars*, unsigned char*);
+                                           int*, Scalars*, unsigned char*);
 template cudaError_t cholesky_tiles<dfloat>(cudaStream_t, int64_t, int64_t, dfloat*, dfloat*, dfloat*, const int4*,
-                                            int, int*, unsigned*, Scalars*, unsigned char*);
+                                            int, int*, Scalars*, unsigned char*);
 
 namespace {
 
@@ -1293,13 +1293,13 @@ __global__ void k_df_to_double(int64_t n, double* v) {
 }  // namespace
 
 cudaError_t cholesky_tiles_df(cudaStream_t st, int64_t m, int64_t ldm, double* M, double* dinv, const int4* tasks,
-                              int ntasks, int* state, unsigned* ticket, Scalars* sc) {
+                              int ntasks, int* state, Scalars* sc) {
   const unsigned g = (unsigned)std::min<int64_t>((m * m + 255) / 256, 4736);
   k_df_convert<<<g, 256, 0, st>>>(m, ldm, M, 1);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess)
     e = cholesky_tiles<dfloat>(st, m, ldm, reinterpret_cast<dfloat*>(M), reinterpret_cast<dfloat*>(dinv), nullptr,
-                               tasks, ntasks, state, ticket, sc, nullptr);
+                               tasks, ntasks, state, sc, nullptr);
   if (e != cudaSuccess) return e;
   k_df_convert<<<g, 256, 0, st>>>(m, ldm, M, 0);
   k_df_to_double<<<(unsigned)std::min<int64_t>((m + 255) / 256, 1184), 256, 0, st>>>(m, dinv);

@@ -44,7 +44,7 @@ struct Scalars {
 
 // Counters for the "last block finishes the reduction" pattern and the
 // triangular-solve tickets.
-enum Ticket { T_SCALING = 0, T_PSI, T_STEP, T_NORM, T_NORM2, T_DOT, T_TRSV, T_TRSVB, T_CHOL, T_RES, T_COUNT };
+enum Ticket { T_SCALING = 0, T_PSI, T_STEP, T_NORM, T_NORM2, T_DOT, T_TRSVB, T_RES, T_COUNT };
 
 // ---- exact widening of the stored A ---------------------------------------
 __device__ __forceinline__ double widen(double v) { return v; }
@@ -129,8 +129,8 @@ template <typename T>
 cudaError_t cholesky(cudaStream_t st, int64_t m, int64_t ldm, T* M, T* dinv, Scalars* sc);
 
 // The single-launch tile Cholesky (chol_tiles.cu): 128 x 128 tiles; the task
-// list comes from chol_tile_tasks (built once per m); state holds nb^2 + nb
-// ints (nb = chol_tile_count(m)); ticket is one counter.  Both are cleared here.
+// list comes from chol_tile_tasks (built once per m); state holds nb^2 + nb + 1
+// ints (nb = chol_tile_count(m)), cleared here.
 // Beyond 256 tile rows (m > 32768) the task list (~nb^3/6 tasks, built on
 // the host at handle creation) grows past ~3M entries; such handles keep the
 // multi-launch blocked factor.
@@ -143,7 +143,7 @@ void chol_tile_tasks(int64_t m, int nproc, std::vector<int4>* out);
 // row-major per tile), for trsv_lower_blk / trsv_upper_blk.
 template <typename T>
 cudaError_t cholesky_tiles(cudaStream_t st, int64_t m, int64_t ldm, T* M, T* dinv, T* Uinv, const int4* tasks,
-                           int ntasks, int* state, unsigned* ticket, Scalars* sc, unsigned char* planes);
+                           int ntasks, int* state, Scalars* sc, unsigned char* planes);
 // Bytes of the BF16 operand planes of the FP32 tile factor (every tile below
 // the diagonal, 96 KB each).
 int64_t chol_plane_bytes(int64_t m);
@@ -153,7 +153,7 @@ int64_t chol_plane_bytes(int64_t m);
 // factor's), and turned back into the FP64 factor L and FP64 pivot
 // reciprocals dinv.  A pivot that is not positive sets PDAS_ERR_NOT_SPD.
 cudaError_t cholesky_tiles_df(cudaStream_t st, int64_t m, int64_t ldm, double* M, double* dinv, const int4* tasks,
-                              int ntasks, int* state, unsigned* ticket, Scalars* sc);
+                              int ntasks, int* state, Scalars* sc);
 // The triangular solves with the FP32 tile factor (trsv_blk.cu): out =
 // (L L')^{-1} rhs through z.  z holds the unset pattern (every bit set) in all
 // entries before and after, as does *ticket zero, unless a wait gave up: then
@@ -168,10 +168,10 @@ cudaError_t trsv_blk_solve(cudaStream_t st, int64_t m, int64_t ldm, const float*
 // substitution (the plain FP64 form's direct solve).
 template <typename T>
 cudaError_t trsv_lower(cudaStream_t st, int64_t m, int64_t ldm, const T* L, const T* dinv, const double* v,
-                       double* z, int* flags, unsigned* tickets, Scalars* sc, bool scaled);
+                       double* z, int* flags, Scalars* sc, bool scaled);
 template <typename T>
 cudaError_t trsv_upper_t(cudaStream_t st, int64_t m, int64_t ldm, const T* L, const T* dinv, const double* z,
-                         double* y, int* flags, unsigned* tickets, Scalars* sc, bool scaled);
+                         double* y, int* flags, Scalars* sc, bool scaled);
 
 // sc->mnorm = max_p M[p][p] (before the factorization overwrites it).
 template <typename T>

@@ -274,13 +274,17 @@ __global__ void __launch_bounds__(kThreads) k_step(int64_t m, int64_t n, const d
   }
   if (!last_block(tickets + T_STEP)) return;
   double gc = 0.0, gb = 0.0, gx = 0.0;
-  // one thread combines in block order: the partial count is small
-  if (threadIdx.x == 0) {
-    for (int i = 0; i < (int)gridDim.x; ++i) {
+  if (threadIdx.x < 32) {  // one warp combines, in a fixed order
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += 32) {
       gc += __ldcg(part + 3 * i);
       gb += __ldcg(part + 3 * i + 1);
       gx += __ldcg(part + 3 * i + 2);
     }
+    gc = warp_sum(gc);
+    gb = warp_sum(gb);
+    gx = warp_sum(gx);
+  }
+  if (threadIdx.x == 0) {
     sc->cx = gc;
     sc->by = gb;
     sc->xs = gx;
@@ -520,7 +524,9 @@ cudaError_t launch_residual_norms(cudaStream_t st, int64_t m, int64_t n, const d
 
 cudaError_t launch_scaling(cudaStream_t st, int64_t n, const double* x, const double* s, double* D, double* part,
                            unsigned* tickets, Scalars* sc) {
-  const int g = grid_for(n, 4);
+  // (an element per thread up to 303k: the FP64 divisions of a thread follow one
+  // another at ~400 cycles each; 8192 columns took 10 us with four per thread)
+  const int g = grid_for(n);
   k_scaling<<<g, kThreads, 0, st>>>(n, x, s, D, part, tickets, sc);
   return cudaGetLastError();
 }
@@ -528,14 +534,14 @@ cudaError_t launch_scaling(cudaStream_t st, int64_t n, const double* x, const do
 cudaError_t launch_psi(cudaStream_t st, int64_t n, const double* x, const double* s, const double* dx,
                        const double* ds, double alpha, double* part, unsigned* tickets, Scalars* sc,
                        bool capped) {
-  k_psi<<<grid_for(n, 4), kThreads, 0, st>>>(n, x, s, dx, ds, alpha, part, tickets, sc, capped ? 1 : 0);
+  k_psi<<<grid_for(n), kThreads, 0, st>>>(n, x, s, dx, ds, alpha, part, tickets, sc, capped ? 1 : 0);
   return cudaGetLastError();
 }
 
 cudaError_t launch_step(cudaStream_t st, int64_t m, int64_t n, const double* b, const double* c, double* x,
                         double* y, double* s, const double* dx, const double* dy, const double* ds, double* part,
                         unsigned* tickets, Scalars* sc) {
-  k_step<<<grid_for(n > m ? n : m, 4), kThreads, 0, st>>>(m, n, b, c, x, y, s, dx, dy, ds, part, tickets, sc);
+  k_step<<<grid_for(n > m ? n : m), kThreads, 0, st>>>(m, n, b, c, x, y, s, dx, dy, ds, part, tickets, sc);
   return cudaGetLastError();
 }
 
@@ -564,7 +570,7 @@ cudaError_t launch_cg_dot(cudaStream_t st, int64_t m, const double* a, const dou
 template <typename T>
 cudaError_t launch_diag_max(cudaStream_t st, int64_t m, int64_t ldm, const T* M, double* part, unsigned* tickets,
                             Scalars* sc) {
-  k_diag_max<T><<<grid_for(m, 4), kThreads, 0, st>>>(m, ldm, M, part, tickets, sc);
+  k_diag_max<T><<<grid_for(m), kThreads, 0, st>>>(m, ldm, M, part, tickets, sc);
   return cudaGetLastError();
 }
 template cudaError_t launch_diag_max<double>(cudaStream_t, int64_t, int64_t, const double*, double*, unsigned*,
