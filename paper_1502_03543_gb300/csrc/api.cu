@@ -56,6 +56,7 @@ struct pdas_ctx {
   double* M64 = nullptr;      // FP64 form; mixed forms: the FP64 tier's matrix (allocated at create)
   float* M32 = nullptr;
   double* dinv64 = nullptr;  // reciprocals of the pivots of the FP64 / FP32 factor
+  double* inv64 = nullptr;   // inverses of the FP64 factor's 64 x 64 diagonal blocks (mixed forms)
   float* dinv32 = nullptr;
   void* simt_part = nullptr;        // SIMT normal matrices: partial tiles of their K slices
   unsigned* simt_tickets = nullptr;  // one per tile, zero between launches
@@ -244,7 +245,7 @@ pdas_status reset_status(pdas_ctx* h) {
 }
 
 // A v -> out (base == null) or base - A v -> out; norm_slot as in launch_gemv.
-// Double-float passes over A (gemv_df.cu) are available to the mixed forms
+// Double-float passes over A (passes.cu) are available to the mixed forms
 // when A is exact in FP32 (stored as FP32 or BF16) and exact_passes is off.
 // The solve uses them only for the conjugate-gradient operator M p of the
 // refinement while it factors in FP32: every quantity the acceptance test or
@@ -406,9 +407,7 @@ pdas_status factor(pdas_ctx* h) {
     int k = 0;
     CK(cholesky_dig(h->st, &h->cdig, h->ldm, h->M64, h->dinv64, h->sc, &k));
     h->launches += k;
-    return PDAS_OK;
-  }
-  if (h->cur_f64 && is_mixed(h) && h->chol_ntasks > 0 && !h->no_dffactor_once &&
+  } else if (h->cur_f64 && is_mixed(h) && h->chol_ntasks > 0 && !h->no_dffactor_once &&
       h->last_rel_gap > h->opt.df_factor_floor) {
     // FP64 tier of a mixed form: the double-float tile factor (FP32 pipes),
     // while the iterate is not yet close to the optimum
@@ -428,6 +427,8 @@ pdas_status factor(pdas_ctx* h) {
                              h->chol_state, h->sc, h->chol_planes),
        1);
   }
+  if (h->cur_f64 && h->inv64)
+    KL(launch_invert_diag64(h->st, h->m, h->ldm, h->M64, h->dinv64, h->inv64, h->sc), 1);
   return PDAS_OK;
 }
 
@@ -446,16 +447,11 @@ pdas_status factor_solve(pdas_ctx* h, double* rhs, double* out, const CgStep* up
   }
   if (upd) KL(launch_cg_update(h->st, h->m, *upd, rhs, h->part, h->tickets, h->sc), 1);
   if (h->cur_f64) {
-    KL(trsv_lower<double>(h->st, h->m, h->ldm, h->M64, h->dinv64, rhs, h->z, h->flags, h->sc,
-                          is_mixed(h)),
-       1);
-    KL(trsv_upper_t<double>(h->st, h->m, h->ldm, h->M64, h->dinv64, h->z, out, h->flags, h->sc,
-                            is_mixed(h)),
-       1);
+    KL(trsv_lower<double>(h->st, h->m, h->ldm, h->M64, h->dinv64, h->inv64, rhs, h->z, h->flags, h->sc), 1);
+    KL(trsv_upper_t<double>(h->st, h->m, h->ldm, h->M64, h->dinv64, h->inv64, h->z, out, h->flags, h->sc), 1);
   } else {
-    KL(trsv_lower<float>(h->st, h->m, h->ldm, h->M32, h->dinv32, rhs, h->z, h->flags, h->sc, true), 1);
-    KL(trsv_upper_t<float>(h->st, h->m, h->ldm, h->M32, h->dinv32, h->z, out, h->flags, h->sc, true),
-       1);
+    KL(trsv_lower<float>(h->st, h->m, h->ldm, h->M32, h->dinv32, nullptr, rhs, h->z, h->flags, h->sc), 1);
+    KL(trsv_upper_t<float>(h->st, h->m, h->ldm, h->M32, h->dinv32, nullptr, h->z, out, h->flags, h->sc), 1);
   }
   if (nrz) {
     KL(launch_cg_dot(h->st, h->m, rhs, out, h->part, rz_part(h), h->tickets, h->sc), 1);
@@ -872,6 +868,7 @@ pdas_status pdas_create(int64_t m, int64_t n, const pdas_options* opt_in, pdas_h
     if (opt.form != PDAS_FP64) {
       al((void**)&h->M32, sizeof(float) * h->ldm * m);
       al((void**)&h->dinv32, sizeof(float) * m);
+      al((void**)&h->inv64, sizeof(double) * nblk * kTile * kTile);
       if (opt.a_dtype != PDAS_A_F64) al((void**)&h->d2, sizeof(float2) * n);
       if (opt.drop_tol > 0) {
         al((void**)&h->akept, dtype_size(opt.a_dtype) * m * n);

@@ -225,8 +225,8 @@ __device__ __forceinline__ int red_row(int lane) { return 4 * ((lane >> 4) & 1) 
 // Arithmetic in T (the factor's precision; the FP32 factor of the mixed forms
 // is a preconditioner, refined in FP64 afterwards); v, z in FP64.  Warp w
 // owns rows 8w..8w+7 of the block, lane l owns columns l, l+32; the diagonal
-// block is solved by warp 0.  SCALED (the FP64 tier of the mixed forms,
-// whose refinement takes the solve as a preconditioner): on its rows divided
+// block is solved by warp 0.  SCALED (the FP32 blocked factor of the mixed forms,
+// a preconditioner of their refinement): on its rows divided
 // by their pivots, z_r = v_r / L_rr - sum_{c<r} (L_rc / L_rr) z_c, so a step
 // of its chain is one shuffle and one multiply-add, and the eight row sums
 // of a warp are combined by a reduce-scatter.  Otherwise (the plain FP64
@@ -421,6 +421,180 @@ __global__ void __launch_bounds__(kThreads) k_trsv_upper_t(int64_t m, int64_t ld
   }
 }
 
+// inv = the inverses of the factor's 64 x 64 diagonal blocks, row-major, one
+// after another (rows and columns past m are the identity's).  One CTA per
+// block, right-looking on its rows divided by their pivots: after step k row
+// k of R is final up to its pivot, and R_rc -= (L_rk / L_rr) R_kc for r > k,
+// c <= k.  Thread (c, q) takes column c, so the warps of columns past k skip.
+// Bound by the FP64 pipe, ~25 us whatever m: the blocks are independent.
+__global__ void __launch_bounds__(kThreads) k_invert_diag64(int64_t m, int64_t ldm, const double* __restrict__ L,
+                                                            const double* __restrict__ dinv,
+                                                            double* __restrict__ inv, const Scalars* sc) {
+  extern __shared__ double sm[];
+  double(*Lh)[kTile] = reinterpret_cast<double(*)[kTile]>(sm);
+  double(*R)[kTile] = reinterpret_cast<double(*)[kTile]>(sm + kTile * kTile);
+  __shared__ double rcp[kTile];
+  if (dev_failed(sc)) return;
+  const int64_t r0 = (int64_t)blockIdx.x * kTile;
+  const int rb = (int)(m - r0 < kTile ? m - r0 : kTile);
+  for (int e = threadIdx.x; e < kTile * kTile; e += blockDim.x) {
+    const int i = e / kTile, j = e % kTile;
+    Lh[i][j] = (i < rb && j < i) ? L[(r0 + i) * ldm + r0 + j] * dinv[r0 + i] : 0.0;
+    R[i][j] = i == j ? 1.0 : 0.0;
+  }
+  if (threadIdx.x < kTile) rcp[threadIdx.x] = threadIdx.x < rb ? dinv[r0 + threadIdx.x] : 1.0;
+  __syncthreads();
+  const int c = threadIdx.x & (kTile - 1), q = threadIdx.x >> 6;
+  for (int k = 0; k < kTile - 1; ++k) {
+    if ((c & 32) <= k) {  // (R_kc is zero for c > k)
+      const double x = R[k][c];
+      for (int r = k + 1 + q; r < kTile; r += kThreads / kTile) R[r][c] = fma(-Lh[r][k], x, R[r][c]);
+    }
+    __syncthreads();
+  }
+  // R is inv(D^{-1} L) with D the pivots: L^{-1} = R D^{-1}, columns scaled
+  double* out = inv + (int64_t)blockIdx.x * kTile * kTile;
+  for (int e = threadIdx.x; e < kTile * kTile; e += blockDim.x) out[e] = R[e / kTile][e % kTile] * rcp[e % kTile];
+}
+
+// The two solves of the FP64 tier's refinement (a preconditioner: what they
+// lose in the last bits the conjugate gradients make good).  A link of the
+// block chain is what it costs, and in a link every warp-wide FP64
+// instruction holds its sub-partition for 64 cycles: so the 64-step
+// substitution (7,400 cycles on one warp) is a product with L_bb^{-1} on all
+// eight (1,800), and a row's 64 terms are split over four neighbouring
+// threads, whose sums take two shuffles.  The block's own inverse waits in
+// registers.  m = 4096: the two
+// solves of a refinement step 1043 -> 571 us.
+__global__ void __launch_bounds__(kThreads) k_trsv_lower_inv(int64_t m, int64_t ldm, const double* __restrict__ L,
+                                                             const double* __restrict__ inv,
+                                                             const double* __restrict__ v, double* z, int* flags,
+                                                             unsigned* ticket, Scalars* sc) {
+  __shared__ double acc[kTile];
+  __shared__ int sbi;
+  if (threadIdx.x == 0) sbi = (int)atomicAdd(ticket, 1u);
+  __syncthreads();
+  if (dev_failed(sc)) return;
+  const int64_t b = sbi;
+  const int64_t r0 = b * kTile;
+  const int rb = (int)(m - r0 < kTile ? m - r0 : kTile);
+  const int w = threadIdx.x >> 5, r = threadIdx.x >> 2, q = threadIdx.x & 3;
+  const bool in = r < rb;
+  const int64_t row = (r0 + (in ? r : 0)) * ldm;  // (rows are 16-byte aligned: ldm is a multiple of 16)
+  const double vr = in ? v[r0 + r] : 0.0;
+  double2 u[8];  // columns 2q + 8i, + 1 of row r; zero past the diagonal
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+    u[i] = *reinterpret_cast<const double2*>(inv + (b * kTile + r) * kTile + 2 * q + 8 * i);
+  double part = 0.0, part2 = 0.0;
+  bool ok = true;
+  for (int64_t jb = 0; jb < b && ok; ++jb) {
+    double2 l[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      l[i] = in ? __ldg(reinterpret_cast<const double2*>(L + row + jb * kTile + 2 * q + 8 * i)) : make_double2(0.0, 0.0);
+    ok = warp_wait(flags, jb, sc);
+    if (!ok) break;
+    double2 zv[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) zv[i] = __ldcg(reinterpret_cast<const double2*>(z + jb * kTile + 2 * q + 8 * i));
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      part = fma(l[i].x, zv[i].x, part);
+      part2 = fma(l[i].y, zv[i].y, part2);
+    }
+  }
+  double t = part + part2;
+  t += __shfl_xor_sync(0xffffffffu, t, 1);
+  t += __shfl_xor_sync(0xffffffffu, t, 2);
+  if (q == 0) acc[r] = vr - t;  // (zero past the last row)
+  if (__syncthreads_or(!ok)) return;  // a wait gave up: the status says why
+  double z0 = 0.0, z1 = 0.0;
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+    if (i <= w) {  // (row 8w + 7 ends in columns 8w ..)
+      z0 = fma(u[i].x, acc[2 * q + 8 * i], z0);
+      z1 = fma(u[i].y, acc[2 * q + 8 * i + 1], z1);
+    }
+  z0 += z1;
+  z0 += __shfl_xor_sync(0xffffffffu, z0, 1);
+  z0 += __shfl_xor_sync(0xffffffffu, z0, 2);
+  if (q == 0 && in) z[r0 + r] = z0;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) st_release(flags + b, 1);
+}
+
+// As above for L' y = z, blocks from the last to the first: warp w sums rows
+// 8w .. 8w + 7 of a block into columns lane and lane + 32, and at the end four
+// threads add a column's eight sums.
+__global__ void __launch_bounds__(kThreads) k_trsv_upper_inv(int64_t m, int64_t ldm, const double* __restrict__ L,
+                                                             const double* __restrict__ inv,
+                                                             const double* __restrict__ zin, double* y, int* flags,
+                                                             unsigned* ticket, Scalars* sc) {
+  __shared__ double red[8][kTile];
+  __shared__ double acc[kTile];
+  __shared__ int sbi;
+  const int64_t nblk = (m + kTile - 1) / kTile;
+  if (threadIdx.x == 0) sbi = (int)atomicAdd(ticket, 1u);
+  __syncthreads();
+  if (dev_failed(sc)) return;
+  const int64_t b = nblk - 1 - sbi;
+  const int64_t r0 = b * kTile;
+  const int rb = (int)(m - r0 < kTile ? m - r0 : kTile);
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, c = threadIdx.x >> 2, q = threadIdx.x & 3;
+  const double zc = c < rb ? zin[r0 + c] : 0.0;
+  double u[16];  // rows q + 4i of column c; zero before the diagonal
+#pragma unroll
+  for (int i = 0; i < 16; ++i) u[i] = inv[(b * kTile + q + 4 * i) * kTile + c];
+  double p0 = 0.0, p1 = 0.0;
+  bool ok = true;
+  for (int64_t kb = nblk - 1; kb > b && ok; --kb) {
+    const int64_t k0 = kb * kTile;
+    const int kr = (int)(m - k0 < kTile ? m - k0 : kTile);
+    double l0[8], l1[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int k = 8 * w + i;
+      const double* row = L + (k0 + k) * ldm + r0;  // (this block is a full one: kb follows it)
+      l0[i] = k < kr ? row[lane] : 0.0;
+      l1[i] = k < kr ? row[lane + 32] : 0.0;
+    }
+    ok = warp_wait(flags, kb, sc);
+    if (!ok) break;
+    double yv[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) yv[i] = 8 * w + i < kr ? __ldcg(y + k0 + 8 * w + i) : 0.0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      p0 = fma(l0[i], yv[i], p0);
+      p1 = fma(l1[i], yv[i], p1);
+    }
+  }
+  red[w][lane] = p0;
+  red[w][lane + 32] = p1;
+  if (__syncthreads_or(!ok)) return;  // a wait gave up: the status says why
+  double t = red[q][c] + red[q + 4][c];
+  t += __shfl_xor_sync(0xffffffffu, t, 1);
+  t += __shfl_xor_sync(0xffffffffu, t, 2);
+  if (q == 0) acc[c] = zc - t;  // (zero past the last column)
+  __syncthreads();
+  double y0 = 0.0, y1 = 0.0;
+#pragma unroll
+  for (int i = 0; i < 16; i += 2)
+    if (i >= 2 * w) {  // (column 8w starts in row 8w)
+      y0 = fma(u[i], acc[q + 4 * i], y0);
+      y1 = fma(u[i + 1], acc[q + 4 * i + 4], y1);
+    }
+  y0 += y1;
+  y0 += __shfl_xor_sync(0xffffffffu, y0, 1);
+  y0 += __shfl_xor_sync(0xffffffffu, y0, 2);
+  if (q == 0 && c < rb) y[r0 + c] = y0;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) st_release(flags + b, 1);
+}
+
 }  // namespace
 
 template <typename T>
@@ -445,29 +619,42 @@ cudaError_t cholesky(cudaStream_t st, int64_t m, int64_t ldm, T* M, T* dinv, Sca
   return cudaGetLastError();
 }
 
+cudaError_t launch_invert_diag64(cudaStream_t st, int64_t m, int64_t ldm, const double* L, const double* dinv,
+                                 double* inv, const Scalars* sc) {
+  constexpr int kSmem = 2 * kTile * kTile * (int)sizeof(double);
+  const cudaError_t e = cudaFuncSetAttribute(k_invert_diag64, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+  if (e != cudaSuccess) return e;
+  k_invert_diag64<<<(unsigned)((m + kTile - 1) / kTile), kThreads, kSmem, st>>>(m, ldm, L, dinv, inv, sc);
+  return cudaGetLastError();
+}
+
 template <typename T>
-cudaError_t trsv_lower(cudaStream_t st, int64_t m, int64_t ldm, const T* L, const T* dinv, const double* v, double* z,
-                       int* flags, Scalars* sc, bool scaled) {
+cudaError_t trsv_lower(cudaStream_t st, int64_t m, int64_t ldm, const T* L, const T* dinv, const T* inv,
+                       const double* v, double* z, int* flags, Scalars* sc) {
   const int64_t nblk = (m + kTile - 1) / kTile;
   unsigned* ticket = reinterpret_cast<unsigned*>(flags + nblk);  // (cleared with the flags)
   const cudaError_t e = cudaMemsetAsync(flags, 0, sizeof(int) * (nblk + 1), st);
   if (e != cudaSuccess) return e;
-  if (scaled)
+  if constexpr (sizeof(T) == 4)
     k_trsv_lower<T, true><<<(unsigned)nblk, kThreads, 0, st>>>(m, ldm, L, dinv, v, z, flags, ticket, sc);
+  else if (inv)
+    k_trsv_lower_inv<<<(unsigned)nblk, kThreads, 0, st>>>(m, ldm, L, inv, v, z, flags, ticket, sc);
   else
     k_trsv_lower<T, false><<<(unsigned)nblk, kThreads, 0, st>>>(m, ldm, L, dinv, v, z, flags, ticket, sc);
   return cudaGetLastError();
 }
 
 template <typename T>
-cudaError_t trsv_upper_t(cudaStream_t st, int64_t m, int64_t ldm, const T* L, const T* dinv, const double* z,
-                         double* y, int* flags, Scalars* sc, bool scaled) {
+cudaError_t trsv_upper_t(cudaStream_t st, int64_t m, int64_t ldm, const T* L, const T* dinv, const T* inv,
+                         const double* z, double* y, int* flags, Scalars* sc) {
   const int64_t nblk = (m + kTile - 1) / kTile;
   unsigned* ticket = reinterpret_cast<unsigned*>(flags + nblk);  // (cleared with the flags)
   const cudaError_t e = cudaMemsetAsync(flags, 0, sizeof(int) * (nblk + 1), st);
   if (e != cudaSuccess) return e;
-  if (scaled)
+  if constexpr (sizeof(T) == 4)
     k_trsv_upper_t<T, true><<<(unsigned)nblk, kThreads, 0, st>>>(m, ldm, L, dinv, z, y, flags, ticket, sc);
+  else if (inv)
+    k_trsv_upper_inv<<<(unsigned)nblk, kThreads, 0, st>>>(m, ldm, L, inv, z, y, flags, ticket, sc);
   else
     k_trsv_upper_t<T, false><<<(unsigned)nblk, kThreads, 0, st>>>(m, ldm, L, dinv, z, y, flags, ticket, sc);
   return cudaGetLastError();
@@ -476,12 +663,12 @@ cudaError_t trsv_upper_t(cudaStream_t st, int64_t m, int64_t ldm, const T* L, co
 template cudaError_t cholesky<double>(cudaStream_t, int64_t, int64_t, double*, double*, Scalars*);
 template cudaError_t cholesky<float>(cudaStream_t, int64_t, int64_t, float*, float*, Scalars*);
 template cudaError_t trsv_lower<double>(cudaStream_t, int64_t, int64_t, const double*, const double*, const double*,
-                                        double*, int*, Scalars*, bool);
-template cudaError_t trsv_lower<float>(cudaStream_t, int64_t, int64_t, const float*, const float*, const double*,
-                                       double*, int*, Scalars*, bool);
+                                        const double*, double*, int*, Scalars*);
+template cudaError_t trsv_lower<float>(cudaStream_t, int64_t, int64_t, const float*, const float*, const float*,
+                                       const double*, double*, int*, Scalars*);
 template cudaError_t trsv_upper_t<double>(cudaStream_t, int64_t, int64_t, const double*, const double*, const double*,
-                                          double*, int*, Scalars*, bool);
-template cudaError_t trsv_upper_t<float>(cudaStream_t, int64_t, int64_t, const float*, const float*, const double*,
-                                         double*, int*, Scalars*, bool);
+                                          const double*, double*, int*, Scalars*);
+template cudaError_t trsv_upper_t<float>(cudaStream_t, int64_t, int64_t, const float*, const float*, const float*,
+                                         const double*, double*, int*, Scalars*);
 
 }  // namespace pdas

@@ -163,15 +163,19 @@ cudaError_t cholesky_tiles_df(cudaStream_t st, int64_t m, int64_t ldm, double* M
 cudaError_t trsv_blk_solve(cudaStream_t st, int64_t m, int64_t ldm, const float* L, const float* Uinv, double* rhs,
                            double* z, double* out, const CgStep* upd, double* dpart, double* npart, unsigned* ticket,
                            Scalars* sc);
-// scaled: the diagonal blocks are solved on pivot-scaled rows (the FP64 tier
-// of the mixed forms, a preconditioner: shorter chains); else by plain
-// substitution (the plain FP64 form's direct solve).
+// inv != null (launch_invert_diag64's; the FP64 tier of the mixed forms, a
+// preconditioner): the diagonal blocks are applied as inverses, a shorter chain.
+// Else by substitution: FP32 on pivot-scaled rows, FP64 plain (the plain FP64
+// form's direct solve).  L's rows are 16-byte aligned.
 template <typename T>
-cudaError_t trsv_lower(cudaStream_t st, int64_t m, int64_t ldm, const T* L, const T* dinv, const double* v,
-                       double* z, int* flags, Scalars* sc, bool scaled);
+cudaError_t trsv_lower(cudaStream_t st, int64_t m, int64_t ldm, const T* L, const T* dinv, const T* inv,
+                       const double* v, double* z, int* flags, Scalars* sc);
 template <typename T>
-cudaError_t trsv_upper_t(cudaStream_t st, int64_t m, int64_t ldm, const T* L, const T* dinv, const double* z,
-                         double* y, int* flags, Scalars* sc, bool scaled);
+cudaError_t trsv_upper_t(cudaStream_t st, int64_t m, int64_t ldm, const T* L, const T* dinv, const T* inv,
+                         const double* z, double* y, int* flags, Scalars* sc);
+// inv (round_up(m, 64) x 64) = the inverses of L's 64 x 64 diagonal blocks.
+cudaError_t launch_invert_diag64(cudaStream_t st, int64_t m, int64_t ldm, const double* L, const double* dinv,
+                                 double* inv, const Scalars* sc);
 
 // sc->mnorm = max_p M[p][p] (before the factorization overwrites it).
 template <typename T>
