@@ -116,7 +116,7 @@ typedef struct {
                               factor's trailing updates run on the tensor cores from digit
                               planes of each panel (FP64-grade at every gap);
                               0 = double-float formation (normal_form 2) and the factors of
-                              df_factor_floor.  PDAS_FP64: 1 = the factor of (b) at every m (a
+                              df_factor_floor.  PDAS_FP64: 1 = the factor of (b) for m <= 4096 (a
                               matrix that it finds not positive definite is factored again on the
                               SIMT pipes); 0 = the SIMT factor                                 (1) */
   double df_factor_floor;  /* mixed forms in the FP64 tier without the tensor-core factor: the

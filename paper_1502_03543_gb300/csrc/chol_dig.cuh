@@ -8,9 +8,12 @@
 namespace pdas {
 
 // Smallest m whose FP64 tier takes this factor (below it the double-float tile
-// factor is as fast).  The plain FP64 form takes it at every m: against the
-// SIMT factor 52 to 96 us at m = 64, 1.15 to 5.96 ms at m = 1000.
+// factor is as fast).
 constexpr int64_t kCholDigMinM = 256;
+// The plain FP64 form takes it up to this many rows (pdas_create says why the
+// line lies here): against the SIMT factor 52 to 96 us at m = 64, 1.15 to 5.96
+// ms at m = 1000.
+constexpr int64_t kFp64FormDigMaxM = 4096;
 
 struct CholDigWorkspace {
   int64_t m = 0;           // 0: not created
