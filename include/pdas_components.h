@@ -86,6 +86,12 @@ pdas_status pdas_gemv_t(pdas_handle h, const void* A, const double* u, double* o
  * deadlock-free. */
 int64_t pdas_chol_tile_tasks(int64_t m, int32_t nproc, int32_t* out, int64_t cap);
 
+/* Host-only.  How far the FP32 factor's 16-byte loads of the 32-column panels
+ * of its diagonal tiles reach into M (m rows of ldm elements): returns one past
+ * the last element they touch, at most m ldm; *row_end (may be NULL): one past
+ * the last column, at most ldm. */
+int64_t pdas_chol_panel_extent(int64_t m, int64_t ldm, int64_t* row_end);
+
 /* Size of the fixed device scratch behind pdas_gemv_t_noalloc: 8 MiB. */
 #define PDAS_NOALLOC_SCRATCH_BYTES (8u << 20)
 

@@ -119,6 +119,7 @@ SIGNATURES = {
     "pdas_gemv_t": ([_H, _P, _P, _P], _I),
     "pdas_gemv_t_noalloc": ([_I64, _I64, _I, _P, _P, _P, _P], _I),
     "pdas_chol_tile_tasks": ([_I64, _I, _P, _I64], _I64),
+    "pdas_chol_panel_extent": ([_I64, _I64, ctypes.POINTER(_I64)], _I64),
     "pdas_batch_default_options": ([ctypes.POINTER(BatchOptions)], None),
     "pdas_batch_create": ([_I, _P, _P, _P, _P, _P, _P, _P, _P, ctypes.POINTER(BatchOptions), ctypes.POINTER(_H)],
                           _I),

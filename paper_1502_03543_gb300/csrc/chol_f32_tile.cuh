@@ -367,25 +367,34 @@ __device__ __forceinline__ void trsm_update(Tile C, const float (*P)[kPt], int k
 // rows from 32 b on, 16-byte loads through L2 (thread unit v of 4: row r,
 // columns 32 b + c .. + 3), then into a column-major panel buffer (entries above
 // the diagonal are never used; rows past m are the identity's).
-__device__ __forceinline__ void panel_rc(int v, int& r, int& c) {
-  const int lane = threadIdx.x & 31, u = (threadIdx.x >> 5) + 8 * v;
+__host__ __device__ __forceinline__ void panel_rc(int tid, int v, int& r, int& c) {
+  const int lane = tid & 31, u = (tid >> 5) + 8 * v;
   r = 16 * (u & 7) + (lane & 15);
   c = 8 * (u >> 3) + 4 * (lane >> 4);
+}
+// Whether the vector at row r, column c of that tile is read: only where it
+// starts on or below the diagonal, so at a column <= its row < m, from where a
+// row padded to a multiple of 16 columns holds all of it.  (A panel's 32
+// columns can reach past the padding: m = 33 has rows of 48 and a panel from 32
+// to 63.)
+__host__ __device__ __forceinline__ bool panel_reads(int64_t m, int64_t q0, int r, int c) {
+  return c <= r && q0 + r < m;
 }
 __device__ __forceinline__ void fetch_panel(float4 (&x)[4], int64_t m, int64_t ldm, const float* M, int64_t q0, int b) {
 #pragma unroll
   for (int v = 0; v < 4; ++v) {
     int r, c;
-    panel_rc(v, r, c);
-    x[v] = (r >= 32 * b && q0 + r < m) ? __ldcg(reinterpret_cast<const float4*>(M + (q0 + r) * ldm + q0 + 32 * b + c))
-                                      : make_float4(0.f, 0.f, 0.f, 0.f);
+    panel_rc(threadIdx.x, v, r, c);
+    x[v] = panel_reads(m, q0, r, 32 * b + c)
+               ? __ldcg(reinterpret_cast<const float4*>(M + (q0 + r) * ldm + q0 + 32 * b + c))
+               : make_float4(0.f, 0.f, 0.f, 0.f);
   }
 }
 __device__ __forceinline__ void put_panel(const float4 (&x)[4], Tile P) {
 #pragma unroll
   for (int v = 0; v < 4; ++v) {
     int r, c;
-    panel_rc(v, r, c);
+    panel_rc(threadIdx.x, v, r, c);
     P[c][r] = x[v].x, P[c + 1][r] = x[v].y, P[c + 2][r] = x[v].z, P[c + 3][r] = x[v].w;
   }
 }

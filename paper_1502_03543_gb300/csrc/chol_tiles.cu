@@ -861,7 +861,7 @@ __device__ void chol_chain(int me, int64_t m, int64_t ldm, float* M, float* dinv
 #pragma unroll
           for (int v = 0; v < 4; ++v) {
             int r, c;
-            ft::panel_rc(v, r, c);
+            ft::panel_rc(tid, v, r, c);
             c += 32 * b;
             if (p0 + r < m && c <= r) {
               float* dst = M + (p0 + r) * ldm + p0 + c;
@@ -1328,4 +1328,24 @@ extern "C" int64_t pdas_chol_tile_tasks(int64_t m, int32_t nproc, int32_t* out, 
     }
   }
   return n;
+}
+
+// Host-only: one past the last element of M (leading dimension ldm) that the
+// FP32 factor's loads of the panels of its diagonal tiles touch, for a test of
+// their bounds; *row_end: the same within a row.
+extern "C" int64_t pdas_chol_panel_extent(int64_t m, int64_t ldm, int64_t* row_end) {
+  int64_t end = 0, cols = 0;
+  for (int64_t q0 = 0; q0 < m; q0 += pdas::kBig)
+    for (int b = 0; b < 4; ++b)
+      for (int tid = 0; tid < pdas::kThreads; ++tid)
+        for (int v = 0; v < 4; ++v) {
+          int r, c;
+          pdas::ft::panel_rc(tid, v, r, c);
+          c += 32 * b;
+          if (!pdas::ft::panel_reads(m, q0, r, c)) continue;
+          cols = std::max(cols, q0 + c + 4);
+          end = std::max(end, (q0 + r) * ldm + q0 + c + 4);
+        }
+  if (row_end) *row_end = cols;
+  return end;
 }
