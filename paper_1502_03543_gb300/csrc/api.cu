@@ -469,7 +469,8 @@ pdas_status factor_solve(pdas_ctx* h, double* rhs, double* out, const CgStep* up
 // Accepted when ||r - M dy||_inf <= refine_tol ||r||_inf, or when the
 // normwise backward error ||r - M dy||_inf / (max_p M_pp ||dy||_inf +
 // ||r||_inf) <= refine_be.  On return h->w = A' dy of the final dy;
-// *ok = 0 if neither test passed within refine_max steps.  A step is four
+// *ok = 0 if neither test passed within refine_max steps.  A step that
+// cg_step_length refuses is not taken and ends the refinement.  A step is four
 // launches (p and u = D A'p; q = A u and p'q; the two triangular solves, which
 // carry the updates and rho'z) and one read of the scalars.  The first read
 // also brings the factor's status (PDAS_ERR_NOT_SPD).
@@ -516,6 +517,7 @@ pdas_status refine(pdas_ctx* h, const void* A, int* ok) {
   } else {
     double *p = h->kp, *pn = h->kp2;
     bool first = true;  // p = z = P^{-1} rho, no direction before it
+    bool stale = false;  // dy has moved since the last true residual
     int nrz = 0;
     if (cap > 0 && (s = factor_solve(h, h->rho, h->kz, nullptr, &nrz)) != PDAS_OK) return s;
     while (its < cap) {
@@ -536,14 +538,15 @@ pdas_status refine(pdas_ctx* h, const void* A, int* ok) {
       first = false;
       if ((s = read_scalars(h)) != PDAS_OK) return s;
       if ((s = device_status(h)) != PDAS_OK) return s;
-      const double rz = h->sc_host->rz[src.par];
-      if (!(rz > 0.0 && isfinite(rz))) break;  // (nothing was updated)
+      double a;
+      if (!cg_step_length(h->sc_host->rz[src.par], h->sc_host->dot_b, &a)) break;  // (nothing was updated)
       ++its;
-      if (!(h->sc_host->dot_b > 0.0)) break;  // the preconditioned operator lost definiteness
+      stale = true;
       res = h->sc_host->rho_norm;
       dyn = h->sc_host->dynorm;
       if (accepted(res, dyn) || its % 10 == 0 || its == cap) {
         if ((s = true_residual()) != PDAS_OK) return s;
+        stale = false;
         res = h->sc_host->rho_norm;
         dyn = h->sc_host->dynorm;
         if (accepted(res, dyn)) {
@@ -553,6 +556,12 @@ pdas_status refine(pdas_ctx* h, const void* A, int* ok) {
         if (its < cap && (s = factor_solve(h, h->rho, h->kz, nullptr, &nrz)) != PDAS_OK) return s;
         first = true;
       }
+    }
+    if (stale) {  // the steps ended in between: w and the residual of this dy
+      if ((s = true_residual()) != PDAS_OK) return s;
+      res = h->sc_host->rho_norm;
+      dyn = h->sc_host->dynorm;
+      *ok = accepted(res, dyn);
     }
   }
   h->last_sweeps = its;

@@ -109,9 +109,18 @@ cudaError_t launch_step(cudaStream_t st, int64_t m, int64_t n, const double* b, 
 // *out = *sc and then *seq = want, both in pinned host memory.
 cudaError_t launch_snapshot(cudaStream_t st, const Scalars* sc, Scalars* out, unsigned* seq, unsigned want);
 cudaError_t launch_axpy(cudaStream_t st, int64_t n, double a, const double* xv, double* yv, const Scalars* sc);
+// The step length rz / pq of the conjugate gradients (rz = rho'z, pq = p'M p).
+// False if there is no step to take: a quotient of two positive numbers that is
+// finite is the only one that descends.  (pq is zero, negative or NaN where M
+// is singular to working precision or where the numbers leave the exponent
+// range; the device and the host decide by this same rule.)
+__host__ __device__ inline bool cg_step_length(double rz, double pq, double* a) {
+  *a = rz / pq;
+  return rz > 0.0 && pq > 0.0 && *a <= 1.7976931348623157e308;
+}
 // One step of the conjugate gradients: with a = *rz / sc->dot_b, dy += a p,
-// rho -= a q (nothing unless *rz is positive and finite), and the largest
-// magnitudes of dy and rho to sc->dynorm and sc->rho_norm.
+// rho -= a q (nothing unless cg_step_length), and the largest magnitudes of dy
+// and rho to sc->dynorm and sc->rho_norm.
 struct CgStep {
   const double* p;
   const double* q;

@@ -237,10 +237,8 @@ __device__ __forceinline__ bool trsv_lower_block(TrsvSmem& sm, int64_t b, int64_
   if ((lane & 1) == 0 && myrow < rb) {
     double r = v[r0 + myrow];
     if constexpr (UPD) {
-      const double rz = *upd.rz;
-      double y = upd.dy[r0 + myrow];
-      if (rz > 0.0 && isfinite(rz)) {
-        const double a = rz / sc->dot_b;
+      double a, y = upd.dy[r0 + myrow];
+      if (cg_step_length(*upd.rz, sc->dot_b, &a)) {
         y = y + a * upd.p[r0 + myrow];
         r = r - a * upd.q[r0 + myrow];
         upd.dy[r0 + myrow] = y;

@@ -313,9 +313,8 @@ __global__ void __launch_bounds__(kThreads) k_cg_update(int64_t m, const CgStep 
                                                         unsigned* tickets, Scalars* sc) {
   __shared__ double sm[32];
   if (failed(sc)) return;
-  const double rz = *upd.rz;
-  const bool go = rz > 0.0 && isfinite(rz);
-  const double a = go ? rz / sc->dot_b : 0.0;
+  double a;
+  const bool go = cg_step_length(*upd.rz, sc->dot_b, &a);
   double mr = 0.0, my = 0.0;
   for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x) {
     double y = upd.dy[j], r = rho[j];
