@@ -289,10 +289,15 @@ __device__ void blk_gemv_t_df(const Ctx& c, const float2* u2, double* out) {
 // M = (A D^1/2)(A D^1/2)' into c.L (packed lower), FP32: 32-column chunks of
 // A D^1/2 staged in shared memory column by column (pitch m_cap + 4; rows past m
 // are zero), and every thread accumulates 8 x 8 units of the lower triangle in
-// registers over all chunks: four 16-byte reads for 64 multiply-adds.  (With 4 x 8
-// outputs a lane, 12 reads for 32 multiply-adds and a read-modify-write of the
-// triangle per chunk, a formation took 1.14M cycles at 239 x 956; the
-// multiply-adds alone take 0.23M.)  m_cap is a multiple of 32.
+// registers over a chunk, then adds them to the triangle: four 16-byte reads for
+// 64 multiply-adds.  (With 4 x 8 outputs a lane, 12 reads for 32 multiply-adds,
+// a formation took 1.14M cycles at 239 x 956; the multiply-adds alone take 0.23M.)
+// The partial sums per chunk are what keeps M accurate enough for the factor:
+// in one chain over all columns its error is several times larger, the FP32
+// factor fails one to four iterations sooner, and the LP spends them in the
+// FP64 tier (512 LPs to 1e-7: 4639 of its iterations instead of 3902), which
+// costs more than the additions save (to a gap of 3e-2: 27 against 24 ms).
+// m_cap is a multiple of 32.
 template <int T>
 __device__ void blk_syrk(const Ctx& c, int m_cap) {
   constexpr int NW = T / 32;
@@ -339,13 +344,19 @@ __device__ void blk_syrk(const Ctx& c, int m_cap) {
         }
       }
       __syncthreads();
-    }
-    if (mine) {
+      if (mine) {
+        const bool add = k0 > 0;
 #pragma unroll
-      for (int x = 0; x < 8; ++x)
+        for (int x = 0; x < 8; ++x)
 #pragma unroll
-        for (int y = 0; y < 8; ++y)
-          if (r + x < m && q + y <= r + x) c.L[pk(r + x, q + y)] = acc[x][y];
+          for (int y = 0; y < 8; ++y) {
+            if (r + x < m && q + y <= r + x) {
+              float* e = c.L + pk(r + x, q + y);
+              *e = add ? *e + acc[x][y] : acc[x][y];
+            }
+            acc[x][y] = 0.f;
+          }
+      }
     }
   }
   __syncthreads();
@@ -463,7 +474,7 @@ __device__ bool blk_chol(const Ctx& c, int pm) {
 #pragma unroll
       for (int a = 0; a < 4; ++a)
 #pragma unroll
-        for (int b = 0; b < 4; ++b) x[a][b] = 0.f;
+        for (int b = 0; b < 4; ++b) x[a][b] = (r + a < m && q + b <= r + a) ? c.L[pk(r + a, q + b)] : 0.f;
 #pragma unroll 8
       for (int k = 0; k < 32; ++k) {
         const float4 a = *reinterpret_cast<const float4*>(P + k * pm + r);
@@ -472,13 +483,13 @@ __device__ bool blk_chol(const Ctx& c, int pm) {
 #pragma unroll
         for (int y = 0; y < 4; ++y)
 #pragma unroll
-          for (int z = 0; z < 4; ++z) x[y][z] = fmaf(aa[y], bb[z], x[y][z]);
+          for (int z = 0; z < 4; ++z) x[y][z] = fmaf(-aa[y], bb[z], x[y][z]);
       }
 #pragma unroll
       for (int a = 0; a < 4; ++a)
 #pragma unroll
         for (int b = 0; b < 4; ++b)
-          if (r + a < m && q + b <= r + a) c.L[pk(r + a, q + b)] -= x[a][b];
+          if (r + a < m && q + b <= r + a) c.L[pk(r + a, q + b)] = x[a][b];
     }
     __syncthreads();
   }
