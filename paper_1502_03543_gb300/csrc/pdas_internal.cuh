@@ -68,6 +68,13 @@ __device__ __forceinline__ double widen_bits(uint32_t u) {
   return __longlong_as_double((long long)(sign | (e64 << 52) | ((unsigned long long)mant << 29)));
 }
 
+// widen() without the conversion instruction.
+__device__ __forceinline__ double widen_int(double v) { return v; }
+__device__ __forceinline__ double widen_int(float v) { return widen_bits(__float_as_uint(v)); }
+__device__ __forceinline__ double widen_int(__nv_bfloat16 v) {
+  return widen_bits((uint32_t)__bfloat16_as_ushort(v) << 16);
+}
+
 __device__ __forceinline__ float widen32(double v) { return (float)v; }
 __device__ __forceinline__ float widen32(float v) { return v; }
 __device__ __forceinline__ float widen32(__nv_bfloat16 v) { return __bfloat162float(v); }

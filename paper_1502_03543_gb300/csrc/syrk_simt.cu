@@ -23,7 +23,13 @@ namespace {
 // multiply-add of a small register tile cost nothing.  So tiles are small, for
 // balance over 152 SMs and little work above the diagonal (32 x 32: 3 % of M at
 // m = 1000; the 16 x 16 quarter above the diagonal of a diagonal tile is
-// skipped), and 16 x 16 where even 32 x 32 tiles leave most SMs idle.
+// skipped), and 16 x 16 where even 32 x 32 tiles leave most SMs idle.  A small
+// tile costs more operands per multiply-add, and what they take of that pipe is
+// what counts: the product A_pk D_k (1/32 of the multiply-adds with 32 rows)
+// stays on it, the widening of a value stored as FP32 or BF16 (2/32) is done on
+// the integer pipes.  BF16 A, n = 2 m, 64 x 64 tiles before -> 32 x 32 with the
+// conversions -> now: m = 3000 50.6 -> 49.7 -> 46.6 ms, 6000 378 -> 390 -> 362, 8192
+// 946 -> 984 -> 916 (FP64 A: 911 -> 915 there).
 // Measured against 64 x 64 tiles without a K split: m = 64, n = 128 (one tile):
 // 139 -> 9.6 us; 1000 x 2500 (136 tiles on 152 SMs): 2697 -> 2388 us (floor 2000).
 template <typename T, int TS>
@@ -55,8 +61,8 @@ __global__ void __launch_bounds__(kThreads) k_syrk_fp64(int64_t m, int64_t n, co
       const int64_t k = k0 + e % kKc;
       const bool kin = k < kend;
       rd[u] = kin ? __ldg(D + k) : 0.0;
-      rp[u] = (kin && p0 + r < m) ? widen(A[(p0 + r) * n + k]) : 0.0;
-      rq[u] = (kin && q0 + r < m) ? widen(A[(q0 + r) * n + k]) : 0.0;
+      rp[u] = (kin && p0 + r < m) ? widen_int(A[(p0 + r) * n + k]) : 0.0;
+      rq[u] = (kin && q0 + r < m) ? widen_int(A[(q0 + r) * n + k]) : 0.0;
     }
   };
   fetch(kbeg);
