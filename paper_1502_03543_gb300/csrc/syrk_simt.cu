@@ -135,11 +135,11 @@ __global__ void __launch_bounds__(kThreads) k_syrk_fp64(int64_t m, int64_t n, co
 // FP64, and A itself, m x ldk FP32 each, so that the product loads 16 bytes
 // whatever the alignment of A's rows.  The planes hold columns c0 .. c0 + ldk - 1
 // (zero past column n); only where both would exceed 4 GB is that not all of A.
-// An FP64 product and two conversions per element hold the FP64 pipe for most of
-// the pass (31 us at 1001 x 3003), so where A is exact in FP32 the product is
-// formed from D as an FP32 pair, a dh + (a dl + the exact error of a dh), which
-// rounds as the FP64 product does but for ties 2^-24 apart; D outside
-// 2^(-100 .. 100) keeps the FP64 product.  A block takes 16 rows of 256 columns.
+// The FP64 product and its conversion to FP32 are what the pass costs beyond its
+// traffic; the widening of A runs on the integer pipes.  (With D as an FP32 pair
+// on the FP32 pipes the whole matrix took 139 us at 1001 x 3003 and 745 at 2000 x
+// 6000, now 132 and 713; and D lost 5 of its 53 bits.)  A block takes 16 rows of
+// 256 columns.
 constexpr int kPlaneRows = 16;
 template <typename T>
 __global__ void __launch_bounds__(kThreads) k_simt_planes(int64_t m, int64_t n, int64_t c0, int64_t ldk,
@@ -151,25 +151,14 @@ __global__ void __launch_bounds__(kThreads) k_simt_planes(int64_t m, int64_t n, 
   if (k >= ldk) return;
   const bool in = c0 + k < n;
   const double d = in ? __ldg(D + c0 + k) : 0.0;
-  const float dh = (float)d, dl = (float)(d - (double)dh);
-  const bool pair = sizeof(T) < 8 && fabs(d) < 0x1p100 && (fabs(d) > 0x1p-100 || d == 0.0);
   for (int64_t p0 = (int64_t)blockIdx.y * kPlaneRows; p0 < m; p0 += (int64_t)gridDim.y * kPlaneRows) {
 #pragma unroll 8
     for (int r = 0; r < kPlaneRows; ++r) {
       const int64_t p = p0 + r;
       if (p >= m) break;
       const T a = in ? A[p * n + c0 + k] : T(0.f);
-      const float af = widen32(a);
-      float b;
-      if (pair) {
-        const float h = af * dh;
-        b = h + fmaf(af, dl, fmaf(af, dh, -h));
-        if (!isfinite(h)) b = h;
-      } else {
-        b = (float)(widen(a) * d);
-      }
-      Bp[p * ldk + k] = b;
-      Ap[p * ldk + k] = af;
+      Bp[p * ldk + k] = (float)(widen_int(a) * d);
+      Ap[p * ldk + k] = widen32(a);
     }
   }
 }
