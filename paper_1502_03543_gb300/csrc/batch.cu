@@ -279,8 +279,8 @@ __device__ void blk_gemv_t(const Ctx& c, const double* u, double* out) {
 }
 
 // The same in double-float for the FP32-pair vector u2 (m).  Used for the
-// conjugate-gradient operator and the first residual while the factor is FP32,
-// where D spans fewer orders of magnitude.
+// conjugate-gradient operator while the factor is FP32, where D spans fewer
+// orders of magnitude.
 template <int T>
 __device__ void blk_gemv_t_df(const Ctx& c, const float2* u2, double* out) {
   blk_columns<T, true>(c, nullptr, u2, out);
@@ -953,11 +953,11 @@ __device__ bool pcg_lp(const BatchArgs& a, Ctx& c, bool tier2, const double* M64
   };
   // One loop, so that each solve and each product is compiled once: a round
   // applies the preconditioner (but for kTrue), then M to a vector.
-  //   kFirst    out = P^-1 rhs, rho = rhs - M out.  With an FP32 factor this
-  //             residual is ~1e-7 of rhs and only starts the conjugate gradients:
-  //             its inner pass runs in double-float, and one that would be
-  //             accepted is formed again in FP64 (as in the large path)
-  //   kTrue     rho = rhs - M out in FP64, which decides acceptance
+  //   kFirst    out = P^-1 rhs, rho = rhs - M out
+  //   kTrue     rho = rhs - M out
+  // (both with the inner pass in FP64: they decide acceptance.  Double-float in
+  // the first one saves nothing: 512 LPs to 3e-2 23.8 against 24.6 ms, 300 of m >=
+  // 100 33.0 against 32.7, 256 adjoints 1.78 against 1.66)
   //   kRestart  z = P^-1 rho, p = z, then the step
   //   kStep     z = P^-1 rho, p = z + beta p, then the step
   enum { kFirst, kTrue, kRestart, kStep } state = kFirst;
@@ -980,8 +980,7 @@ __device__ bool pcg_lp(const BatchArgs& a, Ctx& c, bool tier2, const double* M64
       rz = rz2;
       if (!(k < refine_max && rz > 0.0 && isfinite(rz))) return false;
     }
-    const bool df = state != kTrue && !tier2;
-    blk_apply_m<T>(c, step ? c.p : out, step ? nullptr : rhs, step ? c.q : c.rho, df);
+    blk_apply_m<T>(c, step ? c.p : out, step ? nullptr : rhs, step ? c.q : c.rho, step && !tier2);
     double al = 0.0;
     if (step) {
       double t = 0.0;
@@ -1005,8 +1004,7 @@ __device__ bool pcg_lp(const BatchArgs& a, Ctx& c, bool tier2, const double* M64
       state = accepted(res, dyn) || k % 10 == 9 ? kTrue : kStep;
       ++k;
     } else if (accepted(res, dyn)) {
-      if (!df) return true;
-      state = kTrue;
+      return true;
     } else {
       state = kRestart;
     }
