@@ -702,6 +702,12 @@ bool retry_simt(pdas_ctx* h, pdas_status st) {
   h->plain_simt = true;
   return true;
 }
+// The end of a call that may have been done over: the next one starts with the
+// tensor-core factor again.
+void end_retry(pdas_ctx* h) {
+  if (h->plain_simt) h->no_dffactor_once = false;
+  h->plain_simt = false;
+}
 
 // One step in place, up to the device's status; *read: it was read.
 pdas_status step_once(pdas_ctx* h, const void* A, const double* b, const double* c, double* x, double* y, double* s,
@@ -737,7 +743,7 @@ pdas_status direction_out(pdas_ctx* h, const void* A, const double* x, const dou
     st = device_status(h);
     fill_info(h, info, false);
   } while (retry_simt(h, st));
-  h->plain_simt = false;
+  end_retry(h);
   return st;
 }
 
@@ -1025,7 +1031,7 @@ pdas_status pdas_step(pdas_handle h, const void* A, const double* b, const doubl
     h->err_index = -1;
     st = step_once(h, A, b, c, x, y, s, alpha, variant ? &iv : nullptr, &read);
   } while (retry_simt(h, st));
-  h->plain_simt = false;
+  end_retry(h);
   if (read) fill_info(h, info, st == PDAS_OK);
   if (st != PDAS_OK) return st;
   h->last_rel_gap = variant ? fmax(fabs(h->sc_host->rel_gap), fmax(h->sc_host->pres, h->sc_host->dres))
@@ -1184,9 +1190,24 @@ pdas_status pdas_factor(pdas_handle h) {
   h->err_index = -1;
   pdas_status st = reset_status(h);
   if (st != PDAS_OK) return st;
+  // The plain form's tensor-core factor overwrites M: M is kept in its upper
+  // triangle meanwhile, for the SIMT factor's own verdict on a failed pivot.
+  const bool keep = !is_mixed(h) && h->cdig.m > 0;
+  if (keep) KL(launch_mirror_lower(h->st, h->m, h->ldm, h->M64, h->kq, false), 1);
   if ((st = factor(h)) != PDAS_OK) return st;
   if ((st = read_scalars(h)) != PDAS_OK) return st;
   st = device_status(h);
+  if (keep && st == PDAS_ERR_NOT_SPD) {
+    h->err_index = -1;
+    if ((st = reset_status(h)) != PDAS_OK) return st;
+    KL(launch_mirror_lower(h->st, h->m, h->ldm, h->M64, h->kq, true), 1);
+    h->no_dffactor_once = true;
+    st = factor(h);
+    h->no_dffactor_once = false;
+    if (st != PDAS_OK) return st;
+    if ((st = read_scalars(h)) != PDAS_OK) return st;
+    st = device_status(h);
+  }
   h->have_factor = st == PDAS_OK;
   return st;
 }

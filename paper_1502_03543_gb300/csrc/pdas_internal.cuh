@@ -232,6 +232,10 @@ cudaError_t launch_adjoint_update(cudaStream_t st, int64_t n, const double* D, c
 cudaError_t launch_adjoint_dA(cudaStream_t st, int64_t m, int64_t n, const double* la, const double* x,
                               const double* y, const double* lb, double* dA, const Scalars* sc);
 
+// The lower triangle of M kept in its upper one (the diagonal in diag, m
+// doubles), or put back from there.
+cudaError_t launch_mirror_lower(cudaStream_t st, int64_t m, int64_t ldm, double* M, double* diag, bool put_back);
+
 cudaError_t launch_convert_matrix(cudaStream_t st, int64_t m, int64_t ld_src, const void* src, int src_f64,
                                   int64_t ld_dst, void* dst, int dst_f64);
 

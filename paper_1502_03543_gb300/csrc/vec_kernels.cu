@@ -488,9 +488,35 @@ __global__ void k_convert_matrix(int64_t m, int64_t ld_src, const void* src, int
 }
 
 
+// One 32 x 32 tile (i, j), i >= j, per block of 32 x 8 threads; through shared
+// memory, so that both triangles are read and written by rows.
+__global__ void k_mirror_lower(int64_t m, int64_t ldm, double* M, double* diag, int put_back) {
+  if (blockIdx.x > blockIdx.y) return;
+  __shared__ double t[32][33];
+  const int64_t p0 = (int64_t)blockIdx.y * 32, q0 = (int64_t)blockIdx.x * 32;
+  const int64_t s0 = put_back ? q0 : p0, s1 = put_back ? p0 : q0;  // the tile read: rows s0.., columns s1..
+  const int x = threadIdx.x;
+  for (int y = threadIdx.y; y < 32; y += blockDim.y)
+    if (s0 + y < m && s1 + x < m) t[y][x] = M[(s0 + y) * ldm + s1 + x];
+  __syncthreads();
+  for (int y = threadIdx.y; y < 32; y += blockDim.y) {
+    const int64_t r = s1 + y, c = s0 + x;  // the entry written, the transpose of (c, r)
+    if (r >= m || c >= m) continue;
+    if (put_back ? r > c : r < c) M[r * ldm + c] = t[x][y];
+    else if (r == c && put_back) M[r * ldm + c] = diag[r];
+    else if (r == c) diag[r] = t[x][y];
+  }
+}
+
 }  // namespace
 
 // ---------------------------------------------------------------------------
+cudaError_t launch_mirror_lower(cudaStream_t st, int64_t m, int64_t ldm, double* M, double* diag, bool put_back) {
+  const unsigned t = (unsigned)((m + 31) / 32);
+  k_mirror_lower<<<dim3(t, t), dim3(32, 8), 0, st>>>(m, ldm, M, diag, put_back ? 1 : 0);
+  return cudaGetLastError();
+}
+
 template <typename T>
 cudaError_t launch_gemv_t(cudaStream_t st, int64_t m, int64_t n, const T* A, const double* u, double* part,
                           int chunks, int64_t rows_per_chunk) {
