@@ -420,6 +420,12 @@ __global__ void __launch_bounds__(PR_THREADS) k_dig_panel_rows(int64_t ldm, doub
     const int64_t i = r0 + rr;
     if (i >= rows) break;
     const double v0 = X[rr][2 * lane], v1 = X[rr][2 * lane + 1];
+    // Digits cannot hold an infinity or a NaN (and fmax drops a NaN): the row's
+    // pivot gets one, which the updates keep, and fails when its turn comes, as
+    // it does where the products are formed in floating point.
+    const bool odd = (__double2hiint(v0) & 0x7ff00000) == 0x7ff00000 || (__double2hiint(v1) & 0x7ff00000) == 0x7ff00000;
+    if (__any_sync(0xffffffffu, odd) && lane == 0)
+      M[(k0 + kb + i) * ldm + k0 + kb + i] = __longlong_as_double(0x7ff8000000000000ll);
     double mx = fmax(fabs(v0), fabs(v1));
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
