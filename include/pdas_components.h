@@ -79,11 +79,12 @@ pdas_status pdas_gemv_t(pdas_handle h, const void* A, const double* u, double* o
  * (i, l) by tile columns i and l of step k <= l - 2, or of step k = l - 1 when
  * i = l + 1; 3 = inverse of L_ll (for the blocked triangular solves); 4 =
  * triangular solve of the sub-diagonal tile (l + 1, l) against L_ll, all its
- * updates applied (k = l).  One CTA runs kinds 0 and 4 in the order 0(0),
- * 4(1,0), 0(1), 4(2,1), ...; the others take the rest in list order.  Returns
- * the count (0 for m <= 0); out may be NULL to query it.  Every task comes
- * after the tasks it waits for, which is what makes the launch
- * deadlock-free. */
+ * updates applied (k = l).  Kinds 0 and 4 are the dependency chain 0(0), 4(1,0),
+ * 0(1), 4(2,1), ...; the FP32 factor runs it in two CTAs, which take tile rows in
+ * turn and also apply the kind-2 updates with k = l - 1, the double-float factor
+ * in one.  The other CTAs take the rest in list order.  Returns the count (0 for
+ * m <= 0); out may be NULL to query it.  Every task comes after the tasks it
+ * waits for, which is what makes the launch deadlock-free. */
 int64_t pdas_chol_tile_tasks(int64_t m, int32_t nproc, int32_t* out, int64_t cap);
 
 /* Host-only.  How far the FP32 factor's 16-byte loads of the 32-column panels

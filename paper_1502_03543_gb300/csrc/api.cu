@@ -244,7 +244,7 @@ pdas_status reset_status(pdas_ctx* h) {
   return PDAS_OK;
 }
 
-// A v -> out (base == null) or base - A v -> out; norm_slot as in launch_gemv.
+// A v -> out (base == null) or base - A v -> out; norm_slot as in launch_pass.
 // Double-float passes over A (passes.cu) are available to the mixed forms
 // when A is exact in FP32 (stored as FP32 or BF16) and exact_passes is off.
 // The solve uses them only for the conjugate-gradient operator M p of the
@@ -651,7 +651,7 @@ pdas_status direction(pdas_ctx* h, const void* A, const double* x, const double*
       // w = A' dy of the accepted dy is in h->w: dx = D w - x, ds = -w.  (An
       // FP64 factor is the last tier: its refined direction is used as is.)
       STAGE(h, PDAS_STAGE_DIR);
-      KL(launch_gemv_t_finish(h->st, h->n, 0, nullptr, 3, x, h->D, h->dx, h->ds, h->w, h->sc, rd), 1);
+      KL(launch_direction(h->st, h->n, h->w, x, h->D, h->dx, h->ds, h->sc, rd), 1);
       STAGE_END(h);
       return PDAS_OK;
     }
@@ -922,10 +922,14 @@ pdas_status pdas_create(int64_t m, int64_t n, const pdas_options* opt_in, pdas_h
   }
   if (e == cudaSuccess && opt.form != PDAS_FP64 && opt.a_dtype == PDAS_A_BF16 && opt.fp64_tier_tc)
     e = dig_workspace_create(&h->dig, m, n);
-  // (The plain form takes this factor up to kFp64FormDigMaxM rows.  Whole solves to 1e-8 with it and with the
-  // SIMT factor end with the same residuals and counts at most one apart up to 4096 x 16384 (13.3 -> 11.8 s); at
-  // 8192 x 32768, where nothing refines the end game and the factor is 4 % of the time (115 -> 110 s), the solve
-  // took 55 iterations in place of 53 and ended at a relative gap of -2.6e-8 in place of 9e-10.)
+  // (The plain form takes this factor up to kFp64FormDigMaxM rows.  Nothing refines its end game, and there the
+  // last digits of a run belong to the rounding: 20 LPs of m = 256 to 6144 solved to 1e-8, each in two orders of its
+  // rows, end with the same residuals with this factor and the SIMT one, and their iteration counts differ as those
+  // of the two orders do, by one or two, in either direction.  At 8192 x 32768 one order of four runs stood out: 55
+  // iterations to a relative gap of -2.6e-8 with this factor, where the other order takes 53 to 5.9e-9 and the SIMT
+  // factor 53 in both, to 9.4e-10 and 7.7e-9.  Beyond 4096 the factor is less than 10 % of the time (98 against 107
+  // s at 8192, 11.1 against 12.6 at 4096, 0.2 against 0.4 at 1024), so the line lies on the side where what a solve
+  // returned stays as it was.)
   if (e == cudaSuccess && opt.fp64_tier_tc && (opt.form == PDAS_FP64 ? m <= kFp64FormDigMaxM : m > kCholDigMinM))
     e = chol_dig_create(&h->cdig, m);
   if (e == cudaSuccess && (opt.form == PDAS_BF16_IR || opt.form == PDAS_TF32_IR)) {

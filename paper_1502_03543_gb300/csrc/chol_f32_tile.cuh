@@ -73,26 +73,6 @@ __device__ __forceinline__ void put_tile(const float4 (&x)[16], int64_t m, int64
   }
 }
 
-// The tile to rows p0.., columns q0.. of M (diag: the lower triangle).
-__device__ __forceinline__ void store_tile(const float (*T)[kPt], int64_t m, int64_t ldm, float* M, int64_t p0,
-                                           int64_t q0, bool diag) {
-#pragma unroll
-  for (int v = 0; v < 16; ++v) {
-    int r, c;
-    unit_rc(v, r, c);
-    if (p0 + r >= m || (diag && c > r)) continue;
-    float* dst = M + (p0 + r) * ldm + q0 + c;
-    const float e[4] = {T[c][r], T[c + 1][r], T[c + 2][r], T[c + 3][r]};
-    if (q0 + c + 3 < m && (!diag || c + 3 <= r)) {
-      *reinterpret_cast<float4*>(dst) = make_float4(e[0], e[1], e[2], e[3]);
-    } else {
-#pragma unroll
-      for (int k = 0; k < 4; ++k)
-        if (q0 + c + k < m && (!diag || c + k <= r)) dst[k] = e[k];
-    }
-  }
-}
-
 // Hardware estimates of 1 / d and 1 / sqrt(d) for normal d (within 2 ulp; the
 // FP32 factor is a preconditioner, and every entry of a column is scaled by
 // the same value).

@@ -16,13 +16,12 @@
 // of chol_f32_tile.cuh; the double-float instantiation keeps SIMT products and
 // the tile operations below.
 // A tile's last update and its factorisation or triangular solve run in one
-// task on the tile held in registers (except the sub-diagonal tiles, see
-// below), and the dependency chain of the factorisation (FINAL(l,l) ->
-// SOLVE(l+1,l) -> FINAL(l+1,l+1) ...) runs in one CTA.  Every tile (i, l) of
-// the lower triangle has a counter in global memory: the number of updates
-// applied to it, then l + 1 once it holds its final L values.
+// task on the tile held on the SM (except the sub-diagonal tiles, see below).
+// Every tile (i, l) of the lower triangle has a counter in global memory: the
+// number of updates applied to it, then l + 1 once it holds its final L values.
 //
-// The dependency chain runs in CTAs of its own, so that its head never queues
+// The dependency chain of the factorisation (FINAL(l,l) -> SOLVE(l+1,l) ->
+// FINAL(l+1,l+1) ...) runs in CTAs of its own, so that its head never queues
 // behind trailing updates: in the FP32 factor in blocks 0 and 1 (chol_chain),
 // tile rows in turn, so that the solve of a sub-diagonal tile runs beside the
 // factorisation it depends on, panel by panel; these also apply that tile's last
@@ -61,18 +60,13 @@ namespace {
 
 enum TileTask { TK_FINAL_DIAG = 0, TK_FINAL_OFF = 1, TK_UPDATE = 2, TK_INV = 3, TK_CHAIN_SOLVE = 4 };
 
-// UPDATE operands: K chunks of 32 columns of two 128-row tile columns,
-// row-major with a pitch of 36 floats / 34 doubles (16-byte rows, and 16
-// consecutive rows fall in distinct 16-byte bank groups), double-buffered.
+// UPDATE operands of the double-float factor: K chunks of 32 columns of two
+// 128-row tile columns, row-major with a pitch of 34 8-byte elements (16-byte
+// rows, and 16 consecutive rows fall in distinct 16-byte bank groups),
+// double-buffered.
 constexpr int kUpdK = 32;
-template <typename T>
-constexpr int upd_pitch() {
-  return sizeof(T) == 4 ? 36 : 34;
-}
-template <typename T>
-constexpr int upd_vec() {  // elements per 16-byte load
-  return 16 / (int)sizeof(T);
-}
+constexpr int kUpdPitch = 34;
+constexpr int kUpdVec = 2;  // elements per 16-byte load
 
 // Tensor-core products (FP32 factor).  Every finished off-diagonal tile of L
 // is stored once more as three BF16 planes (x = x0 + x1 + x2, 8 significant
@@ -100,7 +94,7 @@ constexpr int kChainOps = 100 * 1024;
 template <typename T>
 struct TileCholSmem {
   union {
-    T stage[2][2][kBig][upd_pitch<T>()];  // UPDATE (FP64): [buffer][row tile i | row tile l][row][k]
+    T stage[2][2][sizeof(T) == 4 ? 1 : kBig][kUpdPitch];  // UPDATE (double-float): [buffer][row tile i | row tile l][row][k]
     T ls[sizeof(T) == 4 ? 1 : kBig][kBig + 1];  // TRSM (double-float): the factor of the diagonal tile
     struct {
       float c[kBig][ft::kPt];      // FP32: the tile to be solved
@@ -187,7 +181,8 @@ __device__ __forceinline__ void store_tile(const T (&acc)[8][8], T* M, int64_t l
 template <typename T, bool DIAG>
 __device__ __forceinline__ void rank_update(T (&acc)[8][8], int64_t m, int64_t ldm, const T* M, int i, int l, int k,
                                             TileCholSmem<T>& sm) {
-  constexpr int VEC = upd_vec<T>();
+  constexpr int VEC = kUpdVec;
+  static_assert(sizeof(T) == 8, "the FP32 factor's products run on the tensor cores");
   constexpr int CPR = kUpdK / VEC;  // 16-byte copies per row and chunk
   struct alignas(16) V {
     T v[VEC];
@@ -217,8 +212,8 @@ __device__ __forceinline__ void rank_update(T (&acc)[8][8], int64_t m, int64_t l
     if (ch + 1 < NCH) cp_async_wait<1>();
     else cp_async_wait<0>();
     __syncthreads();
-    const T(*P)[upd_pitch<T>()] = sm.stage[buf][0];
-    const T(*Q)[upd_pitch<T>()] = sm.stage[buf][DIAG ? 0 : 1];
+    const T(*P)[kUpdPitch] = sm.stage[buf][0];
+    const T(*Q)[kUpdPitch] = sm.stage[buf][DIAG ? 0 : 1];
 #pragma unroll 1
     for (int kk = 0; kk < kUpdK; kk += VEC) {
       V a[8];

@@ -60,8 +60,8 @@ pdas_status scratch_on_current_device(unsigned char** out) {
 template <typename T>
 cudaError_t run(cudaStream_t st, int64_t m, int64_t n, const void* A, const double* u, double* out,
                 unsigned char* base) {
-  // The row-chunk split of the handle's pdas_gemv_t (chunks of at least 16
-  // rows, at most 64 chunks), coarsened when the partials would not fit.
+  // Chunks of at least 16 rows, at most 64 of them, fewer where their partials
+  // would not fit.
   int64_t rows = (m + 63) / 64;
   if (rows < 16) rows = 16;
   int64_t chunks = (m + rows - 1) / rows;
@@ -76,7 +76,7 @@ cudaError_t run(cudaStream_t st, int64_t m, int64_t n, const void* A, const doub
   if (e != cudaSuccess) return e;
   e = pdas::launch_gemv_t<T>(st, m, n, static_cast<const T*>(A), u, part, (int)chunks, rows);
   if (e != cudaSuccess) return e;
-  return pdas::launch_gemv_t_finish(st, n, (int)chunks, part, 0, nullptr, nullptr, out, nullptr, nullptr, sc);
+  return pdas::launch_gemv_t_sum(st, n, (int)chunks, part, out, sc);
 }
 
 }  // namespace

@@ -416,7 +416,7 @@ __global__ void __launch_bounds__(kThreads, DF ? 2 : sizeof(T) == 8 ? 5 : 3) k_p
   const int nr = (int)(m - p0 < R ? m - p0 : R);
   const T* rows[R];
 #pragma unroll
-  for (int r = 0; r < R; ++r) rows[r] = A + (p0 + (r < nr ? r : 0)) * n;  // (a row past m reads row 0 and is dropped)
+  for (int r = 0; r < R; ++r) rows[r] = A + (p0 + (r < nr ? r : 0)) * n;  // (a row past m reads the CTA's first and is dropped)
   double acc[R];
 #pragma unroll
   for (int r = 0; r < R; ++r) acc[r] = 0.0;

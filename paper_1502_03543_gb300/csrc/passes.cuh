@@ -14,7 +14,7 @@ struct PassTPlan {
 };
 PassTPlan pass_t_plan(int64_t m, int64_t n, int elem_bytes, bool vec);
 // Workspace of any plan of (m, n): doubles of partial column sums, tickets
-// (zero between launches), and the largest number of chunks.
+// (zero between launches).
 int64_t pass_t_part_doubles(int64_t m, int64_t n, int elem_bytes);
 int64_t pass_t_tickets(int64_t n);
 
@@ -36,7 +36,7 @@ struct PassTSrc {
   int absmax = 0;  // max |u| into sc->dynorm
 };
 
-// w = A'u, then per mode (as launch_gemv_t_finish):
+// w = A'u, then per mode:
 //   0: out0 = w
 //   1: direction: out0 = dx = D w - x, out1 = ds = -w, out2 = w (may be null)
 //   2: scaled:    out0 = D w (may be null), out2 = w (may be null), and with pairs != null the

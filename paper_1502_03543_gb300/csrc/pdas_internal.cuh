@@ -86,15 +86,13 @@ template <typename T>
 cudaError_t launch_gemv_t(cudaStream_t st, int64_t m, int64_t n, const T* A, const double* u, double* part,
                           int chunks, int64_t rows_per_chunk);
 
-// w = sum of the gemv_t partials; then per mode:
-//   0: out0 = w
-//   1: direction: out0 = dx = D w - x, out1 = ds = -w, out2 = w (may be null)
-//   2: scaled:    out0 = D w, out2 = w (may be null)
-//   3: direction from a w already in out2 (chunks, part unused)
-// With rd (modes 1 and 3, the infeasible-start variant) ds = rd - w instead of -w.
-cudaError_t launch_gemv_t_finish(cudaStream_t st, int64_t n, int chunks, const double* part, int mode,
-                                 const double* x, const double* D, double* out0, double* out1, double* out2,
-                                 const Scalars* sc, const double* rd = nullptr);
+// out = the sum of those partials.
+cudaError_t launch_gemv_t_sum(cudaStream_t st, int64_t n, int chunks, const double* part, double* out,
+                              const Scalars* sc);
+// The direction from w = A'dy: ds = -w, dx = D w - x; with rd (the
+// infeasible-start variant) ds = rd - w, dx = D (w - rd) - x.
+cudaError_t launch_direction(cudaStream_t st, int64_t n, const double* w, const double* x, const double* D, double* dx,
+                             double* ds, const Scalars* sc, const double* rd = nullptr);
 // Infeasible-start variant: rd = (c - w) - s (w = A'y) and nu = -(D rd), so
 // that b - A nu = b + A D rd is the right-hand side of the normal equations.
 cudaError_t launch_dual_residual(cudaStream_t st, int64_t n, const double* c, const double* s, const double* w,
@@ -156,7 +154,7 @@ int64_t chol_tile_count(int64_t m);
 int chol_tiles_resident();  // resident CTAs on the current device, 0 on error
 void chol_tile_tasks(int64_t m, int nproc, std::vector<int4>* out);
 // Uinv receives U_l = L_ll^{-T} for every diagonal tile (nb x 128 x 128,
-// row-major per tile), for trsv_lower_blk / trsv_upper_blk.
+// row-major per tile), for trsv_blk_solve.
 template <typename T>
 cudaError_t cholesky_tiles(cudaStream_t st, int64_t m, int64_t ldm, T* M, T* dinv, T* Uinv, const int4* tasks,
                            int ntasks, int* state, Scalars* sc, unsigned char* planes);

@@ -120,30 +120,27 @@ __global__ void __launch_bounds__(kThreads) k_gemv_t_part(int64_t m, int64_t n, 
   }
 }
 
-// a7 (second half): w_j = sum_c part[c][j] in chunk order, then the mode's
-// elementwise outputs.
-__global__ void __launch_bounds__(kThreads) k_gemv_t_finish(int64_t n, int chunks, const double* __restrict__ part,
-                                                            int mode, const double* __restrict__ x,
-                                                            const double* __restrict__ D, double* out0,
-                                                            double* out1, double* out2, const Scalars* sc,
-                                                            const double* __restrict__ rd) {
+// out_j = sum_c part[c][j] in chunk order.
+__global__ void __launch_bounds__(kThreads) k_gemv_t_sum(int64_t n, int chunks, const double* __restrict__ part,
+                                                         double* __restrict__ out, const Scalars* sc) {
   if (failed(sc)) return;
   for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x) {
     double w = 0.0;
-    if (mode == 3) w = out2[j];
-    else
-      for (int c = 0; c < chunks; ++c) w += __ldcg(part + (int64_t)c * n + j);
-    if (mode == 0) {
-      out0[j] = w;
-    } else if (mode == 1 || mode == 3) {
-      const double ds = rd ? rd[j] - w : -w;
-      out0[j] = D[j] * (-ds) - x[j];  // dx = D(-ds) - x
-      out1[j] = ds;
-      if (out2 && mode == 1) out2[j] = w;
-    } else {
-      out0[j] = D[j] * w;
-      if (out2) out2[j] = w;
-    }
+    for (int c = 0; c < chunks; ++c) w += __ldcg(part + (int64_t)c * n + j);
+    out[j] = w;
+  }
+}
+
+// The direction from w = A'dy (a7): ds = -w (or rd - w), dx = D(-ds) - x.
+__global__ void __launch_bounds__(kThreads) k_direction(int64_t n, const double* __restrict__ w,
+                                                        const double* __restrict__ x, const double* __restrict__ D,
+                                                        double* __restrict__ dx, double* __restrict__ ds_out,
+                                                        const Scalars* sc, const double* __restrict__ rd) {
+  if (failed(sc)) return;
+  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x) {
+    const double ds = rd ? rd[j] - w[j] : -w[j];
+    dx[j] = D[j] * (-ds) - x[j];
+    ds_out[j] = ds;
   }
 }
 
@@ -527,10 +524,15 @@ cudaError_t launch_gemv_t(cudaStream_t st, int64_t m, int64_t n, const T* A, con
   return cudaGetLastError();
 }
 
-cudaError_t launch_gemv_t_finish(cudaStream_t st, int64_t n, int chunks, const double* part, int mode,
-                                 const double* x, const double* D, double* out0, double* out1, double* out2,
-                                 const Scalars* sc, const double* rd) {
-  k_gemv_t_finish<<<grid_for(n), kThreads, 0, st>>>(n, chunks, part, mode, x, D, out0, out1, out2, sc, rd);
+cudaError_t launch_gemv_t_sum(cudaStream_t st, int64_t n, int chunks, const double* part, double* out,
+                              const Scalars* sc) {
+  k_gemv_t_sum<<<grid_for(n), kThreads, 0, st>>>(n, chunks, part, out, sc);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_direction(cudaStream_t st, int64_t n, const double* w, const double* x, const double* D, double* dx,
+                             double* ds, const Scalars* sc, const double* rd) {
+  k_direction<<<grid_for(n), kThreads, 0, st>>>(n, w, x, D, dx, ds, sc, rd);
   return cudaGetLastError();
 }
 
