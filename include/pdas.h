@@ -61,7 +61,9 @@ typedef enum {
                        split into TF32 parts each call, see splits; A stored as FP64 or
                        FP32), FP32 factor, FP64 refinement of dy                         */
   PDAS_BF16_IR = 2, /* as TF32_IR with BF16 operands (needs A stored as BF16)            */
-  PDAS_FP32_IR = 3  /* M formed with FP32 SIMT arithmetic, FP32 factor, FP64 refinement  */
+  PDAS_FP32_IR = 3  /* M formed with FP32 SIMT arithmetic, FP32 factor, FP64 refinement.
+                       The handle holds two FP32 operand planes of A's size (8 m n bytes,
+                       at most 4 GB)                                                     */
 } pdas_form;
 
 /* Storage dtype of A; every form reads A in this dtype and widens it exactly. */
@@ -118,7 +120,11 @@ typedef struct {
                               0 = double-float formation (normal_form 2) and the factors of
                               df_factor_floor.  PDAS_FP64: 1 = the factor of (b) for m <= 4096 (a
                               matrix that it finds not positive definite is factored again on the
-                              SIMT pipes); 0 = the SIMT factor                                 (1) */
+                              SIMT pipes); 0 = the SIMT factor.  The factor of (b) holds a panel
+                              row to 2^-56 of its largest entry: |L L' - M|_pq <= c u sqrt(M_pp
+                              M_qq), accurate relative to the rows' scale; the SIMT factor's
+                              elementwise bound c u (|L||L'|)_pq is smaller where rows are graded
+                              in opposite directions                                           (1) */
   double df_factor_floor;  /* mixed forms in the FP64 tier without the tensor-core factor: the
                               factor is the double-float tile factor (FP32 pipes) while the
                               relative gap of the iterate is above this, the FP64 SIMT factor
