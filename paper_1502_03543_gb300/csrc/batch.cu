@@ -940,9 +940,15 @@ __device__ bool factor_lp(const BatchArgs& a, Ctx& c, bool& tier2, double* M64, 
 // <= refine_tol ||rhs||_inf or <= refine_tol (mnorm ||out||_inf +
 // ||rhs||_inf).  Uses c.rho, c.z, c.p, c.q; when accepted c.w = A' out (from
 // the FP64 residual that decided it).  Returns whether the tolerance was met within refine_max steps.
+// correction: the solve improves an accepted one.  Its right-hand side is small,
+// its residual is rounding near the tolerance, and now and then stays a little
+// above it (1.05 to 1.4 times) for tens of restarts, each of which ended a batch
+// of 256 later: 5 ms in place of 2.  So the third FP64 residual that is more than half of
+// the one before ends it, with 4 times the tolerance (of 16416 corrections 9 got
+// there, with at most 2 times; all were accepted in the end).
 template <int T>
 __device__ bool pcg_lp(const BatchArgs& a, Ctx& c, bool tier2, const double* M64, const double* dinv64,
-                       double mnorm, const double* rhs, double* out, int refine_max) {
+                       double mnorm, const double* rhs, double* out, int refine_max, bool correction) {
   const int m = c.m;
   double rn = 0.0;
   for (int i = threadIdx.x; i < m; i += T) rn = fmax(rn, fabs(rhs[i]));
@@ -961,7 +967,8 @@ __device__ bool pcg_lp(const BatchArgs& a, Ctx& c, bool tier2, const double* M64
   //   kRestart  z = P^-1 rho, p = z, then the step
   //   kStep     z = P^-1 rho, p = z + beta p, then the step
   enum { kFirst, kTrue, kRestart, kStep } state = kFirst;
-  double rz = 0.0;
+  double rz = 0.0, last = INFINITY;
+  int stalls = 0;
   for (int k = 0;;) {
     if (state != kTrue) {
       const double* v = state == kFirst ? rhs : c.rho;
@@ -1006,6 +1013,11 @@ __device__ bool pcg_lp(const BatchArgs& a, Ctx& c, bool tier2, const double* M64
     } else if (accepted(res, dyn)) {
       return true;
     } else {
+      if (correction) {
+        stalls += res > 0.5 * last;
+        last = res;
+        if (stalls == 3) return accepted(0.25 * res, dyn);
+      }
       state = kRestart;
     }
   }
@@ -1054,7 +1066,7 @@ __device__ void solve_lp(const BatchArgs& a, const BatchLP lp, Ctx& c, int& stat
     }
     if (tier2) ++n_shift;
     // w = A' dy (there if dy was accepted); dx = D w - x; ds = -w
-    if (!pcg_lp<T>(a, c, tier2, M64, dinv64, mnorm, c.r, c.dy, a.refine_max)) {
+    if (!pcg_lp<T>(a, c, tier2, M64, dinv64, mnorm, c.r, c.dy, a.refine_max, false)) {
       ++n_unref;
       blk_gemv_t<T>(c, c.dy, c.w);
       __syncthreads();
@@ -1234,7 +1246,7 @@ __device__ int adjoint_lp(const AdjointArgs& g, const BatchLP lp, Ctx& c) {
     }
     blk_gemv<T>(c, c.un2, nullptr, c.r);  // r = A D g, then A (D r1 - r3 - lb)
     __syncthreads();
-    if (!pcg_lp<T>(a, c, tier2, M64, dinv64, mnorm, c.r, c.dy, 4 * a.refine_max)) {
+    if (!pcg_lp<T>(a, c, tier2, M64, dinv64, mnorm, c.r, c.dy, 4 * a.refine_max, it > 0)) {
       if (it == 0) return PDAS_ERR_NOT_SPD;
       break;  // (no correction that meets the tolerance: it is at the rounding level; keep what we have)
     }
