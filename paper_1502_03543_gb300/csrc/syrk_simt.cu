@@ -168,7 +168,7 @@ __global__ void __launch_bounds__(kThreads) k_simt_planes(int64_t m, int64_t n, 
 // Thread (tx, ty) owns rows 4 ty .. + 3 and 64 + 4 ty .. + 3 and the same of
 // columns by tx, so a step reads four 16-byte vectors for 64 multiply-adds.
 // Bound by the FP32 pipe.  Measured at 1001 x 3003 (36 tiles): 774 us as 36 CTAs
-// with the FP64 products in the loads -> 120 us with the planes and 8 K slices
+// with the FP64 products in the loads -> 113 us with the planes and 8 K slices
 // (288 CTAs; the multiply-adds alone take 46 us).
 constexpr int kPitch = kBig + 4;
 
