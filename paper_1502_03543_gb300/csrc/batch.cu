@@ -1309,9 +1309,9 @@ constexpr int kBuckets = 4;  // m in [1, 64], (64, 128], (128, 192], (192, 256]
 constexpr int kCandidates[3] = {128, 256, 512};
 
 cudaError_t set_smem_attr(int threads, size_t bytes) {
-  if (threads == 128) return cudaFuncSetAttribute(k_batch<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (threads == 256) return cudaFuncSetAttribute(k_batch<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  return cudaFuncSetAttribute(k_batch<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (threads == 128) return allow_smem(k_batch<128>, bytes);
+  if (threads == 256) return allow_smem(k_batch<256>, bytes);
+  return allow_smem(k_batch<512>, bytes);
 }
 cudaError_t occupancy(int threads, size_t bytes, int* blocks) {
   if (threads == 128) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, k_batch<128>, 128, bytes);
@@ -1328,10 +1328,10 @@ cudaError_t launch(int threads, int grid, size_t bytes, cudaStream_t st, const B
 // and CTA size; its grid comes from its own occupancy.
 cudaError_t set_adjoint_smem_attr(int threads, size_t bytes) {
   if (threads == 128)
-    return cudaFuncSetAttribute(k_batch_adjoint<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    return allow_smem(k_batch_adjoint<128>, bytes);
   if (threads == 256)
-    return cudaFuncSetAttribute(k_batch_adjoint<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  return cudaFuncSetAttribute(k_batch_adjoint<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    return allow_smem(k_batch_adjoint<256>, bytes);
+  return allow_smem(k_batch_adjoint<512>, bytes);
 }
 cudaError_t adjoint_occupancy(int threads, size_t bytes, int* blocks) {
   if (threads == 128) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, k_batch_adjoint<128>, 128, bytes);
@@ -1700,7 +1700,7 @@ pdas_status pdas_batch_create(int count, const int* m, const int* n, const float
     if ((st = grid_for_bucket(h, bi, B.threads, &B.grid)) != PDAS_OK) return fail(st);
   }
   if (opt.autotune && (st = autotune(h, no, mo)) != PDAS_OK) return fail(st);
-  for (int bi = 0; bi < kBuckets; ++bi) {  // (the attribute is per function: set it for the final choice)
+  for (int bi = 0; bi < kBuckets; ++bi) {  // the final choice
     auto& B = h->bk[bi];
     if (B.count && (st = grid_for_bucket(h, bi, B.threads, &B.grid)) != PDAS_OK) return fail(st);
     if (B.count) {  // the adjoint kernel of the bucket: same CTA size and shared memory

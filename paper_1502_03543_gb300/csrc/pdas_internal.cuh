@@ -80,6 +80,23 @@ __device__ __forceinline__ float widen32(float v) { return v; }
 __device__ __forceinline__ float widen32(__nv_bfloat16 v) { return __bfloat162float(v); }
 
 // ---- launch helpers (host) ------------------------------------------------
+// Lets a kernel whose dynamic shared memory depends on the handle be launched
+// with `bytes` of it.  The limit belongs to the function, not to a handle: it is
+// set to all that the device gives, so that a handle made later does not lower it
+// under an earlier one.
+template <typename K>
+cudaError_t allow_smem(K* kernel, size_t bytes) {
+  cudaFuncAttributes fa;
+  int dev = 0, most = 0;
+  cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
+  if (e == cudaSuccess) e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e != cudaSuccess) return e;
+  most -= (int)fa.sharedSizeBytes;
+  if (bytes > (size_t)most) return cudaErrorInvalidValue;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+}
+
 // Each returns cudaGetLastError() of its launch.
 // Partial column sums of A'u by row chunks (no handle; passes.cuh has a handle's passes).
 template <typename T>

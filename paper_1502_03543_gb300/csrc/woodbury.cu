@@ -219,13 +219,10 @@ pdas_status pdas_woodbury_create(int64_t m, int64_t n, int a_dtype, void* stream
   if (e == cudaSuccess) e = cudaMemsetAsync(h->simt_tickets, 0, sizeof(unsigned) * simt_ticket_count(m), h->st);
   al((void**)&h->sc, sizeof(Scalars));
   if (e == cudaSuccess) e = cudaMallocHost((void**)&h->sc_host, sizeof(Scalars));
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_wb_step<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)(2 * m * sizeof(double)));
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_wb_step<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)(2 * m * sizeof(double)));
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_wb_step<__nv_bfloat16>,
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)(2 * m * sizeof(double)));
+  const size_t smem = 2 * m * sizeof(double);
+  if (e == cudaSuccess) e = allow_smem(k_wb_step<double>, smem);
+  if (e == cudaSuccess) e = allow_smem(k_wb_step<float>, smem);
+  if (e == cudaSuccess) e = allow_smem(k_wb_step<__nv_bfloat16>, smem);
   if (e != cudaSuccess) {
     pdas_woodbury_destroy(h);
     return PDAS_ERR_CUDA;
