@@ -800,7 +800,8 @@ __device__ void chol_chain(int me, int64_t m, int64_t ldm, float* M, float* dinv
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(sm.chain + kChainOps) + 1023) & ~uintptr_t(1023));
   const uint32_t ops_s = tc::smem_u32(ops), bar = tc::smem_u32(&sm.mma_bar);
   uint32_t parity = 0, full_parity = 0;
-  bool pending = false;  // MMAs have been issued and not been waited for
+  bool pending = false;    // MMAs have been issued and not been waited for
+  bool committed = false;  // ... and their arrival at bar is on its way
   float4 x[16];
 #pragma unroll 1
   for (int l = me; l < nb; l += 2) {
@@ -828,6 +829,7 @@ __device__ void chol_chain(int me, int64_t m, int64_t ldm, float* M, float* dinv
               tc_issue(ops_s + (b >> 1) * kTcChunkBytes, true, tmem, b == 0, 2 * (b & 1), 2 * (b & 1) + 2);
               if (b == 3) tc::umma_commit(bar);
             }
+            committed = b == 3;
           });
       if (!ok) break;
       publish_after_barrier(state, (int64_t)l * nb + l - 1, l);
@@ -879,7 +881,7 @@ __device__ void chol_chain(int me, int64_t m, int64_t ldm, float* M, float* dinv
     }
   }
   if (pending) {  // a wait gave up with MMAs in flight: they end before TMEM is freed
-    if (tid == 0) tc::umma_commit(bar);
+    if (tid == 0 && !committed) tc::umma_commit(bar);  // (a second arrival would pass the phase waited for)
     tc::mbar_wait(bar, parity, nullptr);
   }
 }
